@@ -197,14 +197,43 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
+// tanh of a pair of fp32 pre-activations whose results are rounded to bf16:
+// x P(x^2) / Q(x^2) with P and Q cubic, fitted to tanh on |x| <= 3.5 by
+// weighted least squares (relative error of the fit 1.8e-9; of the fp32
+// evaluation at most 2.8e-7 and 6e-8 rms over [1e-6, 3.5], as tanhf's).  The
+// argument is clamped to +-3.5 first: tanh(3.5) = 0.99818 lies above the
+// midpoint 0.99805 between the two largest bf16 values below and at one, so
+// every |x| >= 3.5 rounds to +-1 as tanh does; infinities clamp and NaN
+// passes.  Nine packed or plain FMA-pipe operations, a reciprocal and a clamp
+// per value, without a branch, where tanhf takes about 18 issue slots and
+// both sides of its branch: the hidden epilogues are bound by instruction
+// issue.  Measured with tanhf and with this: a 72B rollout of 65,536 envs x 64
+// steps 4.91 and 4.18 ms, a Stress rollout of 262,144 x 8 5.44 and 4.56 ms.
+__device__ __forceinline__ float2 tanh2_for_bf16(float2 x) {
+  asm("min.NaN.xorsign.abs.f32 %0, %0, 0f40600000;" : "+f"(x.x));  // 3.5 with x's sign
+  asm("min.NaN.xorsign.abs.f32 %0, %0, 0f40600000;" : "+f"(x.y));
+  const float2 s = __fmul2_rn(x, x);
+  auto both = [](float c) { return make_float2(c, c); };
+  float2 p = __ffma2_rn(both(6.116621e-06f), s, both(2.6453265e-03f));
+  float2 q = __ffma2_rn(both(1.8635452e-04f), s, both(2.2691658e-02f));
+  p = __ffma2_rn(p, s, both(0.1268055f));
+  q = __ffma2_rn(q, s, both(0.46013883f));
+  p = __ffma2_rn(p, s, both(1.0f));
+  q = __ffma2_rn(q, s, both(1.0f));
+  float2 r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(q.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(q.y));
+  return __fmul2_rn(__fmul2_rn(x, p), r);
+}
+
 // tanh of 16 hidden pre-activations (v + bias, one TMEM chunk of a thread's
 // row), rounded to bf16 and packed in pairs; the bias is added with the
 // packed two-lane fp32 add (the same rounding as two adds).
 __device__ __forceinline__ void tanh16_bf16(const float (&v)[16], const float* bias, uint32_t (&pk)[8]) {
 #pragma unroll
   for (int i = 0; i < 16; i += 2) {
-    const float2 z = __fadd2_rn(make_float2(v[i], v[i + 1]), *reinterpret_cast<const float2*>(bias + i));
-    __nv_bfloat162 r = __floats2bfloat162_rn(tanhf(z.x), tanhf(z.y));
+    const float2 t = tanh2_for_bf16(__fadd2_rn(make_float2(v[i], v[i + 1]), *reinterpret_cast<const float2*>(bias + i)));
+    __nv_bfloat162 r = __floats2bfloat162_rn(t.x, t.y);
     pk[i / 2] = *reinterpret_cast<uint32_t*>(&r);
   }
 }

@@ -488,6 +488,45 @@ def test_value_bf16_parity_ragged():
         assert bf16_ok(cpu(out), ov)
 
 
+@pytest.mark.parametrize("D,H", [(32, 256), (64, 512)])
+def test_bf16_tanh_pointwise(D, H):
+    """The hidden layers' tanh at chosen arguments: one-hot observations
+    saturate one hidden unit of layer 1 to exactly 1, so that unit 0 of layer
+    2 sees W2[0][d] + b2[0] and the head returns its bf16 activation.  The fp32
+    value is within 3e-7 (relative) of tanh, so after rounding it may differ
+    only next to a rounding midpoint, by one bf16 step; +-inf gives +-1 and
+    NaN stays NaN."""
+    net = W.NetSpec(D, H, 16, pe.PE_BF16)
+    pol = H * D + H + H * H + H + 16 * H + 16
+    obs = torch.eye(D, dtype=torch.bfloat16, device="cuda")
+    out = torch.empty(D, device="cuda")
+    rng = np.random.default_rng(7)
+    edge = np.array([0.0, 1e-30, 1e-6, 3.0, 3.46, 3.4657, 3.47, 3.5, 3.51, 4.0, 9.0, 1e4, 2.7e6, 1e19, 3e38, 1e-3])
+    seen = off = 0
+    for call in range(12):
+        w = np.concatenate([edge, -edge]) if call == 0 else rng.uniform(-4.5, 4.5, 32) * (10.0 ** -rng.integers(0, 4))
+        b2 = np.float32(0.0 if call == 0 else rng.uniform(-0.1, 0.1) * (10.0 ** -rng.integers(0, 4)))
+        p = np.zeros(W.param_count(D, H, 16), np.float32)
+        p[pol:pol + H * D].reshape(H, D)[np.arange(32), np.arange(32)] = 100.0
+        o = pol + H * D + H
+        p[o:o + 32] = w
+        p[o + H * H] = b2
+        p[o + H * H + H] = 1.0
+        pe.value(net, torch.from_numpy(p).cuda(), obs, out)
+        pe.device_check()
+        z = (torch.from_numpy(w).float().bfloat16().float() + torch.tensor(b2)).double()
+        want = torch.tanh(z).float().bfloat16().float().numpy()
+        got = cpu(out)[:32]
+        step = np.maximum(np.abs(want), 1e-37) * 2.0 ** -7
+        assert np.all(np.abs(got - want) <= step), (call, got, want)
+        seen, off = seen + 32, off + int((got != want).sum())
+    assert off <= seen // 50, (off, seen)
+    for b2, want in ((np.inf, 1.0), (-np.inf, -1.0), (np.nan, np.nan)):
+        p[o + H * H] = b2
+        pe.value(net, torch.from_numpy(p).cuda(), obs, out)
+        assert np.array_equal(cpu(out)[:32], np.full(32, want, np.float32), equal_nan=True)
+
+
 def test_env_checkpoint_roundtrip():
     wl = W.make_tiny(n_envs=50)
     params = torch.from_numpy(W.init_params(wl.net, seed=2)).cuda()
