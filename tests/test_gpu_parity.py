@@ -191,6 +191,22 @@ def test_fleet_parity_more_than_eight_jobs():
     assert c.sum() > 0
 
 
+@pytest.mark.parametrize("spread_w", [0.0, 390.0, 1500.0])
+@pytest.mark.parametrize("N,H,windows", [(3, 9000, [1, 3, 60, 600]), (700, 257, [255, 256, 5]), (2, 6145, [2, 992])])
+def test_fleet_parity_sample_ranges(spread_w, N, H, windows):
+    """The width of the job rows follows the jobs' ranges: 16-bit samples
+    added in groups of four (the fleet as it is) or of two (every job spans
+    about 390 W more), 32-bit prefixes beyond 16 bits.  Few compositions over
+    a long horizon split it into parts; windows around the 256-sample blocks."""
+    fw = W.make_fleet(n_compositions=N, length=2311, seed=6)
+    for j in range(fw.n_jobs):
+        fw.traces[int(np.argmax(fw.job_of_gpu == j)), 100 + j] += np.float32(spread_w)
+    fw.horizon = H
+    c, p = _fleet_gpu(fw, windows)
+    oc, op = O.fleet_windows(fw.traces, fw.job_of_gpu, fw.n_jobs, fw.offsets, H, windows, fw.budget_q)
+    assert np.array_equal(c, oc) and np.array_equal(p, op)
+
+
 def test_fleet_parity_full_size_sampled():
     """380,000-sample traces and 1,000,000 compositions (the full fleet
     workload); the oracle recomputes a seeded sample of compositions."""
@@ -232,6 +248,18 @@ def test_fleet_stagger_bit_exact(L, H, w, stride):
     """Greedy staggered offsets and stage peaks equal the oracle's exactly
     (ragged candidate grids, horizons shorter and longer than the period)."""
     fw = W.make_fleet(n_compositions=1, length=L, seed=3)
+    g_off, g_pk = _stagger_gpu(fw.traces, fw.job_of_gpu, fw.n_jobs, H, w, stride)
+    o_off, o_pk = O.fleet_stagger(fw.traces, fw.job_of_gpu, fw.n_jobs, H, w, stride)
+    assert np.array_equal(g_off, o_off) and np.array_equal(g_pk, o_pk), (g_off, o_off, g_pk, o_pk)
+
+
+@pytest.mark.parametrize("L,H,w,stride", [(1024, 700, 60, 1), (1025, 63, 1, 1), (2500, 40, 60, 3),
+                                          (700, 650, 5, 701), (2100, 2113, 30, 2), (90, 90, 90, 1)])
+def test_fleet_stagger_tile_edges(L, H, w, stride):
+    """The candidate peaks at the edges of their tiles: 1,024 candidates and
+    one more, horizons around the 64-sample items and past the 2,048-sample
+    ones, one window or none in the horizon, one candidate, two residues."""
+    fw = W.make_fleet(n_compositions=1, length=L, seed=4)
     g_off, g_pk = _stagger_gpu(fw.traces, fw.job_of_gpu, fw.n_jobs, H, w, stride)
     o_off, o_pk = O.fleet_stagger(fw.traces, fw.job_of_gpu, fw.n_jobs, H, w, stride)
     assert np.array_equal(g_off, o_off) and np.array_equal(g_pk, o_pk), (g_off, o_off, g_pk, o_pk)
