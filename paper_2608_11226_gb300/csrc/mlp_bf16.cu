@@ -75,7 +75,10 @@ __global__ void weight_image_kernel(const float* __restrict__ params, int A, int
 // Warp roles: warps 0-15 run the epilogues, warp 16 issues cp.async.bulk for
 // stage s into slot s%2 once the MMAs that read the slot's previous stage
 // have completed (tcgen05.commit on the slot's "empty" barrier), warp 17
-// issues the MMAs.  A layer's 512 accumulator columns fill TMEM, so a tile
+// issues the MMAs, warp 18 stores the h1 and h2 tile images of a PPO forward
+// (the buffer's halves are the images' bytes, so one bulk copy of 64 KB stores
+// each; "sa" and "sb" complete when a copy has read its half, and the epilogue
+// that overwrites it waits for that).  A layer's 512 accumulator columns fill TMEM, so a tile
 // cannot overlap another tile; instead the epilogues hand over per 256-column
 // half, and the layer-2 MMAs run beside them:
 //   epilogue 1, half A (h1 columns 0-255) -> MMAs of layer-2 N-half 0 over
@@ -97,7 +100,7 @@ __global__ void weight_image_kernel(const float* __restrict__ params, int A, int
 // balances a tile count that is not a multiple of the SM count.
 // ---------------------------------------------------------------------------
 constexpr int kComputeThreads = 512;
-constexpr int kStreamThreads = kComputeThreads + 64;
+constexpr int kStreamThreads = kComputeThreads + 96;  // + the weight producer, the MMA issuer and the image storer
 
 // the second network of a two-network stream launch (img == NULL: one network)
 struct MlpSecond {
@@ -142,8 +145,10 @@ struct MlpStreamSmem {
   uint64_t full[2], empty[2], fin;
   // one completion per tile each: X written (warps 4-15), head read out of
   // TMEM (warps 0-3), layer-1 N-halves done, h1 halves written, layer-2
-  // N-half 0 done, N-half 1 past K-block 3, N-half 1 done, h2 written, head done
-  uint64_t xin, hd, m1a, m1b, h1a, h1b, m2a, n1lo, m2b, h2in, mh;
+  // N-half 0 done, N-half 1 past K-block 3, N-half 1 done, h2's first half
+  // written, all of h2 written, head done; two per tile: the image of the
+  // half's h1, then of its h2, has been read
+  uint64_t xin, hd, m1a, m1b, h1a, h1b, m2a, n1lo, m2b, h2a, h2in, mh, sa, sb;
   uint32_t tmem_base;
   int32_t err;
 };
@@ -184,8 +189,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     tc::mbar_init(&s.m2a, 1);
     tc::mbar_init(&s.n1lo, 1);
     tc::mbar_init(&s.m2b, 1);
+    tc::mbar_init(&s.h2a, 16);
     tc::mbar_init(&s.h2in, 16);
     tc::mbar_init(&s.mh, 1);
+    tc::mbar_init(&s.sa, 1);
+    tc::mbar_init(&s.sb, 1);
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, 512);
@@ -316,6 +324,32 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       tc::mma_commit(&s.fin);
       if (!tc::mbar_wait(&s.fin, 0)) atomicExch(&s.err, 1);
     }
+  } else if (warp == 18) {
+    // storer: the h1 and h2 images of every tile, in halves
+    if (lane == 0 && save.h1) {
+      constexpr uint32_t kHalf = kTcRows * H;  // bytes
+      bool ok = true;
+      auto store = [&](uint64_t* ready, uint32_t par, uint64_t* done, __nv_bfloat16* img, int64_t tile, int half) {
+        ok = ok && wt(ready, par);
+        if (!ok) return;
+        tc::bulk_s2g(reinterpret_cast<uint8_t*>(img) + tile * (int64_t)(2 * kHalf) + half * kHalf,
+                     s.act + half * kHalf, kHalf);
+        tc::bulk_commit();
+        tc::bulk_wait_read();
+        tc::mbar_arrive(done);
+      };
+      for (int t = 0; t < my_tiles && ok; ++t) {
+        int ni;
+        const int64_t tile = tile_of(t, ni);
+        __nv_bfloat16* const g1 = ni ? second.save.h1 : save.h1;
+        __nv_bfloat16* const g2 = ni ? second.save.h2 : save.h2;
+        store(&s.h1a, t & 1, &s.sa, g1, tile, 0);
+        store(&s.h1b, t & 1, &s.sb, g1, tile, 1);
+        store(&s.h2a, t & 1, &s.sa, g2, tile, 0);
+        store(&s.h2in, t & 1, &s.sb, g2, tile, 1);
+      }
+      tc::bulk_wait();
+    }
   } else {
     // epilogue warps: four TMEM lane quadrants x four column slices
     const int quad = warp & 3, slice = warp >> 2, row = quad * 32 + lane;
@@ -341,7 +375,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       tc::fence_async_smem();
       tc::fence_before();
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+      if (lane == 0) tc::mbar_arrive(bar);
     };
     // columns c .. c + 15 of this thread's row: tanh(acc + bias), packed bf16
     auto chunk = [&](int c, const float* bias, uint32_t (&pk)[8]) {
@@ -349,16 +383,16 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       tc::tmem_ld16(lane_addr + (uint32_t)c, v);
       tc::tanh16_bf16(v, bias + c, pk);
     };
-    // ... into the activation buffer (the next A operand) and the tile image g
-    auto put = [&](int c, const uint32_t (&pk)[8], uint8_t* g) {
+    // ... into the activation buffer (the next A operand)
+    auto put = [&](int c, const uint32_t (&pk)[8]) {
       const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
-      const uint4 lo = make_uint4(pk[0], pk[1], pk[2], pk[3]), hi = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      *reinterpret_cast<uint4*>(s.act + o0) = lo;
-      *reinterpret_cast<uint4*>(s.act + o1) = hi;
-      if (g) {
-        *reinterpret_cast<uint4*>(g + o0) = lo;
-        *reinterpret_cast<uint4*>(g + o1) = hi;
-      }
+      *reinterpret_cast<uint4*>(s.act + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+      *reinterpret_cast<uint4*>(s.act + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    };
+    // wait until the storer has read a half's h1 (q = 0) or h2 (q = 1) of tile t
+    const bool saving = save.h1 != nullptr;
+    auto wait_stored = [&](uint64_t* done, int q) {
+      if (saving) (void)wt(done, q);  // two completions per tile: the first has parity 0
     };
     // head of this CTA's k-th tile from its 16 accumulators (warps 0-3, one row per thread)
     auto head_out = [&](int k, const float (&v)[16]) {
@@ -381,10 +415,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       int ni;
       const int64_t tile = tile_of(t, ni);
       __nv_bfloat16* const sx = ni ? second.save.x : save.x;
-      __nv_bfloat16* const sh1 = ni ? second.save.h1 : save.h1;
-      __nv_bfloat16* const sh2 = ni ? second.save.h2 : save.h2;
-      uint8_t* const gh1 = sh1 ? reinterpret_cast<uint8_t*>(sh1) + tile * (int64_t)(kTcRows * H * 2) : nullptr;
-      uint8_t* const gh2 = sh2 ? reinterpret_cast<uint8_t*>(sh2) + tile * (int64_t)(kTcRows * H * 2) : nullptr;
       const float* const b1 = s.b1[ni];
       const float* const b2 = s.b2[ni];
       if (t > 0) (void)wt(&s.mh, par ^ 1);  // the previous tile's head is done
@@ -400,10 +430,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
             *reinterpret_cast<float4*>(&s.headv[row][j]) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
           tc::fence_before();
           __syncwarp();
-          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&s.hd)) : "memory");
+          if (lane == 0) tc::mbar_arrive(&s.hd);
         }
       } else {
-        // this tile's X (the previous tile's head MMA has read h2)
+        // this tile's X (the previous tile's head MMA and the storer have read h2)
+        if (t > 0) wait_stored(&s.sb, 1);
 #pragma unroll
         for (int q = 0; q < XCH; ++q) {
           const int i = xt + q * 384;
@@ -421,13 +452,14 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       // epilogue 1, half A (h1 K-blocks 0-3), then half B (K-blocks 4-7, the
       // last of which held X: layer-1 N-half 1 is done by then)
       (void)wt(&s.m1a, par);
+      if (t > 0) wait_stored(&s.sa, 1);
       tc::fence_after();
 #pragma unroll 1
       for (int j = 0; j < NJ; ++j) {
         const int c = slice * (H / 8) + j * 16;
         uint32_t pk[8];
         chunk(c, b1, pk);
-        put(c, pk, gh1);
+        put(c, pk);
       }
       handover(&s.h1a);
       (void)wt(&s.m1b, par);
@@ -437,7 +469,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         const int c = H / 2 + slice * (H / 8) + j * 16;
         uint32_t pk[8];
         chunk(c, b1, pk);
-        put(c, pk, gh1);
+        put(c, pk);
       }
       handover(&s.h1b);
       // the previous tile's head epilogue, while the rest of layer-2 N-half 0 runs
@@ -460,25 +492,28 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         chunk(c0, b2, p0);
         chunk(c0 + 16, b2, p1);
         (void)wt(&s.n1lo, par);
+        wait_stored(&s.sa, 0);
         tc::fence_after();
-        put(c0, p0, gh2);
-        put(c0 + 16, p1, gh2);
+        put(c0, p0);
+        put(c0 + 16, p1);
 #pragma unroll 1
         for (int j = 2; j < NJ; ++j) {
           const int c = c0 + j * 16;
           uint32_t pk[8];
           chunk(c, b2, pk);
-          put(c, pk, gh2);
+          put(c, pk);
         }
       }
+      handover(&s.h2a);
       (void)wt(&s.m2b, par);
+      wait_stored(&s.sb, 0);
       tc::fence_after();
 #pragma unroll 1
       for (int j = 0; j < NJ; ++j) {
         const int c = H / 2 + slice * (H / 8) + j * 16;
         uint32_t pk[8];
         chunk(c, b2, pk);
-        put(c, pk, gh2);
+        put(c, pk);
       }
       handover(&s.h2in);
       // the next tile's observation rows, fetched while its X slot waits for this tile's head MMA
@@ -723,7 +758,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       tc::fence_async_smem();
       tc::fence_before();
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
+      if (lane == 0) tc::mbar_arrive(bar);
     };
     fetch_x(0, xv[0]);
     fetch_x(1, xv[1]);
