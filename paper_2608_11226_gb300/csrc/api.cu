@@ -134,9 +134,12 @@ static int obs_width(int kind) {
 // window sums), through the same reset as later episodes
 template <int C>
 __global__ void env_init_kernel(EnvDev env) {
+  __shared__ EnvTab<C> tab;
+  load_tab<C>(env, tab);
+  __syncthreads();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= env.E) return;
-  RegAcc<C> a;
+  RegAcc<C> a(tab);
   a.ring = env.ring + (int64_t)e * kRing;
   env_reset<C>(env, a, (uint32_t)e, 0u, 0u, kDrawInit);
   store_reg<C>(env, e, a);
@@ -371,6 +374,21 @@ pe_status pe_env_create(const pe_env_config* cfg, const float* trace, const uint
   }
   d.st = st; d.ring = ring; d.sums = sums;
   env->flag = flag;
+  if (C == 4) {  // position-major, the phase in the sign bits (see EnvDev::ftrace)
+    std::vector<uint32_t> v(h.size());
+    for (int f = 0; f < F; ++f)
+      for (int i = 0; i < fL[f]; ++i) {
+        const uint32_t label = ph[(size_t)(fpoff[f] + i)];
+        const uint32_t sign[4] = {label & 1u, (label >> 1) & 1u, (label >> 2) & 1u,
+                                  ((uint32_t)cfg->scale_phase_mask >> label) & 1u};
+        for (int c = 0; c < 4; ++c) {
+          uint32_t u = 0;
+          if (c < fC[f]) memcpy(&u, &h[(size_t)(ftoff[f] + (int64_t)c * fL[f] + i)], 4);
+          v[(size_t)(ftoff[f] + (int64_t)i * 4 + c)] = (u & 0x7FFFFFFFu) | (sign[c] << 31);
+        }
+      }
+    memcpy(h.data(), v.data(), sizeof(float) * h.size());
+  }
   PE_TRY_CUDA(cudaMemcpy(dtrace, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
   PE_TRY_CUDA(cudaMemcpy(dphase, ph.data(), ph.size(), cudaMemcpyHostToDevice));
   launch_env_init(d);  // one-time set-up, not profiled

@@ -116,8 +116,10 @@ __device__ __forceinline__ int32_t quant64(float x, float s) {
   return __float2int_rn(__fmul_rn(__fmul_rn(x, s), 64.0f));
 }
 
-__device__ __forceinline__ float ratio_i(int64_t num, int64_t den) {
-  return __fdiv_rn(__ll2float_rn(num), __ll2float_rn(den));
+// fp32 quotient of two whole numbers below 2^31 (every feature's terms are:
+// pe_env_create bounds the window sums and the budgets)
+__device__ __forceinline__ float ratio_i(int32_t num, int32_t den) {
+  return __fdiv_rn(__int2float_rn(num), __int2float_rn(den));
 }
 
 __device__ __forceinline__ float bf16r(float x) {

@@ -8,6 +8,8 @@
 // the violation indicators of Eq. 2 are exact.
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace pe {
@@ -29,8 +31,13 @@ struct EnvDev {
   int32_t span;               // samples one episode may span: ep_len * max ns
   uint64_t seed;
   // trace families (domain randomisation, Sec. 4.2 G2; one family without
-  // it): family f has a [C][fL[f]] trace (channels >= fC[f] are zero), a
-  // [fL[f]] phase array and the budget fB[f] in 1/64 W
+  // it): family f has a trace, a [fL[f]] phase array and the budget fB[f] in
+  // 1/64 W.  Four-channel traces are position-major, [fL[f]][4] with channels
+  // >= fC[f] zero, and carry the phase label (0 to 7) in the sign bits of
+  // channels 0 to 2 and "this phase is actuated" in channel 3's, so that one
+  // 16-byte load brings all that a sample needs: envs sit at unrelated
+  // positions, every scalar load of a warp is 32 requests of the L1, and a
+  // step reads 3 to 14 positions.  Narrower traces are [C][fL[f]].
   int32_t F;
   const float* ftrace[PE_MAX_FAMILIES];
   const uint8_t* fphase[PE_MAX_FAMILIES];
@@ -67,13 +74,67 @@ struct EnvTile {
   uint8_t ring[TE][kRing];  // level of each of those samples
 };
 
-__device__ __forceinline__ float actuator_scale(const EnvDev& env, int level, int c, int ph) {
-  return ((env.phase_mask >> ph) & 1) ? env.scale[level][c] : 1.0f;
+// One trace position: every channel's power and the phase label.
+template <int C>
+struct Samp {
+  float x[C];
+  int ph;
+  bool act;  // the phase is actuated
+};
+
+template <int C>
+__device__ __forceinline__ Samp<C> load_samp(const EnvDev& env, const Fam& fm, int pos) {
+  Samp<C> s;
+  if constexpr (C == 4) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(fm.trace) + pos);
+    s.x[0] = __uint_as_float(v.x & 0x7FFFFFFFu);
+    s.x[1] = __uint_as_float(v.y & 0x7FFFFFFFu);
+    s.x[2] = __uint_as_float(v.z & 0x7FFFFFFFu);
+    s.x[3] = __uint_as_float(v.w & 0x7FFFFFFFu);
+    s.ph = (int)((v.x >> 31) | ((v.y >> 31) << 1) | ((v.z >> 31) << 2));
+    s.act = (v.w >> 31) != 0;
+  } else {
+#pragma unroll
+    for (int c = 0; c < C; ++c) s.x[c] = __ldg(fm.trace + (int64_t)c * fm.L + pos);
+    s.ph = __ldg(fm.phase + pos);
+    s.act = (env.phase_mask >> s.ph) & 1;
+  }
+  return s;
 }
 
-__device__ __forceinline__ int32_t sample_q(const EnvDev& env, const Fam& fm, int c, int pos, int level) {
-  const float x = __ldg(fm.trace + (int64_t)c * fm.L + pos);
-  return quant64(x, actuator_scale(env, level, c, __ldg(fm.phase + pos)));
+// Level-indexed tables in shared memory (envs of a warp are at different
+// levels, and a constant bank serves one address at a time).
+template <int C>
+struct EnvTab {
+  alignas(16) float scale[PE_MAX_LEVELS][C];
+  float tokens[PE_MAX_LEVELS];
+  int32_t ns[PE_MAX_LEVELS];
+};
+
+// by the whole block, before a __syncthreads
+template <int C>
+__device__ __forceinline__ void load_tab(const EnvDev& env, EnvTab<C>& t) {
+  for (int l = threadIdx.x; l < PE_MAX_LEVELS; l += blockDim.x) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) t.scale[l][c] = env.scale[l][c];
+    t.tokens[l] = env.tokens[l];
+    t.ns[l] = env.ns[l];
+  }
+}
+
+// actuated power of every channel of a sample at `level`, in 1/64 W
+template <int C>
+__device__ __forceinline__ void sample_q(const EnvTab<C>& tab, const Samp<C>& s, int level, int32_t (&q)[C]) {
+  float f[C];
+  if constexpr (C == 4) {
+    const float4 v = *reinterpret_cast<const float4*>(tab.scale[level]);
+    f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w;
+  } else {
+#pragma unroll
+    for (int c = 0; c < C; ++c) f[c] = tab.scale[level][c];
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) q[c] = quant64(s.x[c], s.act ? f[c] : 1.0f);
 }
 
 // ---------------------------------------------------------------------------
@@ -86,7 +147,9 @@ __device__ __forceinline__ int32_t sample_q(const EnvDev& env, const Fam& fm, in
 // ---------------------------------------------------------------------------
 template <int TE, int C>
 struct TileAcc {
+  static constexpr int kUnroll = 1;  // the samples are in shared memory
   EnvTile<TE, C>& s;
+  const EnvTab<C>& tab;
   int e;
   __device__ int32_t& pos() { return s.pos[e]; }
   __device__ int32_t& k() { return s.k[e]; }
@@ -99,17 +162,30 @@ struct TileAcc {
   __device__ int32_t& sl(int c) { return s.s_long[e][c]; }
   __device__ uint8_t level_at(int p) const { return s.ring[e][p & (kRing - 1)]; }
   __device__ void set_level_at(int p, int l) { s.ring[e][p & (kRing - 1)] = (uint8_t)l; }
+  __device__ void fill_levels(int l) {
+    for (int i = 0; i < kRing; ++i) s.ring[e][i] = (uint8_t)l;
+  }
   // actuated sample of channel c at a recent position p (p in [pos-64, pos));
   // fm is the env's family view (unused: the tile caches the samples)
   __device__ int32_t q_at(const EnvDev&, const Fam&, int c, int p) const { return s.q[e][c][p & (kRing - 1)]; }
-  __device__ void push(int c, int p, int32_t q) { s.q[e][c][p & (kRing - 1)] = q; }
+  __device__ void q_all(const EnvDev& env, const Fam& fm, int p, int32_t (&q)[C]) const {
+#pragma unroll
+    for (int c = 0; c < C; ++c) q[c] = q_at(env, fm, c, p);
+  }
+  __device__ void push(int p, const int32_t (&q)[C]) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) s.q[e][c][p & (kRing - 1)] = q[c];
+  }
 };
 
 template <int C>
 struct RegAcc {
   int32_t pos_, k_, level_, prev_, b_, til_, fam_;
   int32_t ss_[C], sl_[C];
+  static constexpr int kUnroll = 4;  // samples of a batch whose loads are in flight together
   uint8_t* ring;  // global [64]
+  const EnvTab<C>& tab;
+  __device__ explicit RegAcc(const EnvTab<C>& t) : tab(t) {}
   __device__ int32_t& fam() { return fam_; }
   __device__ int32_t& pos() { return pos_; }
   __device__ int32_t& k() { return k_; }
@@ -121,29 +197,49 @@ struct RegAcc {
   __device__ int32_t& sl(int c) { return sl_[c]; }
   __device__ uint8_t level_at(int p) const { return ring[p & (kRing - 1)]; }
   __device__ void set_level_at(int p, int l) { ring[p & (kRing - 1)] = (uint8_t)l; }
-  // recomputed from the trace of the env's family (view fm) and the level ring
-  __device__ int32_t q_at(const EnvDev& env, const Fam& fm, int c, int p) const {
-    return sample_q(env, fm, c, p, level_at(p));
+  __device__ void fill_levels(int l) {
+    const uint32_t w = 0x01010101u * (uint32_t)l;
+#pragma unroll
+    for (int i = 0; i < kRing / 16; ++i) reinterpret_cast<uint4*>(ring)[i] = make_uint4(w, w, w, w);
   }
-  __device__ void push(int, int, int32_t) {}
+  // recomputed from the trace of the env's family (view fm) and the level ring
+  __device__ void q_all(const EnvDev& env, const Fam& fm, int p, int32_t (&q)[C]) const {
+    sample_q<C>(tab, load_samp<C>(env, fm, p), level_at(p), q);
+  }
+  __device__ int32_t q_at(const EnvDev& env, const Fam& fm, int c, int p) const {
+    int32_t q[C];
+    q_all(env, fm, p, q);
+    return q[c];
+  }
+  __device__ void push(int, const int32_t (&)[C]) {}
 };
 
-// 60-sample history before the current position at the recorded levels
+// 60-sample history before the current position at the recorded levels (for
+// a new episode every one of them is the default level, and the loads do not
+// wait for the ring)
 template <int C, class Acc>
-__device__ void rebuild_history(const EnvDev& env, Acc& a) {
+__device__ void rebuild_history(const EnvDev& env, Acc& a, int fixed_level = -1) {
   const int p = a.pos();
   const Fam fm = fam_of(env, a.fam());
-  for (int c = 0; c < C; ++c) {
-    int32_t ss = 0, sl = 0;
-    for (int i = 1; i <= kWLong; ++i) {
-      const int pp = p - i;
-      const int32_t q = sample_q(env, fm, c, pp, a.level_at(pp));
-      a.push(c, pp, q);
-      sl += q;
-      if (i <= kWShort) ss += q;
+  int32_t ss[C], sl[C];
+#pragma unroll
+  for (int c = 0; c < C; ++c) ss[c] = sl[c] = 0;
+#pragma unroll 4
+  for (int i = 1; i <= kWLong; ++i) {
+    const int pp = p - i;
+    int32_t q[C];
+    sample_q<C>(a.tab, load_samp<C>(env, fm, pp), fixed_level >= 0 ? fixed_level : (int)a.level_at(pp), q);
+    a.push(pp, q);
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      sl[c] += q[c];
+      if (i <= kWShort) ss[c] += q[c];
     }
-    a.ss(c) = ss;
-    a.sl(c) = sl;
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    a.ss(c) = ss[c];
+    a.sl(c) = sl[c];
   }
 }
 
@@ -156,8 +252,8 @@ __device__ void env_reset_at(const EnvDev& env, Acc& a, int o) {
   a.prev() = env.level_init;
   a.b() = env.b_init;
   a.til() = 0;
-  for (int i = 0; i < kRing; ++i) a.set_level_at(i, env.level_init);
-  rebuild_history<C>(env, a);
+  a.fill_levels(env.level_init);
+  rebuild_history<C>(env, a, env.level_init);
 }
 
 // new episode at a random offset (Sec. 4.1); with several trace families,
@@ -194,14 +290,14 @@ __device__ __forceinline__ int32_t Qcl(const EnvDev& env, Acc& a, const Fam& fm,
 //   callers that write a whole observation
 template <int C, int OBS, class Acc>
 __device__ __forceinline__ float feature(const EnvDev& env, Acc& a, const Fam& fm, int f) {
-  const int64_t B = fm.B;
+  const int32_t B = fm.B;
   if (OBS == PE_OBS_TINY8) {
     if (f < 5) return ratio_i(Qcl<C>(env, a, fm, 4 - f), B);
     if (f == 5) return ratio_i(B - Qcl<C>(env, a, fm, 0), B);
     if (f == 6) return (float)__ldg(fm.phase + a.pos() - 1);
     return ratio_i(a.level(), env.n_levels - 1);
   }
-  int64_t S20 = 0, S60 = 0;
+  int32_t S20 = 0, S60 = 0;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     S20 += a.ss(c);
@@ -216,7 +312,7 @@ __device__ __forceinline__ float feature(const EnvDev& env, Acc& a, const Fam& f
       case 11: return ratio_i(a.level() - env.g_min, env.g_max - env.g_min);
       case 12: return ratio_i(a.b() - env.b_min, env.b_max - env.b_min);
       case 13: return ratio_i(S20, kWShort * B);
-      case 14: return ratio_i((int64_t)Qcl<C>(env, a, fm, 0) - Qcl<C>(env, a, fm, 10), B);
+      case 14: return ratio_i(Qcl<C>(env, a, fm, 0) - Qcl<C>(env, a, fm, 10), B);
       default: return 0.0f;
     }
   }
@@ -226,104 +322,121 @@ __device__ __forceinline__ float feature(const EnvDev& env, Acc& a, const Fam& f
     case 1: return ratio_i(S20, kWShort * B);
     case 2: return ratio_i(S60, kWLong * B);
     case 3: return ratio_i(kWLong * B - S60, kWLong * B);
-    case 4: return ratio_i((int64_t)Qcl<C>(env, a, fm, 0) - Qcl<C>(env, a, fm, 10), B);
+    case 4: return ratio_i(Qcl<C>(env, a, fm, 0) - Qcl<C>(env, a, fm, 10), B);
     case 5: return ratio_i(a.level() + 1, env.n_levels);
     case 6: return ratio_i(a.prev() + 1, env.n_levels);
-    case 7: return fminf(env.cadence ? ratio_i(env.ns[a.level()], 40) : ratio_i(a.til(), 40), 1.0f);
+    case 7: return fminf(env.cadence ? ratio_i(a.tab.ns[a.level()], 40) : ratio_i(a.til(), 40), 1.0f);
     default: break;
   }
   if (OBS == PE_OBS_OCC32) {
     if (f < 24) {
       const int c = (f - 8) >> 2, i = (f - 8) & 3;
-      return c < fm.C ? ratio_i((int64_t)fm.C * Qc<C>(env, a, fm, c, 3 - i), B) : 0.0f;
+      return c < fm.C ? ratio_i(fm.C * Qc<C>(env, a, fm, c, 3 - i), B) : 0.0f;
     }
     if (f < 28) {
       const int c = f - 24;
-      return c < fm.C ? ratio_i((int64_t)fm.C * a.sl(c), kWLong * B) : 0.0f;
+      return c < fm.C ? ratio_i(fm.C * a.sl(c), kWLong * B) : 0.0f;
     }
     return 0.0f;
   }
   // OCC64
   if (f < 56) {
     const int c = (f - 8) / 12, i = (f - 8) % 12;
-    return c < fm.C ? ratio_i((int64_t)fm.C * Qc<C>(env, a, fm, c, 11 - i), B) : 0.0f;
+    return c < fm.C ? ratio_i(fm.C * Qc<C>(env, a, fm, c, 11 - i), B) : 0.0f;
   }
   if (f < 60) {
     const int c = f - 56;
-    return c < fm.C ? ratio_i((int64_t)fm.C * a.ss(c), kWShort * B) : 0.0f;
+    return c < fm.C ? ratio_i(fm.C * a.ss(c), kWShort * B) : 0.0f;
   }
   const int c = f - 60;
-  return c < fm.C ? ratio_i((int64_t)fm.C * a.sl(c), kWLong * B) : 0.0f;
+  return c < fm.C ? ratio_i(fm.C * a.sl(c), kWLong * B) : 0.0f;
 }
 
-// All D features of an Eq. 5 observation (OCC32 / OCC64) for an env whose
-// samples are recomputed from the trace (RegAcc): the actuated samples the
-// features read -- positions pos-1 .. pos-NB and pos-11, every channel -- are
-// fetched once, with all their loads independent, instead of per feature.
-// The arithmetic is feature()'s, so the results are the same bits.
+// What the Eq. 5 observations read of the past: the actuated samples of
+// positions p0, p0 - 1, .. and p0 - 10.
+template <int C, int OBS>
+struct Recent {
+  static constexpr int NB = OBS == PE_OBS_OCC32 ? 4 : 12;   // recent samples per channel
+  static constexpr int NP = NB > 10 ? NB : NB + 1;          // back positions read, p0 - 10 included
+  static constexpr int I10 = NB > 10 ? 10 : NB;             // index of p0 - 10
+  __device__ static constexpr int back(int i) { return i < NB ? i : 10; }
+  Samp<C> newest;  // position p0 before the actuator
+  int32_t q[NP][C];
+};
+
+// the 12 levels of positions p0 - 11 .. p0 as three words (oldest first): two
+// 16-byte loads of the env's ring instead of a byte load per position
+template <int C>
+__device__ __forceinline__ void recent_levels(const RegAcc<C>& a, int p0, uint32_t (&r)[3]) {
+  const int start = (p0 - 11) & (kRing - 1), chunk = start >> 4;
+  const uint4 lo = reinterpret_cast<const uint4*>(a.ring)[chunk];
+  const uint4 hi = reinterpret_cast<const uint4*>(a.ring)[(chunk + 1) & (kRing / 16 - 1)];
+  const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  const int k = (start >> 2) & 3, sh = (start & 3) * 8;
+  uint32_t v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = k < 2 ? (k == 0 ? w[i] : w[i + 1]) : (k == 2 ? w[i + 2] : w[i + 3]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) r[i] = __funnelshift_r(v[i], v[i + 1], sh);
+}
+
+// loads of the history that ends at position p0, all independent
+template <int C, int OBS>
+__device__ __forceinline__ void load_recent(const EnvDev& env, const RegAcc<C>& a, const Fam& fm, int p0,
+                                            Recent<C, OBS>& h) {
+  using R = Recent<C, OBS>;
+  uint32_t r[3];
+  recent_levels<C>(a, p0, r);
+#pragma unroll
+  for (int i = 0; i < R::NP; ++i) {
+    const Samp<C> s = load_samp<C>(env, fm, p0 - R::back(i));
+    const int byte = 11 - R::back(i);
+    sample_q<C>(a.tab, s, (int)((r[byte / 4] >> (8 * (byte & 3))) & 255u), h.q[i]);
+    if (i == 0) h.newest = s;
+  }
+}
+
+// All D features of an Eq. 5 observation (OCC32 / OCC64) from the recent
+// samples h of the position before a.pos().  The arithmetic is feature()'s
+// (every quotient's terms are whole numbers below 2^31), so the results are
+// the same bits.
 template <int C, int OBS, int D>
-__device__ __forceinline__ void features_eq5(const EnvDev& env, RegAcc<C>& a, const Fam& fm, float (&o)[D]) {
+__device__ __forceinline__ void features_eq5(const EnvDev& env, RegAcc<C>& a, const Fam& fm,
+                                             const Recent<C, OBS>& h, float (&o)[D]) {
   static_assert(OBS == PE_OBS_OCC32 || OBS == PE_OBS_OCC64, "Eq. 5 observations");
-  constexpr int NB = OBS == PE_OBS_OCC32 ? 4 : 12;  // recent samples per channel
-  constexpr int NP = NB > 10 ? NB : NB + 1;          // back positions read, pos-11 included
-  const int p0 = a.pos() - 1;
-  uint8_t lv[NP], ph[NP];
-  float x[C][NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    const int pp = p0 - (i < NB ? i : 10);
-    lv[i] = a.level_at(pp);
-    ph[i] = __ldg(fm.phase + pp);
-#pragma unroll
-    for (int c = 0; c < C; ++c) x[c][i] = __ldg(fm.trace + (int64_t)c * fm.L + pp);
-  }
-  int32_t q[C][NP];
-#pragma unroll
-  for (int i = 0; i < NP; ++i)
-#pragma unroll
-    for (int c = 0; c < C; ++c) q[c][i] = quant64(x[c][i], actuator_scale(env, lv[i], c, ph[i]));
-  const int i10 = NB > 10 ? 10 : NB;
-  int32_t Q0 = 0, Q10 = 0;
+  using R = Recent<C, OBS>;
+  int32_t Q0 = 0, Q10 = 0, S20 = 0, S60 = 0;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    Q0 += q[c][0];
-    Q10 += q[c][i10];
-  }
-  const int64_t B = fm.B;
-  int64_t S20 = 0, S60 = 0;
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
+    Q0 += h.q[0][c];
+    Q10 += h.q[R::I10][c];
     S20 += a.ss(c);
     S60 += a.sl(c);
   }
+  const int32_t B = fm.B;
   o[0] = ratio_i(Q0, B);
   o[1] = ratio_i(S20, kWShort * B);
   o[2] = ratio_i(S60, kWLong * B);
   o[3] = ratio_i(kWLong * B - S60, kWLong * B);
-  o[4] = ratio_i((int64_t)Q0 - Q10, B);
+  o[4] = ratio_i(Q0 - Q10, B);
   o[5] = ratio_i(a.level() + 1, env.n_levels);
   o[6] = ratio_i(a.prev() + 1, env.n_levels);
-  o[7] = fminf(env.cadence ? ratio_i(env.ns[a.level()], 40) : ratio_i(a.til(), 40), 1.0f);
+  o[7] = fminf(env.cadence ? ratio_i(a.tab.ns[a.level()], 40) : ratio_i(a.til(), 40), 1.0f);
+#pragma unroll
+  for (int f = 8; f < 8 + 4 * R::NB; ++f) {
+    const int c = (f - 8) / R::NB, i = (f - 8) % R::NB;
+    o[f] = c < fm.C ? ratio_i(fm.C * h.q[R::NB - 1 - i][c], B) : 0.0f;
+  }
   if (OBS == PE_OBS_OCC32) {
 #pragma unroll
-    for (int f = 8; f < 24; ++f) {
-      const int c = (f - 8) >> 2, i = (f - 8) & 3;
-      o[f] = c < fm.C ? ratio_i((int64_t)fm.C * q[c][3 - i], B) : 0.0f;
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) o[24 + c] = c < fm.C ? ratio_i((int64_t)fm.C * a.sl(c), kWLong * B) : 0.0f;
+    for (int c = 0; c < 4; ++c) o[24 + c] = c < fm.C ? ratio_i(fm.C * a.sl(c), kWLong * B) : 0.0f;
 #pragma unroll
     for (int f = 28; f < D; ++f) o[f] = 0.0f;
   } else {
 #pragma unroll
-    for (int f = 8; f < 56; ++f) {
-      const int c = (f - 8) / 12, i = (f - 8) % 12;
-      o[f] = c < fm.C ? ratio_i((int64_t)fm.C * q[c][11 - i], B) : 0.0f;
-    }
-#pragma unroll
     for (int c = 0; c < 4; ++c) {
-      o[56 + c] = c < fm.C ? ratio_i((int64_t)fm.C * a.ss(c), kWShort * B) : 0.0f;
-      o[60 + c] = c < fm.C ? ratio_i((int64_t)fm.C * a.sl(c), kWLong * B) : 0.0f;
+      o[56 + c] = c < fm.C ? ratio_i(fm.C * a.ss(c), kWShort * B) : 0.0f;
+      o[60 + c] = c < fm.C ? ratio_i(fm.C * a.sl(c), kWLong * B) : 0.0f;
     }
   }
 }
@@ -340,8 +453,11 @@ struct StepOut {
 
 // Apply action act and consume one sample (Sec. 4.1 actuator and action set
 // with the Sec. 4.2 floor g_min; Eqs. 1-3; G1 or Eq. 6 reward).
-template <int C, class Acc>
-__device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, float lambda) {
+// ONE: every step consumes one sample (no cadence table); `next`: that
+// sample, when the caller has fetched it ahead.
+template <int C, bool ONE = false, class Acc>
+__device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, float lambda,
+                                            const Samp<C>* next = nullptr) {
   int nl = a.level();
   if (env.act_kind == PE_ACT_INCDEC) {
     if (act == 1 && nl > env.g_min) --nl;
@@ -359,7 +475,7 @@ __device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, 
   // summed; the Eq. 6 peak term is the batch's largest 30 s excess
   const Fam fm = fam_of(env, a.fam());
   const int64_t B60 = (int64_t)kWLong * fm.B;
-  float rate = env.tokens[nl];
+  float rate = a.tab.tokens[nl];
   if (env.act_kind == PE_ACT_INCDEC) rate = __fdiv_rn(rate * (float)a.b(), (float)env.b_init);
   StepOut o;
   o.q = 0;
@@ -368,37 +484,57 @@ __device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, 
   o.tokens = 0.0f;
   o.excess = 0.0f;
   float peak_w = 0.0f, fixed = 0.0f;
-  const int n = env.ns[nl];
-  for (int i = 0; i < n; ++i) {
+  const int n = ONE ? 1 : a.tab.ns[nl];
+  // U consecutive samples: what they read of the trace and the history is
+  // fetched together (positions 20 and 60 back lie before all of them), then
+  // they are consumed in order
+  auto consume = [&](auto tag) {
+    constexpr int U = decltype(tag)::value;
     const int p = a.pos();
-    const int ph = __ldg(fm.phase + p);
-    int32_t Q = 0;
-    int64_t S60 = 0;
+    Samp<C> sn[U];
+    int32_t q20[U][C], q60[U][C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const int32_t qin = quant64(__ldg(fm.trace + (int64_t)c * fm.L + p), actuator_scale(env, nl, c, ph));
-      const int32_t q20 = a.q_at(env, fm, c, p - kWShort);
-      const int32_t q60 = a.q_at(env, fm, c, p - kWLong);
-      a.ss(c) += qin - q20;
-      a.sl(c) += qin - q60;
-      a.push(c, p, qin);
-      Q += qin;
-      S60 += a.sl(c);
+    for (int u = 0; u < U; ++u) {
+      sn[u] = ONE && next ? *next : load_samp<C>(env, fm, p + u);
+      a.q_all(env, fm, p + u - kWShort, q20[u]);
+      a.q_all(env, fm, p + u - kWLong, q60[u]);
     }
-    a.set_level_at(p, nl);  // after the window updates: slot p & 63 held position p - 64
-    const int v1 = Q > fm.B, v60 = S60 > B60;
-    const float exc_w = v60 ? __fdiv_rn(__ll2float_rn(S60 - B60), 3840.0f) : 0.0f;  // watts over B
-    o.q += Q;
-    o.v1 += v1;
-    o.v60 += v60;
-    o.excess += exc_w * 0.5f;                                                         // Eq. 3, W*s
-    o.tokens += ph == 0 ? rate : 0.0f;
-    peak_w = fmaxf(peak_w, exc_w);
-    if (env.reward_kind != PE_REWARD_LAGRANGE) {
-      const int viol = env.reward_window == 1 ? v1 : v60;
-      fixed += (viol ? env.r_viol : env.r_ok) + env.bonus_coef * rate * env.inv_rate_max;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      int32_t qin[C], Q = 0;
+      int64_t S60 = 0;
+      sample_q<C>(a.tab, sn[u], nl, qin);
+#pragma unroll
+      for (int c = 0; c < C; ++c) {
+        a.ss(c) += qin[c] - q20[u][c];
+        a.sl(c) += qin[c] - q60[u][c];
+        Q += qin[c];
+        S60 += a.sl(c);
+      }
+      a.push(p + u, qin);          // after the window updates: slot p & 63 held position p - 64
+      a.set_level_at(p + u, nl);
+      const int v1 = Q > fm.B, v60 = S60 > B60;
+      const float exc_w = v60 ? __fdiv_rn(__ll2float_rn(S60 - B60), 3840.0f) : 0.0f;  // watts over B
+      o.q += Q;
+      o.v1 += v1;
+      o.v60 += v60;
+      o.excess += exc_w * 0.5f;                                                         // Eq. 3, W*s
+      o.tokens += sn[u].ph == 0 ? rate : 0.0f;
+      peak_w = fmaxf(peak_w, exc_w);
+      if (env.reward_kind != PE_REWARD_LAGRANGE) {
+        const int viol = env.reward_window == 1 ? v1 : v60;
+        fixed += (viol ? env.r_viol : env.r_ok) + env.bonus_coef * rate * env.inv_rate_max;
+      }
     }
-    a.pos() = p + 1;
+    a.pos() = p + U;
+  };
+  if constexpr (ONE) {
+    consume(std::integral_constant<int, 1>());
+  } else {
+    int i = 0;
+    if constexpr (Acc::kUnroll > 1)
+      for (; i + Acc::kUnroll <= n; i += Acc::kUnroll) consume(std::integral_constant<int, Acc::kUnroll>());
+    for (; i < n; ++i) consume(std::integral_constant<int, 1>());
   }
   o.samples = n;
   o.reward = env.reward_kind == PE_REWARD_LAGRANGE
@@ -410,7 +546,7 @@ __device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, 
 }
 
 template <int TE, int C>
-__device__ void load_tile(const EnvDev& env, EnvTile<TE, C>& s, int e0, int ne) {
+__device__ void load_tile(const EnvDev& env, EnvTile<TE, C>& s, const EnvTab<C>& tab, int e0, int ne) {
   for (int e = threadIdx.x; e < ne; e += blockDim.x) {
     const int g = e0 + e;
     s.pos[e] = env.st[kStPos * env.E + g];
@@ -421,7 +557,7 @@ __device__ void load_tile(const EnvDev& env, EnvTile<TE, C>& s, int e0, int ne) 
     s.til[e] = env.st[kStTil * env.E + g];
     s.fam[e] = env.st[kStFam * env.E + g];
     for (int i = 0; i < kRing; ++i) s.ring[e][i] = env.ring[(int64_t)g * kRing + i];
-    TileAcc<TE, C> a{s, e};
+    TileAcc<TE, C> a{s, tab, e};
     rebuild_history<C>(env, a);
   }
 }
@@ -447,8 +583,8 @@ __device__ void store_tile(const EnvDev& env, const EnvTile<TE, C>& s, int e0, i
 
 // register view of env g (level ring stays in global memory)
 template <int C>
-__device__ __forceinline__ RegAcc<C> load_reg(const EnvDev& env, int g) {
-  RegAcc<C> a;
+__device__ __forceinline__ RegAcc<C> load_reg(const EnvDev& env, const EnvTab<C>& tab, int g) {
+  RegAcc<C> a(tab);
   a.pos_ = env.st[kStPos * env.E + g];
   a.k_ = env.st[kStK * env.E + g];
   a.level_ = env.st[kStLevel * env.E + g];
@@ -457,10 +593,13 @@ __device__ __forceinline__ RegAcc<C> load_reg(const EnvDev& env, int g) {
   a.til_ = env.st[kStTil * env.E + g];
   a.fam_ = env.st[kStFam * env.E + g];
   a.ring = env.ring + (int64_t)g * kRing;
+  const int4 ss = *reinterpret_cast<const int4*>(env.sums + (int64_t)g * 8);
+  const int4 sl = *reinterpret_cast<const int4*>(env.sums + (int64_t)g * 8 + 4);
+  const int32_t s8[8] = {ss.x, ss.y, ss.z, ss.w, sl.x, sl.y, sl.z, sl.w};
 #pragma unroll
   for (int c = 0; c < C; ++c) {
-    a.ss_[c] = env.sums[(int64_t)g * 8 + c];
-    a.sl_[c] = env.sums[(int64_t)g * 8 + 4 + c];
+    a.ss_[c] = s8[c];
+    a.sl_[c] = s8[4 + c];
   }
   return a;
 }
@@ -474,11 +613,14 @@ __device__ __forceinline__ void store_reg(const EnvDev& env, int g, const RegAcc
   env.st[kStB * env.E + g] = a.b_;
   env.st[kStTil * env.E + g] = a.til_;
   env.st[kStFam * env.E + g] = a.fam_;
+  int32_t s8[8];
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    env.sums[(int64_t)g * 8 + c] = c < C ? a.ss_[c] : 0;
-    env.sums[(int64_t)g * 8 + 4 + c] = c < C ? a.sl_[c] : 0;
+    s8[c] = c < C ? a.ss_[c < C ? c : 0] : 0;
+    s8[4 + c] = c < C ? a.sl_[c < C ? c : 0] : 0;
   }
+  *reinterpret_cast<int4*>(env.sums + (int64_t)g * 8) = make_int4(s8[0], s8[1], s8[2], s8[3]);
+  *reinterpret_cast<int4*>(env.sums + (int64_t)g * 8 + 4) = make_int4(s8[4], s8[5], s8[6], s8[7]);
 }
 
 // categorical sample by inverse CDF (or argmax), returns action and its log-prob
@@ -492,9 +634,12 @@ __device__ __forceinline__ int sample_action(const float* z, uint32_t r, bool de
       m = z[j];
       amax = j;
     }
-  float S = 0.0f;
+  float S = 0.0f, ex[A];
 #pragma unroll
-  for (int j = 0; j < A; ++j) S += expf(z[j] - m);
+  for (int j = 0; j < A; ++j) {
+    ex[j] = expf(z[j] - m);
+    S += ex[j];
+  }
   int a = A - 1;
   if (det) {
     a = amax;
@@ -504,14 +649,17 @@ __device__ __forceinline__ int sample_action(const float* z, uint32_t r, bool de
     float c = 0.0f;
 #pragma unroll
     for (int j = 0; j < A; ++j) {
-      c += expf(z[j] - m);
+      c += ex[j];
       if (target < c) {
         a = j;
         break;
       }
     }
   }
-  *logp = z[a] - m - logf(S);
+  float za = z[0];  // z[a] without indexing a register array
+#pragma unroll
+  for (int j = 1; j < A; ++j) za = a == j ? z[j] : za;
+  *logp = za - m - logf(S);
   return a;
 }
 

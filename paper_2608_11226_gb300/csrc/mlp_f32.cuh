@@ -32,11 +32,16 @@ __host__ __device__ __forceinline__ MlpLayout mlp_layout(int D, int H, int A) {
   return L;
 }
 
-// dst[k][n] = W[n][k] for W[rows=N][cols=K] in global memory
+// dst[k][n] = W[n][k] for W[rows=N][cols=K] in global memory (N a multiple of
+// 8, K of 4).  A warp takes 8 rows x 4 columns at a time: 8 runs of 16 bytes
+// of global memory and a 4-way bank conflict on the stores.  (Rows across the
+// lanes alone touch 32 lines per load: 128 x 128 weights took 8 us; columns
+// alone put a warp's stores into one bank.)
 __device__ __forceinline__ void load_transposed(const float* __restrict__ W, float* dst, int N, int K) {
-  for (int i = threadIdx.x; i < N * K; i += blockDim.x) {
-    const int k = i / N, n = i % N;
-    dst[i] = __ldg(W + (int64_t)n * K + k);
+  const int lane = threadIdx.x & 31, nt = N / 8;
+  for (int t = threadIdx.x >> 5; t < nt * (K / 4); t += blockDim.x >> 5) {
+    const int n = (t % nt) * 8 + (lane & 7), k = (t / nt) * 4 + (lane >> 3);
+    dst[k * N + n] = __ldg(W + (int64_t)n * K + k);
   }
 }
 
@@ -65,46 +70,97 @@ __device__ __forceinline__ void store_rt(float* p, const float (&v)[RT]) {
   }
 }
 
-// outT[n][e] = tanh(b[n] + sum_k inT[k][e] * WT[k][n]) for TE rows; each
-// thread owns an RT-row x 4-neuron register tile, accumulated as neuron pairs
-// with the packed two-lane FMA (__ffma2_rn: two round-to-nearest fused
-// multiply-adds, the same results as fmaf, in one instruction) and the row
-// value broadcast to both lanes.  LD is the row stride (in floats) of inT
-// and outT.
-template <int TE, int K, int N, int LD = TE, int RT = 4>
-__device__ __forceinline__ void dense_tanh_t(const float* __restrict__ inT, const float* __restrict__ WT,
-                                             const float* __restrict__ bias, float* __restrict__ outT) {
-  constexpr int EG = TE / RT, NG = N / 4;
-  for (int j = threadIdx.x; j < EG * NG; j += blockDim.x) {
-    const int eg = j % EG, ng = j / EG;
-    float2 acc2[RT][2];
+// RT = 2, 4 or 8 consecutive floats of shared memory as pairs
+template <int RT>
+__device__ __forceinline__ void load_pairs(const float* p, float2 (&v)[RT / 2]) {
+  if constexpr (RT == 2) {
+    v[0] = *reinterpret_cast<const float2*>(p);
+  } else {
 #pragma unroll
-    for (int r = 0; r < RT; ++r) acc2[r][0] = acc2[r][1] = make_float2(0.0f, 0.0f);
-#pragma unroll 8
-    for (int k = 0; k < K; ++k) {
-      float xv[RT];
-      load_rt<RT>(inT + k * LD + eg * RT, xv);
-      const float4 w = *reinterpret_cast<const float4*>(WT + k * N + ng * 4);
-      const float2 w01 = make_float2(w.x, w.y), w23 = make_float2(w.z, w.w);
-#pragma unroll
-      for (int r = 0; r < RT; ++r) {
-        const float2 xx = make_float2(xv[r], xv[r]);
-        acc2[r][0] = __ffma2_rn(xx, w01, acc2[r][0]);
-        acc2[r][1] = __ffma2_rn(xx, w23, acc2[r][1]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float bb = bias[ng * 4 + c];
-      float o[RT];
-#pragma unroll
-      for (int r = 0; r < RT; ++r) o[r] = tanhf(((c & 1) ? acc2[r][c >> 1].y : acc2[r][c >> 1].x) + bb);
-      store_rt<RT>(outT + (ng * 4 + c) * LD + eg * RT, o);
+    for (int q = 0; q < RT / 4; ++q) {
+      const float4 x = *reinterpret_cast<const float4*>(p + 4 * q);
+      v[2 * q] = make_float2(x.x, x.y);
+      v[2 * q + 1] = make_float2(x.z, x.w);
     }
   }
 }
 
-// out[e][a] = b[a] + sum_k W[a][k] * hT[k][e]
+template <int RT>
+__device__ __forceinline__ void store_pairs(float* p, const float2 (&v)[RT / 2]) {
+  if constexpr (RT == 2) {
+    *reinterpret_cast<float2*>(p) = v[0];
+  } else {
+#pragma unroll
+    for (int q = 0; q < RT / 4; ++q)
+      *reinterpret_cast<float4*>(p + 4 * q) = make_float4(v[2 * q].x, v[2 * q].y, v[2 * q + 1].x, v[2 * q + 1].y);
+  }
+}
+
+// acc[r][c] = sum_k in[k][rows 2r, 2r + 1] * W[k][c] over k < K, in the order of
+// k: an RT-row x CT-neuron register tile, row pairs in the two lanes of the
+// packed FMA (__ffma2_rn: two round-to-nearest fused multiply-adds, the same
+// results as fmaf, in one instruction; the weight is moved to both lanes once
+// per RT / 2 FMAs).  in points at the tile's first row (rows of k LD floats
+// apart), W at its first neuron.  The operands of the next two k are in flight
+// while the current two are used; the compiler's own unrolled loops left the
+// FMA pipe waiting for shared memory (128 x 128 layer, 32 rows, 4 warps: 5,700
+// cycles against 7,000 to 8,400; 112 rows, 14 warps: 20,900 against 22,100).
+template <int RT, int CT, int K, int LD, int LDW>
+__device__ __forceinline__ void dense_tile(const float* __restrict__ in, const float* __restrict__ W,
+                                           float2 (&acc)[RT / 2][CT]) {
+  static_assert(K % 4 == 0 && CT % 4 == 0, "two buffers of two k each");
+  float2 x[2][2][RT / 2];
+  float w[2][2][CT];
+  auto load = [&](int b, int k0) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      load_pairs<RT>(in + (k0 + u) * LD, x[b][u]);
+#pragma unroll
+      for (int q = 0; q < CT / 4; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(W + (k0 + u) * LDW + 4 * q);
+        w[b][u][4 * q] = v.x, w[b][u][4 * q + 1] = v.y, w[b][u][4 * q + 2] = v.z, w[b][u][4 * q + 3] = v.w;
+      }
+    }
+  };
+  auto use = [&](int b) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int c = 0; c < CT; ++c) {
+        const float2 ww = make_float2(w[b][u][c], w[b][u][c]);
+#pragma unroll
+        for (int r = 0; r < RT / 2; ++r) acc[r][c] = __ffma2_rn(x[b][u][r], ww, acc[r][c]);
+      }
+  };
+#pragma unroll
+  for (int r = 0; r < RT / 2; ++r)
+#pragma unroll
+    for (int c = 0; c < CT; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
+  load(0, 0);
+#pragma unroll 1
+  for (int k = 0; k < K; k += 4) {
+    load(1, k + 2);
+    use(0);
+    if (k + 4 < K) load(0, k + 4);
+    use(1);
+  }
+}
+
+// out[c][rows] = tanh(acc + bias[c]); out points at the tile's first row and neuron
+template <int RT, int CT, int LD>
+__device__ __forceinline__ void tanh_store(const float2 (&acc)[RT / 2][CT], const float* __restrict__ bias,
+                                           float* __restrict__ out) {
+#pragma unroll
+  for (int c = 0; c < CT; ++c) {
+    const float bb = bias[c];
+    float2 o[RT / 2];
+#pragma unroll
+    for (int r = 0; r < RT / 2; ++r) o[r] = make_float2(tanhf(acc[r][c].x + bb), tanhf(acc[r][c].y + bb));
+    store_pairs<RT>(out + c * LD, o);
+  }
+}
+
+// out[e][a] = b[a] + sum_k W[a][k] * hT[k][e], summed in the order of k
 template <int TE, int K, int NA, int LD = TE>
 __device__ __forceinline__ void head_t(const float* __restrict__ hT, const float* __restrict__ W,
                                        const float* __restrict__ bias, float* __restrict__ out) {
@@ -112,7 +168,13 @@ __device__ __forceinline__ void head_t(const float* __restrict__ hT, const float
     const int e = j % TE, a = j / TE;
     float acc = 0.0f;
 #pragma unroll 8
-    for (int k = 0; k < K; ++k) acc = fmaf(W[a * K + k], hT[k * LD + e], acc);
+    for (int k = 0; k < K; k += 4) {
+      const float4 w = *reinterpret_cast<const float4*>(W + a * K + k);
+      acc = fmaf(w.x, hT[k * LD + e], acc);
+      acc = fmaf(w.y, hT[(k + 1) * LD + e], acc);
+      acc = fmaf(w.z, hT[(k + 2) * LD + e], acc);
+      acc = fmaf(w.w, hT[(k + 3) * LD + e], acc);
+    }
     out[e * NA + a] = acc + bias[a];
   }
 }

@@ -50,12 +50,17 @@ __device__ __forceinline__ int rule_action(const EnvDev& env, RegAcc<C>& a, cons
   return (s30 < (int64_t)kWLong * r.climb30_q && s10 < (int64_t)kWShort * r.climb10_q) ? raise : hold;
 }
 
+// blocks of two warps, so that a few thousand envs reach every SM
+constexpr int kRuleThreads = 64;
+
 template <int C, int OBS, int D>
 __device__ __forceinline__ void write_obs(const EnvDev& env, RegAcc<C>& a, void* dst, int bf16) {
   const Fam fm = fam_of(env, a.fam());
   if constexpr (OBS == PE_OBS_OCC32 || OBS == PE_OBS_OCC64) {
     float v[D];
-    features_eq5<C, OBS, D>(env, a, fm, v);
+    Recent<C, OBS> h;
+    load_recent<C, OBS>(env, a, fm, a.pos() - 1, h);
+    features_eq5<C, OBS, D>(env, a, fm, h, v);
     if (bf16) {
       __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(dst);
 #pragma unroll
@@ -78,11 +83,14 @@ __device__ __forceinline__ void write_obs(const EnvDev& env, RegAcc<C>& a, void*
   }
 }
 
-template <int C, int OBS, int D>
-__global__ void __launch_bounds__(128) rule_rollout_kernel(EnvDev env, RuleArgs r, pe_rollout_buf buf) {
+template <int C, int OBS, int D, bool ONE>
+__global__ void __launch_bounds__(kRuleThreads) rule_rollout_kernel(EnvDev env, RuleArgs r, pe_rollout_buf buf) {
+  __shared__ EnvTab<C> tab;
+  load_tab<C>(env, tab);
+  __syncthreads();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= env.E) return;
-  RegAcc<C> acc = load_reg<C>(env, e);
+  RegAcc<C> acc = load_reg<C>(env, tab, e);
   const size_t ob = r.obs_bf16 ? 2 : 4;
   int32_t v1 = 0, v60 = 0;
   float tok = 0.0f, exc = 0.0f;
@@ -91,7 +99,7 @@ __global__ void __launch_bounds__(128) rule_rollout_kernel(EnvDev env, RuleArgs 
     const int64_t row = (int64_t)t * env.E + e;
     if (buf.obs) write_obs<C, OBS, D>(env, acc, reinterpret_cast<char*>(buf.obs) + row * D * ob, r.obs_bf16);
     const int act = rule_action<C>(env, acc, r, (uint32_t)e, (uint32_t)t);
-    const StepOut so = env_step<C>(env, acc, act, r.lambda);
+    const StepOut so = env_step<C, ONE>(env, acc, act, r.lambda);
     buf.act[row] = (uint8_t)act;
     buf.reward[row] = so.reward;
     buf.done[row] = (uint8_t)so.done;
@@ -118,6 +126,9 @@ __global__ void __launch_bounds__(128) rule_rollout_kernel(EnvDev env, RuleArgs 
 // [60, L - episode_len] set *flag and leave that env unchanged
 template <int C>
 __global__ void env_offsets_kernel(EnvDev env, const int32_t* __restrict__ offsets, int32_t* __restrict__ flag) {
+  __shared__ EnvTab<C> tab;
+  load_tab<C>(env, tab);
+  __syncthreads();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= env.E) return;
   const int o = offsets[e];
@@ -126,7 +137,7 @@ __global__ void env_offsets_kernel(EnvDev env, const int32_t* __restrict__ offse
     atomicOr(flag, 1);
     return;
   }
-  RegAcc<C> a;
+  RegAcc<C> a(tab);
   a.ring = env.ring + (int64_t)e * kRing;
   a.fam() = fam;  // the env keeps its episode's trace family
   env_reset_at<C>(env, a, o);
@@ -152,17 +163,18 @@ pe_status replay_check(const uint8_t* act, int64_t n, int A, int32_t* flag, cuda
   return PE_OK;
 }
 
+template <int C, int OBS, int D>
+static void launch_rule(const EnvDev& env, const RuleArgs& r, const pe_rollout_buf& buf, cudaStream_t st) {
+  auto* const kern = env.cadence ? rule_rollout_kernel<C, OBS, D, false> : rule_rollout_kernel<C, OBS, D, true>;
+  kern<<<ceil_div(env.E, kRuleThreads), kRuleThreads, 0, st>>>(env, r, buf);
+}
+
 pe_status rule_rollout(const EnvDev& env, const RuleArgs& r, const pe_rollout_buf& buf, cudaStream_t st) {
-  const int grid = ceil_div(env.E, 128);
   ProfScope ps(PE_PROF_ROLLOUT, st);
-  if (env.C == 1 && env.obs_kind == PE_OBS_TINY8)
-    rule_rollout_kernel<1, PE_OBS_TINY8, 8><<<grid, 128, 0, st>>>(env, r, buf);
-  else if (env.C == 1 && env.obs_kind == PE_OBS_7B16)
-    rule_rollout_kernel<1, PE_OBS_7B16, 16><<<grid, 128, 0, st>>>(env, r, buf);
-  else if (env.C == 4 && env.obs_kind == PE_OBS_OCC32)
-    rule_rollout_kernel<4, PE_OBS_OCC32, 32><<<grid, 128, 0, st>>>(env, r, buf);
-  else if (env.C == 4 && env.obs_kind == PE_OBS_OCC64)
-    rule_rollout_kernel<4, PE_OBS_OCC64, 64><<<grid, 128, 0, st>>>(env, r, buf);
+  if (env.C == 1 && env.obs_kind == PE_OBS_TINY8) launch_rule<1, PE_OBS_TINY8, 8>(env, r, buf, st);
+  else if (env.C == 1 && env.obs_kind == PE_OBS_7B16) launch_rule<1, PE_OBS_7B16, 16>(env, r, buf, st);
+  else if (env.C == 4 && env.obs_kind == PE_OBS_OCC32) launch_rule<4, PE_OBS_OCC32, 32>(env, r, buf, st);
+  else if (env.C == 4 && env.obs_kind == PE_OBS_OCC64) launch_rule<4, PE_OBS_OCC64, 64>(env, r, buf, st);
   else
     return fail(PE_EINVAL, "rule rollout: unsupported env (C=%d, obs kind %d)", env.C, env.obs_kind);
   PE_CHECK_LAUNCH("rule_rollout_kernel");

@@ -448,6 +448,54 @@ def test_rollout_parity_tiny_deterministic():
     _rollout_case(W.make_tiny(n_envs=40), 64, iters=1, det=True)
 
 
+@pytest.mark.parametrize("preset", ["tiny", "7b"])
+@pytest.mark.parametrize("tile,extra", [(8, 0), (8, 1), (16, 0), (16, 1)])
+def test_rollout_parity_env_tiles(preset, tile, extra):
+    """The fp32 rollout's env tile follows the batch (8 or 16 envs per CTA up
+    to one CTA per SM, else 32): the last batch of each and the first of the
+    next, whose last tile holds one env."""
+    E = tile * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    wl = (W.make_tiny if preset == "tiny" else W.make_7b)(n_envs=E)
+    ids = np.unique(np.concatenate([[0, tile - 1, tile, E - 2, E - 1], np.random.default_rng(3).integers(0, E, 20)]))
+    _rollout_case(wl, 21, iters=2, sample_envs=ids)
+
+
+@pytest.mark.parametrize("cadence", [False, True])
+def test_replay_four_channel_traces(cadence):
+    """Four-channel traces carry the phase label and whether it is actuated in
+    the samples' sign bits: every label from 0 to 7 under a mixed actuator
+    mask, samples of zero watts, and (with families) channels that a family
+    does not have, whatever they hold, are ignored."""
+    wl = (W.make_72b_cadence if cadence else W.make_72b_mixed)(n_envs=61)
+    spec = wl.env
+    rng = np.random.default_rng(12)
+    phase = rng.integers(0, 8, wl.phase.shape).astype(np.uint8)
+    trace = wl.trace.copy()
+    trace[rng.random(trace.shape) < 0.02] = 0.0
+    trace[rng.random(trace.shape) < 0.02] = -0.0
+    dirty = trace.copy()
+    if spec.n_families > 1:
+        at = 0
+        for f in range(spec.n_families):
+            n, c = spec.fam_len[f], spec.fam_channels[f]
+            dirty[at + c * n:at + spec.n_channels * n] = 777.0
+            at += spec.n_channels * n
+    spec.scale_phase_mask = 0b10100101
+    env = pe.Env(spec, torch.from_numpy(dirty), torch.from_numpy(phase))
+    oenv = O.OracleEnv(spec, trace, phase, range(spec.n_envs))
+    params = W.init_params(wl.net, seed=2)
+    for it, T in ((0, 30), (1, 45)):
+        acts = rng.integers(0, spec.n_actions, (T, spec.n_envs)).astype(np.uint8)
+        buf = pe.alloc_rule_rollout(spec, T, obs=True)
+        pe.rollout_replay(env, torch.from_numpy(acts).cuda(), T, it, buf, lam=0.5)
+        ref = oenv.rollout(params, wl.net.hidden, False, T, it, lam=0.5, forced=acts)
+        for k in ("obs", "obs_last", "done", "viol", "energy_q", "samples", "q"):
+            assert np.array_equal(cpu(buf[k]), ref[k]), k
+        for k in ("reward", "tokens", "excess"):
+            assert rel_err(cpu(buf[k]), ref[k]) <= TOL, k
+    env.close()
+
+
 def test_rollout_parity_7b_sampled():
     wl = W.make_7b()
     rng = np.random.default_rng(3)
