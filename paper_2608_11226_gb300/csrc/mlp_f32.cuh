@@ -49,27 +49,6 @@ __device__ __forceinline__ void load_copy(const float* __restrict__ src, float* 
   for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = __ldg(src + i);
 }
 
-// RT consecutive floats (RT = 2 or 4) from shared memory
-template <int RT>
-__device__ __forceinline__ void load_rt(const float* p, float (&v)[RT]) {
-  if constexpr (RT == 4) {
-    const float4 q = *reinterpret_cast<const float4*>(p);
-    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-  } else {
-    const float2 q = *reinterpret_cast<const float2*>(p);
-    v[0] = q.x; v[1] = q.y;
-  }
-}
-
-template <int RT>
-__device__ __forceinline__ void store_rt(float* p, const float (&v)[RT]) {
-  if constexpr (RT == 4) {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-  } else {
-    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
-  }
-}
-
 // RT = 2, 4 or 8 consecutive floats of shared memory as pairs
 template <int RT>
 __device__ __forceinline__ void load_pairs(const float* p, float2 (&v)[RT / 2]) {

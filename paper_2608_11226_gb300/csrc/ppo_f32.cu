@@ -37,7 +37,6 @@ namespace pe {
 constexpr int kPpoS = 128;          // samples per slice (a 7B CTA's whole share of a minibatch)
 constexpr int kPpoLD = kPpoS + 4;   // row stride of feature-major activations
 constexpr int kPpoNT = 512;         // threads per gradient CTA
-constexpr int kPpoRT = 4;           // sample rows per thread tile in the dense layers
 constexpr int kPpoMaxEpochs = 16;
 constexpr int kPpoMaxNC = 128;      // CTAs per network: above half the SMs of any GB300
 
@@ -88,115 +87,111 @@ __global__ void ppo_advstats_kernel(const float* __restrict__ adv, int64_t N, in
 }
 
 // Dense-layer register tiles for the sample slices: a thread owns RT
-// sample rows x 4 neurons; a warp covers 2 row groups x 16 neuron groups (the
-// fastest of the warp shapes measured on the 7B network: 2x16, 4x8, 8x4 and
-// 16x2 lie within 3% of each other).
-template <int TE, int N, int RT>
-__device__ __forceinline__ bool dense_job(int j, int& eg, int& ng) {
-  constexpr int EG = TE / RT, NG = N / 4, BE = EG / 2;  // BE: 2-row-group blocks along the slice
-  static_assert(EG % 2 == 0 && NG % 16 == 0, "dense tile layout");
-  const int wb = j >> 5, lane = j & 31;
-  eg = (wb % BE) * 2 + (lane & 1);
-  ng = (wb / BE) * 16 + (lane >> 1);
-  return ng < NG;
+// samples x 4 outputs (dense_tile; per output the sum runs over k in order,
+// whatever the tile).  A warp covers 2 sample groups x 16 output groups (4 x 8
+// and 1 x 32 lie within 3% of it, 8 x 4 and 16 x 2 take up to 1.8 times as
+// long: their sample loads fall into the same banks).
+template <int N, int RT, class F>
+__device__ __forceinline__ void dense_jobs(int SV, F f) {
+  constexpr int NB = N / 4 / 16;
+  static_assert(N % 64 == 0 && (RT == 2 || RT == 4), "dense tile layout");
+  const int lane = threadIdx.x & 31, eb = SV / RT / 2 + (SV / RT % 2);  // 2-group blocks along the slice
+  for (int w = threadIdx.x >> 5; w < eb * NB; w += kPpoNT / 32) {
+    const int eg = (w % eb) * 2 + (lane & 1), ng = (w / eb) * 16 + (lane >> 1);
+    if (eg * RT < SV) f(eg, ng);
+  }
 }
 
 // outT[n][e] = tanh(b[n] + sum_k inT[k][e] WT[k][n]) for samples e < SV (a
-// multiple of RT; later rows are left as they are); WT rows are LDW floats apart.
-// Neuron pairs accumulate with the packed two-lane FMA (__ffma2_rn: two
-// round-to-nearest fused multiply-adds, the same results as fmaf, in one
-// instruction), the sample value broadcast to both lanes.
-template <int TE, int K, int N, int LD, int RT, int LDW = N>
-__device__ __forceinline__ void dense_fwd_w(const float* __restrict__ inT, const float* __restrict__ WT,
-                                            const float* __restrict__ bias, float* __restrict__ outT, int SV) {
-  constexpr int JOBS = (TE / RT) * (N / 4);
-  for (int j = threadIdx.x; j < JOBS; j += blockDim.x) {
-    int eg, ng;
-    if (!dense_job<TE, N, RT>(j, eg, ng) || eg * RT >= SV) continue;
-    float2 acc2[RT][2];
-#pragma unroll
-    for (int r = 0; r < RT; ++r) acc2[r][0] = acc2[r][1] = make_float2(0.0f, 0.0f);
-#pragma unroll 8
-    for (int k = 0; k < K; ++k) {
-      float xv[RT];
-      load_rt<RT>(inT + k * LD + eg * RT, xv);
-      const float4 w = *reinterpret_cast<const float4*>(WT + k * LDW + ng * 4);
-      const float2 w01 = make_float2(w.x, w.y), w23 = make_float2(w.z, w.w);
-#pragma unroll
-      for (int r = 0; r < RT; ++r) {
-        const float2 xx = make_float2(xv[r], xv[r]);
-        acc2[r][0] = __ffma2_rn(xx, w01, acc2[r][0]);
-        acc2[r][1] = __ffma2_rn(xx, w23, acc2[r][1]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float bb = bias[ng * 4 + c];
-      float o[RT];
-#pragma unroll
-      for (int r = 0; r < RT; ++r) o[r] = tanhf(((c & 1) ? acc2[r][c >> 1].y : acc2[r][c >> 1].x) + bb);
-      store_rt<RT>(outT + (ng * 4 + c) * LD + eg * RT, o);
-    }
-  }
+// multiple of 8; later rows are left as they are); WT rows are LDW floats apart.
+template <int K, int N, int LD, int RT, int LDW>
+__device__ __forceinline__ void dense_fwd_tile(const float* __restrict__ inT, const float* __restrict__ WT,
+                                               const float* __restrict__ bias, float* __restrict__ outT, int SV) {
+  dense_jobs<N, RT>(SV, [&](int eg, int ng) {
+    float2 acc[RT / 2][4];
+    dense_tile<RT, 4, K, LD, LDW>(inT + eg * RT, WT + ng * 4, acc);
+    tanh_store<RT, 4, LD>(acc, bias + ng * 4, outT + ng * 4 * LD + eg * RT);
+  });
 }
 
 // back through a tanh layer, in place, from the transposed weights:
 //   hT[k][e] <- (sum_n inT[n][e] W[n][k]) * (1 - hT[k][e]^2),  W[n][k] = WT[k][n]
-// A thread owns RT = 4 samples x 4 outputs k; per 4 n it loads a 4x4 block of
-// WT (rows k, columns n..n+3) and of inT and does 64 FMAs as 32 packed
-// two-lane FMAs over sample pairs (the weight broadcast to both lanes).  A warp covers 16
-// sample groups x 2 output groups, so its WT loads touch two rows (4 rows
-// apart, different banks with the padded stride) and are broadcasts.
-template <int TE, int K, int N, int LD, int LDW>
-__device__ __forceinline__ void dense_bwd_wt(const float* __restrict__ inT, const float* __restrict__ WT,
-                                             float* hT, int SV) {
-  constexpr int RT = 4, EG = TE / RT, NG = N / 4, JOBS = EG * NG;
-  static_assert(K % 4 == 0 && EG % 16 == 0, "backward tile layout");
-  for (int j = threadIdx.x; j < JOBS; j += blockDim.x) {
-    const int eg = j % EG, kg = j / EG;
-    if (eg * RT >= SV) continue;  // samples past the slice's valid rows
-    float2 acc2[2][4];  // acc2[rp][c] = (acc[2 rp][c], acc[2 rp + 1][c])
+// A thread owns RT samples x the 4 outputs k = kg + c N / 4; per 4 n it loads
+// a 4 x 4 block of WT (rows k, columns n .. n + 3; rows of adjacent kg fall in
+// different banks with the padded stride) and 4 rows of inT.
+template <int K, int N, int LD, int RT, int LDW>
+__device__ __forceinline__ void dense_bwd_tile(const float* __restrict__ inT, const float* __restrict__ WT, float* hT,
+                                               int SV) {
+  static_assert(K % 4 == 0, "backward tile layout");
+  dense_jobs<N, RT>(SV, [&](int eg, int kg) {
+    float2 acc[RT / 2][4];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc2[0][c] = acc2[1][c] = make_float2(0.0f, 0.0f);
+    for (int r = 0; r < RT / 2; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.0f, 0.0f);
 #pragma unroll 2
     for (int n = 0; n < K; n += 4) {
-      float4 w[4], d[4];
+      float4 w[4];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) w[c] = *reinterpret_cast<const float4*>(WT + (kg * 4 + c) * LDW + n);
+      for (int c = 0; c < 4; ++c) w[c] = *reinterpret_cast<const float4*>(WT + (kg + c * (N / 4)) * LDW + n);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) d[q] = *reinterpret_cast<const float4*>(inT + (n + q) * LD + eg * RT);
+      for (int q = 0; q < 4; ++q) {
+        float2 d[RT / 2];
+        load_pairs<RT>(inT + (n + q) * LD + eg * RT, d);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float wc[4] = {w[c].x, w[c].y, w[c].z, w[c].w};
+        for (int c = 0; c < 4; ++c) {
+          const float wv = q == 0 ? w[c].x : q == 1 ? w[c].y : q == 2 ? w[c].z : w[c].w;
+          const float2 ww = make_float2(wv, wv);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float2 ww = make_float2(wc[q], wc[q]);
-          acc2[0][c] = __ffma2_rn(make_float2(d[q].x, d[q].y), ww, acc2[0][c]);
-          acc2[1][c] = __ffma2_rn(make_float2(d[q].z, d[q].w), ww, acc2[1][c]);
+          for (int r = 0; r < RT / 2; ++r) acc[r][c] = __ffma2_rn(d[r], ww, acc[r][c]);
         }
       }
     }
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      float h[RT], o[RT];
-      load_rt<RT>(hT + (kg * 4 + c) * LD + eg * RT, h);
-      const float a4[4] = {acc2[0][c].x, acc2[0][c].y, acc2[1][c].x, acc2[1][c].y};
+      float* hp = hT + (kg + c * (N / 4)) * LD + eg * RT;
+      float2 h[RT / 2], o[RT / 2];
+      load_pairs<RT>(hp, h);
 #pragma unroll
-      for (int r = 0; r < RT; ++r) o[r] = a4[r] * (1.0f - h[r] * h[r]);
-      store_rt<RT>(hT + (kg * 4 + c) * LD + eg * RT, o);
+      for (int r = 0; r < RT / 2; ++r)
+        o[r] = make_float2(acc[r][c].x * (1.0f - h[r].x * h[r].x), acc[r][c].y * (1.0f - h[r].y * h[r].y));
+      store_pairs<RT>(hp, o);
     }
-  }
+  });
+}
+
+// The tile by the slice's rows: 4 samples per thread, 2 up to 32 rows (the
+// short slices of small minibatches are latency, and smaller tiles spread them
+// over more warps).  8 samples per thread took 25,500 cycles instead of 22,100
+// for the forward 128 x 128 layer of a 7B CTA's 112 rows (a longer tanh tail
+// per thread, and spills), backward 21,000 instead of 19,300 by itself (16
+// sample groups across a warp, as before: 26,500).
+template <int K, int N, int LD, int LDW = N>
+__device__ __forceinline__ void dense_fwd_w(const float* __restrict__ inT, const float* __restrict__ WT,
+                                            const float* __restrict__ bias, float* __restrict__ outT, int SV) {
+  if (SV > 32) dense_fwd_tile<K, N, LD, 4, LDW>(inT, WT, bias, outT, SV);
+  else dense_fwd_tile<K, N, LD, 2, LDW>(inT, WT, bias, outT, SV);
+}
+
+template <int K, int N, int LD, int LDW>
+__device__ __forceinline__ void dense_bwd_wt(const float* __restrict__ inT, const float* __restrict__ WT, float* hT,
+                                             int SV) {
+  if (SV > 32) dense_bwd_tile<K, N, LD, 4, LDW>(inT, WT, hT, SV);
+  else dense_bwd_tile<K, N, LD, 2, LDW>(inT, WT, hT, SV);
 }
 
 // dst[m][n] (+)= sum_s aT[m][s] bT[n][s] (weight gradients).  Each thread owns
-// 4x4 tiles whose rows and columns are interleaved (m = mg + i*M/4,
+// TR x 4 tiles whose rows and columns are interleaved (m = mg + i*M/TR,
 // n = ng + j*N/4); a warp covers WM x WN (mg, ng) pairs, so one float4 load of
 // the warp touches WM (or WN) distinct rows in distinct shared-memory bank
-// groups: one wavefront each.
-template <int M, int N, int NT>
+// groups, and a store of the warp WM runs of WN floats of the partial row.  TR
+// = 8 where the tiles number the threads (the 128 x 128 layer: 12 loads per
+// 128 FMAs against 8 per 64), with WM = 2: 112 samples take 21,200 cycles, TR
+// = 4 with WM = 8 took 27,400.
+template <int M, int N, int NT, int TR>
 struct WGradAcc {
-  static constexpr int MG = M / 4, NG = N / 4;
-  static constexpr int WN = NG < 4 ? NG : 4, WM = 32 / WN;
+  static constexpr int MG = M / TR, NG = N / 4;
+  static constexpr int WN = NG < 16 ? NG : 16, WM = 32 / WN;
   static constexpr int TM = (MG + WM - 1) / WM, TN = NG / WN;
   static constexpr int NWARP = NT / 32, WT = TM * TN, PER = (WT + NWARP - 1) / NWARP;
   __device__ __forceinline__ bool job(int q, int& mg, int& ng) const {
@@ -205,7 +200,7 @@ struct WGradAcc {
     ng = (wt % TN) * WN + lane % WN;
     return wt < WT && mg < MG;
   }
-  // dst (+)= sum_s aT[m][s] bT[n][s] over s < SV, one 4x4 tile at a time (16
+  // dst (+)= sum_s aT[m][s] bT[n][s] over s < SV, one tile at a time (4 TR
   // packed accumulators live), even and odd samples in the two lanes of a
   // packed two-lane FMA and added at the end; rows of dst ld floats apart
   template <int S, int LD>
@@ -215,28 +210,28 @@ struct WGradAcc {
     for (int q = 0; q < PER; ++q) {
       int mg, ng;
       if (!job(q, mg, ng)) continue;
-      float2 v2[4][4];
+      float2 v2[TR][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) v2[i][j] = make_float2(0.0f, 0.0f);
-#pragma unroll 2
+#pragma unroll(TR == 4 ? 2 : 1)
       for (int s = 0; s < SV; s += 4) {
-        float4 a[4], b[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(aT + (mg + i * MG) * LD + s);
+        float4 b[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(bT + (ng + j * NG) * LD + s);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < TR; ++i) {
+          const float4 a = *reinterpret_cast<const float4*>(aT + (mg + i * MG) * LD + s);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            v2[i][j] = __ffma2_rn(make_float2(a[i].x, a[i].y), make_float2(b[j].x, b[j].y), v2[i][j]);
-            v2[i][j] = __ffma2_rn(make_float2(a[i].z, a[i].w), make_float2(b[j].z, b[j].w), v2[i][j]);
+            v2[i][j] = __ffma2_rn(make_float2(a.x, a.y), make_float2(b[j].x, b[j].y), v2[i][j]);
+            v2[i][j] = __ffma2_rn(make_float2(a.z, a.w), make_float2(b[j].z, b[j].w), v2[i][j]);
           }
+        }
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TR; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           float* d = dst + (mg + i * MG) * ld + ng + j * NG;
@@ -423,10 +418,10 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
   // head backward: thread (k = tid / 4, quarter q = tid % 4) owns row k of the
   // head weight gradient and of the layer-2 bias gradient over samples 4i + q
   const int hk = tid >> 2, hq = tid & 3;
-  float g3[NA], gb2 = 0.0f, gb1 = 0.0f, gb3 = 0.0f;
-#pragma unroll
-  for (int a = 0; a < NA; ++a) g3[a] = 0.0f;
-  float st[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // pg, entropy, kl, clip, value (threads < S)
+  // no sum lives in registers from one phase to the next (the weight-gradient
+  // tiles take them all): each slice's goes to the partial row, or to the
+  // statistics in shared memory, at once
+  auto put = [&](int64_t at, float v) { row[at] = nsl == 0 ? v : row[at] + v; };
 
   for (int base = c0; base < c1; base += S) {
     // nv valid samples; the tiles cover the first SV rows (nv rounded up to
@@ -439,9 +434,9 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
     }
     __syncthreads();
     // forward
-    dense_fwd_w<S, D, H, LD, kPpoRT>(s.xt, s.w1t, s.b1, s.h1t, SV);
+    dense_fwd_w<D, H, LD>(s.xt, s.w1t, s.b1, s.h1t, SV);
     __syncthreads();
-    dense_fwd_w<S, H, H, LD, kPpoRT, w2t_ld<H>()>(s.h1t, s.w2t, s.b2, s.h2t, SV);
+    dense_fwd_w<H, H, LD, w2t_ld<H>()>(s.h1t, s.w2t, s.b2, s.h2t, SV);
     __syncthreads();
     // head: job (sample si = j / 8, K-part q = j % 8) sums k = q, q+8, ...
     // for every action; the 8 parts (adjacent lanes) are shuffle-combined
@@ -472,6 +467,7 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
     __syncthreads();
     // loss terms and dLoss/dhead per sample (written over the head outputs)
     if (tid < S) {
+      float st[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};  // pg, entropy, kl, clip, value
       float* z = s.z + tid * NA;
       if (!s.valid[tid]) {
 #pragma unroll
@@ -501,26 +497,37 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
         const float rho = expf(logr);
         const float rc = fminf(fmaxf(rho, 1.0f - g.clip), 1.0f + g.clip);
         const float s1 = rho * an, s2 = rc * an;
-        st[0] += -fminf(s1, s2);
-        st[1] += Hs;
-        st[2] += kl_term(logr);
-        st[3] += fabsf(rho - 1.0f) > g.clip ? 1.0f : 0.0f;
+        st[0] = -fminf(s1, s2);
+        st[1] = Hs;
+        st[2] = kl_term(logr);
+        st[3] = fabsf(rho - 1.0f) > g.clip ? 1.0f : 0.0f;
         const float dlp = (s1 <= s2 ? -an : 0.0f) * rho * g.inv_cnt;
 #pragma unroll
         for (int j = 0; j < NA; ++j)
           z[j] = dlp * ((j == a ? 1.0f : 0.0f) - p[j]) + g.ent_coef * g.inv_cnt * p[j] * (lp[j] + Hs);
       } else {
         const float V = z[0], R = s.ret[tid];
-        st[4] += (R - V) * (R - V);
+        st[4] = (R - V) * (R - V);
         z[0] = g.vf_coef * 2.0f * (V - R) * g.inv_cnt;
+      }
+      // the sample's statistics take its inputs' place; warps that the
+      // layer-1 weight gradient leaves idle sum them
+      s.lpo[tid] = POL ? st[0] : st[4];
+      if (POL) {
+        s.advn[tid] = st[1];
+        s.ret[tid] = st[2];
+        s.act[tid] = __float_as_int(st[3]);
       }
     }
     __syncthreads();
     // head weight gradient, back through the head into layer 2 (in place over h2)
     if (hk < H) {
-      float w3k[NA];
+      float w3k[NA], g3[NA], gb2 = 0.0f;
 #pragma unroll
-      for (int a = 0; a < NA; ++a) w3k[a] = s.w3[a * H + hk];
+      for (int a = 0; a < NA; ++a) {
+        w3k[a] = s.w3[a * H + hk];
+        g3[a] = 0.0f;
+      }
 #pragma unroll 4
       for (int i = 0; i < SV / 4; ++i) {
         const int si = 4 * i + hq;
@@ -536,26 +543,50 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
         s.h2t[hk * LD + si] = d2;
         gb2 += d2;
       }
+#pragma unroll
+      for (int a = 0; a < NA; ++a) {
+        g3[a] += __shfl_xor_sync(0xffffffffu, g3[a], 1);
+        g3[a] += __shfl_xor_sync(0xffffffffu, g3[a], 2);
+      }
+      gb2 += __shfl_xor_sync(0xffffffffu, gb2, 1);
+      gb2 += __shfl_xor_sync(0xffffffffu, gb2, 2);
+      if (hq == 0) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a) put(oW3 + (int64_t)a * H + hk, g3[a]);
+        put(oB2 + hk, gb2);
+      }
     }
     if (tid < NA) {
       float acc = 0.0f;
       for (int si = 0; si < S; ++si) acc += s.z[si * NA + tid];
-      gb3 += acc;
+      put(oB3 + tid, acc);
     }
     __syncthreads();
     // layer-2 weight gradient
     {
-      WGradAcc<H, H, kPpoNT> g2;
+      WGradAcc<H, H, kPpoNT, (H >= 128 ? 8 : 4)> g2;
       g2.template accumulate<S, LD>(s.h2t, s.h1t, SV, row + oW2, H, nsl == 0);
     }
     __syncthreads();
     // back into layer 1 (in place over h1)
-    dense_bwd_wt<S, H, H, LD, w2t_ld<H>()>(s.h2t, s.w2t, s.h1t, SV);
+    dense_bwd_wt<H, H, LD, w2t_ld<H>()>(s.h2t, s.w2t, s.h1t, SV);
     __syncthreads();
     // layer-1 weight and bias gradients (the bias by the warps the tiles leave idle)
     {
-      WGradAcc<H, D, kPpoNT> g1;
+      WGradAcc<H, D, kPpoNT, 4> g1;
       g1.template accumulate<S, LD>(s.h1t, s.xt, SV, row + oW1, D, nsl == 0);
+    }
+    if (tid >= kPpoNT - H - S && tid < kPpoNT - H) {
+      // statistics per 32 samples, fixed shuffle tree
+      const int si = tid - (kPpoNT - H - S);
+      float st[4] = {s.lpo[si], POL ? s.advn[si] : 0.0f, POL ? s.ret[si] : 0.0f, POL ? __int_as_float(s.act[si]) : 0.0f};
+#pragma unroll
+      for (int k = 0; k < (POL ? 4 : 1); ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) st[k] += __shfl_xor_sync(0xffffffffu, st[k], o);
+        float& at = s.stat[si >> 5][POL ? k : 4];
+        if ((si & 31) == 0) at = nsl == 0 ? st[k] : at + st[k];
+      }
     }
     if (tid >= kPpoNT - H) {
       const int n = tid - (kPpoNT - H), lane = tid & 31;
@@ -564,39 +595,18 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
         const int e = (i + lane) & (S - 1);
         if (e < SV) acc += s.h1t[n * LD + e];
       }
-      gb1 += acc;
+      put(oB1 + n, acc);
     }
     ++nsl;
   }
-  // the rest of the partial gradient row (the hidden-layer weight gradients
-  // are zero if the CTA's share held no sample)
+  // a share without samples
   if (nsl == 0) {
     for (int i = tid; i < H * H; i += blockDim.x) row[oW2 + i] = 0.0f;
     for (int i = tid; i < H * D; i += blockDim.x) row[oW1 + i] = 0.0f;
-  }
-#pragma unroll
-  for (int a = 0; a < NA; ++a) {
-    g3[a] += __shfl_xor_sync(0xffffffffu, g3[a], 1);
-    g3[a] += __shfl_xor_sync(0xffffffffu, g3[a], 2);
-  }
-  gb2 += __shfl_xor_sync(0xffffffffu, gb2, 1);
-  gb2 += __shfl_xor_sync(0xffffffffu, gb2, 2);
-  if (hq == 0 && hk < H) {
-#pragma unroll
-    for (int a = 0; a < NA; ++a) row[oW3 + (int64_t)a * H + hk] = g3[a];
-    row[oB2 + hk] = gb2;
-  }
-  if (tid >= kPpoNT - H) row[oB1 + tid - (kPpoNT - H)] = gb1;
-  if (tid < NA) row[oB3 + tid] = gb3;
-  // statistics of the CTA's samples (held by threads < S), fixed shuffle tree
-  if (tid < S) {
-#pragma unroll
-    for (int k = 0; k < 5; ++k)
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) st[k] += __shfl_xor_sync(0xffffffffu, st[k], o);
-    if ((tid & 31) == 0)
-#pragma unroll
-      for (int k = 0; k < 5; ++k) s.stat[tid >> 5][k] = st[k];
+    for (int i = tid; i < NA * H; i += blockDim.x) row[oW3 + i] = 0.0f;
+    if (tid < H) row[oB1 + tid] = row[oB2 + tid] = 0.0f;
+    if (tid < NA) row[oB3 + tid] = 0.0f;
+    if (tid < S / 32 * 8) s.stat[tid / 8][tid % 8] = 0.0f;
   }
   __syncthreads();
   if (tid == 0) {
@@ -604,7 +614,8 @@ __device__ __forceinline__ bool ppo_role(PpoSmem<D, H, A>& s, const PpoArgs& g, 
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
       float t = 0.0f;
-      for (int w = 0; w < S / 32; ++w) t += s.stat[w][k];
+      if ((k < 4) == POL)
+        for (int w = 0; w < S / 32; ++w) t += s.stat[w][k];
       sp[k] = t;
     }
   }
