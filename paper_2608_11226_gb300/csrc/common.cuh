@@ -83,13 +83,13 @@ __host__ __device__ __forceinline__ uint32_t lowbias32(uint32_t x) {
   return x;
 }
 
-__host__ __device__ __forceinline__ uint64_t feistel_round4(const Feistel& f, uint64_t x) {
-  const uint64_t mask = (1ull << f.half) - 1ull;
-  uint64_t L = x >> f.half, R = x & mask;
+// The domain has at most 32 bits (n < 2^31), so 32-bit words hold it.
+__host__ __device__ __forceinline__ uint32_t feistel_round4(const Feistel& f, uint32_t x) {
+  const uint32_t mask = (1u << f.half) - 1u;
+  uint32_t L = x >> f.half, R = x & mask;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
-    const uint64_t F = (uint64_t)lowbias32((uint32_t)R ^ f.k[r]) & mask;
-    const uint64_t t = L ^ F;
+    const uint32_t t = L ^ (lowbias32(R ^ f.k[r]) & mask);
     L = R;
     R = t;
   }
@@ -100,10 +100,11 @@ __host__ __device__ __forceinline__ uint64_t feistel_round4(const Feistel& f, ui
 // the Feistel map is a permutation of the domain and i < n lies on a cycle
 // that re-enters [0, n)
 __host__ __device__ __forceinline__ uint32_t feistel_index(const Feistel& f, uint64_t i) {
-  uint64_t y = feistel_round4(f, i);
+  const uint32_t n = (uint32_t)f.n;
+  uint32_t y = feistel_round4(f, (uint32_t)i);
   const uint64_t limit = 4ull * f.n + 4ull;
-  for (uint64_t it = 0; y >= f.n && it < limit; ++it) y = feistel_round4(f, y);
-  return (uint32_t)(y < f.n ? y : i % f.n);  // the fallback is unreachable for a permutation
+  for (uint64_t it = 0; y >= n && it < limit; ++it) y = feistel_round4(f, y);
+  return y < n ? y : (uint32_t)(i % f.n);  // the fallback is unreachable for a permutation
 }
 
 Feistel make_feistel(uint64_t n, uint64_t seed, uint32_t epoch, uint32_t iteration);
