@@ -128,80 +128,60 @@ __global__ void __launch_bounds__(32 * NW)
 }
 
 
-// Wide batches (E >= 32,768): one thread per V envs walks the whole horizon
+// Wide batches (E >= 32,768): one thread per env walks the whole horizon
 // backwards, A_t = delta_t + gamma lambda (1 - d_t) A_{t+1} in the same
 // order as the recursion, with no barrier and no shared memory.  The loads of
 // the next P steps are kept in flight in a register ring, so each SM holds
 // enough outstanding bytes to cover HBM latency; every warp streams
-// 32 * V consecutive envs of a row (coalesced).  Measured on GB300: one env
-// per thread with 16 loads in flight reaches 74% of the HBM copy peak at
-// 65,536 envs (14 warps per SM); at 262,144 envs four envs per thread (8
-// steps in flight) keep the launch to one wave and reach 77%, where two
-// envs per thread at 94 registers spilled into a second wave (54%).
-template <int V, int P>
-__global__ void __launch_bounds__(128)
+// 32 consecutive envs of a row (coalesced).  Measured: 2,048 steps of 262,144
+// envs with 32 steps in flight 1.59 ms, 85% of the HBM copy peak (16 steps
+// 1.62, two envs per thread 1.63, four 1.72); 1,024 x 65,536 with 16 steps and
+// blocks of 64, which spread evenly over the SMs, 197 us, 85% (blocks of 128:
+// 207 us).
+template <int P, int NT>
+__global__ void __launch_bounds__(NT)
     gae_stream_kernel(const float* __restrict__ r, const float* __restrict__ v, const uint8_t* __restrict__ d,
                       const float* __restrict__ last_v, int T, int E, float gamma, float lam,
                       float* __restrict__ adv, float* __restrict__ ret) {
-  using FV = typename std::conditional<V == 4, float4, typename std::conditional<V == 2, float2, float>::type>::type;
-  using BV = typename std::conditional<V == 4, uchar4, typename std::conditional<V == 2, uchar2, unsigned char>::type>::type;
-  const int e0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
-  if (e0 >= E) return;
+  const int e = blockIdx.x * NT + threadIdx.x;
+  if (e >= E) return;
   const float gl = gamma * lam;
-  FV rb[P], vb[P];
-  BV db[P];
+  float rb[P], vb[P];
+  uint8_t db[P];
   auto load = [&](int k, int t) {
-    const int64_t o = (int64_t)t * E + e0;
-    rb[k] = __ldcs(reinterpret_cast<const FV*>(r + o));
-    vb[k] = __ldcs(reinterpret_cast<const FV*>(v + o));
-    db[k] = __ldcs(reinterpret_cast<const BV*>(d + o));
+    const int64_t o = (int64_t)t * E + e;
+    rb[k] = __ldcs(r + o);
+    vb[k] = __ldcs(v + o);
+    db[k] = __ldcs(d + o);
   };
 #pragma unroll
   for (int k = 0; k < P; ++k)
     if (T - 1 - k >= 0) load(k, T - 1 - k);
-  float A[V], vn[V];
-  {
-    const FV q = *reinterpret_cast<const FV*>(last_v + e0);
-    const float* qp = reinterpret_cast<const float*>(&q);
-#pragma unroll
-    for (int u = 0; u < V; ++u) {
-      A[u] = 0.0f;
-      vn[u] = qp[u];
-    }
-  }
+  float A = 0.0f, vn = last_v[e];
   for (int base = T - 1; base >= 0; base -= P) {
 #pragma unroll
     for (int k = 0; k < P; ++k) {
       const int t = base - k;
       if (t >= 0) {
-        const float* rp = reinterpret_cast<const float*>(&rb[k]);
-        const float* vp = reinterpret_cast<const float*>(&vb[k]);
-        const unsigned char* dp = reinterpret_cast<const unsigned char*>(&db[k]);
-        float ao[V], ro[V];
-#pragma unroll
-        for (int u = 0; u < V; ++u) {
-          const float nt = 1.0f - (float)dp[u];
-          const float delta = rp[u] + gamma * vn[u] * nt - vp[u];
-          A[u] = delta + gl * nt * A[u];
-          ao[u] = A[u];
-          ro[u] = A[u] + vp[u];
-          vn[u] = vp[u];
-        }
+        const float nt = 1.0f - (float)db[k], vt = vb[k];
+        const float delta = rb[k] + gamma * vn * nt - vt;
+        A = delta + gl * nt * A;
+        vn = vt;
         if (t - P >= 0) load(k, t - P);
-        const int64_t o = (int64_t)t * E + e0;
-        __stcs(reinterpret_cast<FV*>(adv + o), *reinterpret_cast<FV*>(ao));
-        __stcs(reinterpret_cast<FV*>(ret + o), *reinterpret_cast<FV*>(ro));
+        const int64_t o = (int64_t)t * E + e;
+        __stcs(adv + o, A);
+        __stcs(ret + o, A + vt);
       }
     }
   }
 }
 
-template <int V, int P>
+template <int P, int NT>
 static pe_status gae_stream_run(const float* r, const float* v, const uint8_t* d, const float* last_v, int T,
                                 int E, float gamma, float lam, float* adv, float* ret, cudaStream_t st) {
   {
     ProfScope ps(PE_PROF_GAE, st);
-    gae_stream_kernel<V, P><<<ceil_div(E / V, 128), 128, 0, st>>>(r, v, d, last_v, T, E, gamma, lam, adv, ret);
+    gae_stream_kernel<P, NT><<<ceil_div(E, NT), NT, 0, st>>>(r, v, d, last_v, T, E, gamma, lam, adv, ret);
   }
   PE_CHECK_LAUNCH("gae_stream_kernel");
   return PE_OK;
@@ -230,11 +210,17 @@ pe_status gae_launch(const float* r, const float* v, const uint8_t* d, const flo
                                       reinterpret_cast<uintptr_t>(adv) | reinterpret_cast<uintptr_t>(ret) |
                                       reinterpret_cast<uintptr_t>(last_v)) % 8 == 0) &&
                    reinterpret_cast<uintptr_t>(d) % 2 == 0;
-  if (E >= 196608 && al4) return gae_stream_run<4, 8>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (E >= 49152) return gae_stream_run<1, 16>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (E >= 32768) return gae_stream_run<1, 32>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E >= 196608) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E >= 49152) return gae_stream_run<16, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E >= 32768) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (n >= ((int64_t)1 << 28) && al4) return gae_run<4, 8, 4>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (E >= 16384 && al2) return gae_run<4, 16, 2>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  // one CTA of 1,024 threads fills an SM: beyond one per SM, CTAs of 512 (800
+  // steps of 7,766 envs: 32.8 against 41.2 us)
+  int dev = 0, sms = 0;
+  PE_TRY_CUDA(cudaGetDevice(&dev));
+  PE_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  if (E > 32 * sms) return gae_run<8, 16, 1>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   return gae_run<8, 32, 1>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
 }
 
