@@ -29,25 +29,51 @@ constexpr int kTcRows = 128;     // rows (envs / samples) per tile, the MMA M
 constexpr int kTcThreads = 512;  // 16 warps: 4 TMEM lane quadrants x 4 column slices
 constexpr int kHeadN = 16;       // head width (logits or value padded to 16)
 
+// The loss inputs of one sample.  A kernel fetches a row's gather index a
+// tile ahead and the inputs an epilogue ahead: read where they are used, the
+// two dependent global loads were most of the loss's 6,500 cycles, which the
+// backward products of the tile wait for.
+struct LossIn {
+  float adv, logp_old, ret;
+  int act;
+};
+
+__device__ __forceinline__ uint32_t loss_index(const uint32_t* gather, int64_t j, int64_t n) {
+  return j < n ? __ldg(gather + j) : 0u;
+}
+
+__device__ __forceinline__ LossIn loss_inputs(const PpoHead& L, int value_net, uint32_t i) {
+  LossIn in{0.0f, 0.0f, 0.0f, 0};
+  if (value_net) {
+    in.ret = __ldg(L.ret + i);
+  } else {
+    in.adv = __ldg(L.adv + i);
+    in.logp_old = __ldg(L.logp_old + i);
+    in.act = __ldg(L.act + i);
+  }
+  return in;
+}
+
 // Head epilogue of a PPO forward pass for row `row` (0..127) of tile `tile`:
-// z[16] are the head accumulators of the row (before the bias).  Called by
-// all 32 lanes of a head warp (warp < 4); rows past n contribute zero.  The
-// dz row goes to the tile image and, when dz_smem is given, to the same
-// place of a shared-memory copy of the tile.
-__device__ __forceinline__ void ppo_head_row(const PpoHead& L, int value_net, int A, const float* b3,
-                                             const uint32_t* gather, int64_t tile, int row, int64_t n,
-                                             const float (&acc)[16], int warp, uint8_t* dz_smem = nullptr) {
+// acc[16] are the head accumulators of the row (before the bias), `in` its
+// loss inputs.  Called by all 32 lanes of a head warp (warp < 4); rows past n
+// contribute zero.  The dz row goes to the tile image and, when dz_smem is
+// given, to the same place of a shared-memory copy of the tile.
+__device__ __forceinline__ void ppo_head_row(const PpoHead& L, int value_net, int A, const float* b3, const LossIn& in,
+                                             int64_t tile, int row, int64_t n, const float (&acc)[16], int warp,
+                                             uint8_t* dz_smem = nullptr) {
   constexpr int kW = 32;
-  const int64_t j = tile * kTcRows + row;
-  const bool valid = j < n;
-  float v[22];
-#pragma unroll
-  for (int k = 0; k < 22; ++k) v[k] = 0.0f;
+  const int lane = threadIdx.x & 31;
+  const bool valid = tile * kTcRows + row < n;
   uint32_t pk[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (valid) {
-    const uint32_t i = gather[j];
-    if (!value_net) {
-      const float2 as = *L.advstat;
+  float* const pr = L.part + (tile * 4 + warp) * kW;
+  if (!value_net) {
+    // pg loss, entropy, approximate KL, clip indicator, then dLoss/dlogits
+    float v[4 + kHeadN];
+#pragma unroll
+    for (int k = 0; k < 4 + kHeadN; ++k) v[k] = 0.0f;
+    if (valid) {
+      const float2 as = __ldg(L.advstat);
       float z[kHeadN];
 #pragma unroll
       for (int a = 0; a < kHeadN; ++a) z[a] = a < A ? acc[a] + b3[a] : -INFINITY;
@@ -58,20 +84,19 @@ __device__ __forceinline__ void ppo_head_row(const PpoHead& L, int value_net, in
 #pragma unroll
       for (int a = 0; a < kHeadN; ++a) se += a < A ? expf(z[a] - m) : 0.0f;
       const float lse = m + logf(se);
-      float lp[kHeadN], pr[kHeadN], Hs = 0.0f;
+      float lp[kHeadN], p[kHeadN], Hs = 0.0f;
 #pragma unroll
       for (int a = 0; a < kHeadN; ++a) {
         lp[a] = a < A ? z[a] - lse : 0.0f;
-        pr[a] = a < A ? expf(lp[a]) : 0.0f;
-        Hs -= pr[a] * lp[a];
+        p[a] = a < A ? expf(lp[a]) : 0.0f;
+        Hs -= p[a] * lp[a];
       }
-      const int act = L.act[i];
-      const float an = (L.adv[i] - as.x) * as.y;
+      const float an = (in.adv - as.x) * as.y;
       float lpa = 0.0f;
 #pragma unroll
       for (int a = 0; a < kHeadN; ++a)
-        if (a == act) lpa = lp[a];
-      const float logr = lpa - L.logp_old[i];
+        if (a == in.act) lpa = lp[a];
+      const float logr = lpa - in.logp_old;
       const float rho = expf(logr);
       const float rc = fminf(fmaxf(rho, 1.0f - L.clip), 1.0f + L.clip);
       const float s1 = rho * an, s2 = rc * an;
@@ -83,46 +108,61 @@ __device__ __forceinline__ void ppo_head_row(const PpoHead& L, int value_net, in
 #pragma unroll
       for (int a = 0; a < kHeadN; a += 2) {
         float d0 = 0.0f, d1 = 0.0f;
-        if (a < A) d0 = dlp * ((a == act ? 1.0f : 0.0f) - pr[a]) + L.ent_coef * L.inv_cnt * pr[a] * (lp[a] + Hs);
+        if (a < A) d0 = dlp * ((a == in.act ? 1.0f : 0.0f) - p[a]) + L.ent_coef * L.inv_cnt * p[a] * (lp[a] + Hs);
         if (a + 1 < A)
-          d1 = dlp * ((a + 1 == act ? 1.0f : 0.0f) - pr[a + 1]) + L.ent_coef * L.inv_cnt * pr[a + 1] * (lp[a + 1] + Hs);
-        v[5 + a] = d0;
-        v[5 + a + 1] = d1;
+          d1 = dlp * ((a + 1 == in.act ? 1.0f : 0.0f) - p[a + 1]) + L.ent_coef * L.inv_cnt * p[a + 1] * (lp[a + 1] + Hs);
+        v[4 + a] = d0;
+        v[5 + a] = d1;
         pk[a / 2] = tc::pack_bf16(d0, d1);
       }
-    } else {
-      const float V = acc[0] + b3[0], R = L.ret[i];
-      v[4] = (R - V) * (R - V);
-      const float dV = L.vf_coef * 2.0f * (V - R) * L.inv_cnt;
-      v[21] = dV;
+    }
+    // This warp's partial row: the fixed xor tree over the lanes (16, 8, 4, 2,
+    // 1), of all values at once -- at each step a lane passes on the half of
+    // its values that its partner keeps, and lane k ends with value k.  The
+    // sums are those of a tree per value (31 shuffles in place of 100).
+    float w[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const bool two = k + 16 < 4 + kHeadN;
+      const float hi = two ? v[two ? k + 16 : 0] : 0.0f;
+      const float mine = (lane & 16) ? hi : v[k], theirs = (lane & 16) ? v[k] : hi;
+      w[k] = mine + __shfl_xor_sync(0xffffffffu, theirs, 16);
+    }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) {
+        const float mine = (lane & o) ? w[k + o] : w[k], theirs = (lane & o) ? w[k] : w[k + o];
+        w[k] = mine + __shfl_xor_sync(0xffffffffu, theirs, o);
+      }
+    if (lane < 4 + kHeadN) pr[lane < 4 ? lane : lane + 1] = w[0];
+  } else {
+    float se = 0.0f, dV = 0.0f;
+    if (valid) {
+      const float V = acc[0] + b3[0];
+      se = (in.ret - V) * (in.ret - V);
+      dV = L.vf_coef * 2.0f * (V - in.ret) * L.inv_cnt;
       pk[0] = tc::pack_bf16(dV, 0.0f);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      se += __shfl_xor_sync(0xffffffffu, se, o);
+      dV += __shfl_xor_sync(0xffffffffu, dV, o);
+    }
+    if (lane == 0) {
+      pr[4] = se;
+      pr[21] = dV;
     }
   }
   // dz row (zeros past the minibatch): 16-byte chunk c at (c ^ ((row >> 2) & 1)) * 16
   uint8_t* dzr = L.dz + tile * (int64_t)(kTcRows * 32) + row * 32;
   const int sw = (row >> 2) & 1;
-  *reinterpret_cast<uint4*>(dzr + (sw << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-  *reinterpret_cast<uint4*>(dzr + ((1 ^ sw) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+  const uint4 c0 = make_uint4(pk[0], pk[1], pk[2], pk[3]), c1 = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+  *reinterpret_cast<uint4*>(dzr + (sw << 4)) = c0;
+  *reinterpret_cast<uint4*>(dzr + ((1 ^ sw) << 4)) = c1;
   if (dz_smem) {
-    *reinterpret_cast<uint4*>(dz_smem + row * 32 + (sw << 4)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    *reinterpret_cast<uint4*>(dz_smem + row * 32 + ((1 ^ sw) << 4)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-  }
-  // this warp's partial row
-#pragma unroll
-  for (int k = 0; k < 22; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  if ((threadIdx.x & 31) == 0) {
-    float* pr = L.part + (tile * 4 + warp) * kW;
-    if (!value_net) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) pr[k] = v[k];
-#pragma unroll
-      for (int k = 5; k < 21; ++k) pr[k] = v[k];
-    } else {
-      pr[4] = v[4];
-      pr[21] = v[21];
-    }
+    *reinterpret_cast<uint4*>(dz_smem + row * 32 + (sw << 4)) = c0;
+    *reinterpret_cast<uint4*>(dz_smem + row * 32 + ((1 ^ sw) << 4)) = c1;
   }
 }
 

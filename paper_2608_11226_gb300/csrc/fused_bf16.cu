@@ -338,12 +338,18 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
     // shared dz tile (zeros for a slot without a tile); slot s by the four
     // warps of column slice s (one per TMEM lane quadrant), so that the two
     // slots' losses run side by side
+    LossIn lin{0.0f, 0.0f, 0.0f, 0};
+    auto lindex = [&](int p) -> uint32_t {  // this thread's sample of pair p (slices 0 and 1: one slot each)
+      const int k = 2 * p + slice;
+      return slice < 2 && k < my_tiles ? loss_index(g.save.gather, tile_of(k) * kTcRows + row, g.n) : 0u;
+    };
+    uint32_t lidx = lindex(0);
     auto head_epi = [&](int sl, int k) {
       if (slice != sl) return;
       if (k < my_tiles) {
         float v[16];
         tc::tmem_ld16(lane_base + (uint32_t)(sl * 256), v);
-        ppo_head_row(g.save.loss, g.value_net, g.A, s.b3, g.save.gather, tile_of(k), row, g.n, v, quad, s.dz[sl]);
+        ppo_head_row(g.save.loss, g.value_net, g.A, s.b3, lin, tile_of(k), row, g.n, v, quad, s.dz[sl]);
       } else {
         *reinterpret_cast<uint4*>(s.dz[sl] + row * 32) = make_uint4(0, 0, 0, 0);
         *reinterpret_cast<uint4*>(s.dz[sl] + row * 32 + 16) = make_uint4(0, 0, 0, 0);
@@ -388,6 +394,11 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
         tc::fence_after();
         hidden(sl, s.b1);
         handover(&s.h1in[sl]);
+      }
+      // the loss inputs, in flight during layer 2, and the next pair's index
+      if (slice < 2) {
+        lin = loss_inputs(g.save.loss, g.value_net, lidx);
+        lidx = lindex(p + 1);
       }
       for (int sl = 0; sl < 2; ++sl) {
         (void)wt(&s.mma2[sl], par);

@@ -394,14 +394,28 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     auto wait_stored = [&](uint64_t* done, int q) {
       if (saving) (void)wt(done, q);  // two completions per tile: the first has parity 0
     };
+    // the loss inputs of the row's sample (warps 0-3): its index a tile ahead
+    const bool losing = save.loss.dz != nullptr && warp < 4;
+    uint32_t lidx = 0;
+    LossIn lin{0.0f, 0.0f, 0.0f, 0};
+    auto lindex = [&](int k) -> uint32_t {
+      int ni;
+      const int64_t tl = tile_of(k, ni);
+      return loss_index(ni ? second.save.gather : save.gather, tl * kTcRows + row, n);
+    };
+    auto linputs = [&](int k) {
+      int ni;
+      (void)tile_of(k, ni);
+      lin = ni ? loss_inputs(second.save.loss, 1, lidx) : loss_inputs(save.loss, value_net, lidx);
+    };
     // head of this CTA's k-th tile from its 16 accumulators (warps 0-3, one row per thread)
     auto head_out = [&](int k, const float (&v)[16]) {
       int ni;
       const int64_t tl = tile_of(k, ni);
       if (ni) {
-        ppo_head_row(second.save.loss, 1, A, s.b3[1], second.save.gather, tl, row, n, v, warp);
+        ppo_head_row(second.save.loss, 1, A, s.b3[1], lin, tl, row, n, v, warp);
       } else if (save.loss.dz) {
-        ppo_head_row(save.loss, value_net, A, s.b3[0], save.gather, tl, row, n, v, warp);
+        ppo_head_row(save.loss, value_net, A, s.b3[0], lin, tl, row, n, v, warp);
       } else if (tl * kTcRows + row < n) {
         float* o = out + (tl * kTcRows + row) * out_stride;
 #pragma unroll
@@ -462,6 +476,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         put(c, pk);
       }
       handover(&s.h1a);
+      if (losing) {  // the previous tile's inputs, in flight during half B; this tile's index
+        if (t > 0) linputs(t - 1);
+        lidx = lindex(t);
+      }
       (void)wt(&s.m1b, par);
       tc::fence_after();
 #pragma unroll 1
@@ -521,6 +539,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     }
     // the last tile's head
     if (warp < 4 && my_tiles > 0) {
+      if (losing) linputs(my_tiles - 1);
       (void)wt(&s.mh, (my_tiles - 1) & 1);
       tc::fence_after();
       float v[16];
@@ -583,8 +602,7 @@ template <int D, int H>
 __global__ void __launch_bounds__(kPairThreads, 1)
     mlp_bf16_pair_kernel(const uint8_t* __restrict__ img, const float* __restrict__ params, int A,
                          int value_net, const __nv_bfloat16* __restrict__ obs, int64_t n,
-                         float* __restrict__ out, int out_stride, int nout, int32_t* __restrict__ err,
-                         MlpSave save) {
+                         float* __restrict__ out, int out_stride, int nout, int32_t* __restrict__ err) {
   using I = Img<D, H>;
   static_assert(H == 256, "two tiles in flight need 2 x 256 TMEM columns");
   constexpr int KB2 = H / 64;   // W2 stages per tile
@@ -710,8 +728,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         const int64_t rr = tl * kTcRows + r;
         dst[q] = make_uint4(0, 0, 0, 0);
         if (k < my_tiles && rr < n) {
-          const int64_t src = save.gather ? (int64_t)__ldg(save.gather + rr) : rr;
-          dst[q] = __ldg(reinterpret_cast<const uint4*>(obs + src * D) + c);
+          dst[q] = __ldg(reinterpret_cast<const uint4*>(obs + rr * D) + c);
         }
       }
     };
@@ -722,9 +739,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         const int nr = (int)(n - tl * kTcRows < kTcRows ? n - tl * kTcRows : kTcRows);
         float v[16];
         tc::tmem_ld16(lane_base + (uint32_t)(sl * 256), v);
-        if (save.loss.dz) {
-          ppo_head_row(save.loss, value_net, A, s.b3, save.gather, tl, row, n, v, warp);
-        } else if (row < nr) {
+        if (row < nr) {
           float* o = out + (tl * kTcRows + row) * out_stride;
 #pragma unroll
           for (int j = 0; j < kHeadN; ++j)
@@ -732,11 +747,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         }
       }
     };
-    // hidden layer epilogue of slot sl: tanh(acc + bias) -> bf16 -> act[sl] (+ the tile image)
-    auto hidden = [&](int sl, const float* bias, __nv_bfloat16* gsave, int k) {
-      const int64_t tl = blockIdx.x + (int64_t)k * gridDim.x;
-      uint8_t* g = (gsave && k < my_tiles) ? reinterpret_cast<uint8_t*>(gsave) + tl * (int64_t)(kTcRows * H * 2)
-                                           : nullptr;
+    // hidden layer epilogue of slot sl: tanh(acc + bias) -> bf16 -> act[sl]
+    auto hidden = [&](int sl, const float* bias) {
 #pragma unroll
       for (int j = 0; j < H / 64; ++j) {
         const int c = slice * (H / 4) + j * 16;
@@ -745,13 +757,8 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         uint32_t pk[8];
         tc::tanh16_bf16(v, bias + c, pk);
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
-        const uint4 lo = make_uint4(pk[0], pk[1], pk[2], pk[3]), hi = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        *reinterpret_cast<uint4*>(s.act[sl] + o0) = lo;
-        *reinterpret_cast<uint4*>(s.act[sl] + o1) = hi;
-        if (g) {
-          *reinterpret_cast<uint4*>(g + o0) = lo;
-          *reinterpret_cast<uint4*>(g + o1) = hi;
-        }
+        *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
       }
     };
     auto handover = [&](uint64_t* bar) {
@@ -773,15 +780,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
           tc::fence_after();
           head_out(sl, k - 2);
         }
-        const int64_t tl = blockIdx.x + (int64_t)k * gridDim.x;
 #pragma unroll
         for (int q = 0; q < XCH; ++q) {
           const int i = tid + q * kTcThreads, r = i / CPR, c = i % CPR;
-          const uint32_t off = tc::swz_offset<I::RB1>(r, c * 8, kTcRows);
-          *reinterpret_cast<uint4*>(s.act[sl] + off) = xv[sl][q];
-          if (save.x && k < my_tiles)
-            *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(save.x) + tl * (int64_t)(kTcRows * D * 2) + off) =
-                xv[sl][q];
+          *reinterpret_cast<uint4*>(s.act[sl] + tc::swz_offset<I::RB1>(r, c * 8, kTcRows)) = xv[sl][q];
         }
         handover(&s.xin[sl]);
       }
@@ -790,13 +792,13 @@ __global__ void __launch_bounds__(kPairThreads, 1)
       for (int sl = 0; sl < 2; ++sl) {
         if (!tc::mbar_wait(&s.mma1[sl], par)) atomicExch(&s.err, 1);
         tc::fence_after();
-        hidden(sl, s.b1, save.h1, 2 * p + sl);
+        hidden(sl, s.b1);
         handover(&s.h1in[sl]);
       }
       for (int sl = 0; sl < 2; ++sl) {
         if (!tc::mbar_wait(&s.mma2[sl], par)) atomicExch(&s.err, 1);
         tc::fence_after();
-        hidden(sl, s.b2, save.h2, 2 * p + sl);
+        hidden(sl, s.b2);
         handover(&s.h2in[sl]);
       }
     }
@@ -963,13 +965,13 @@ static pe_status launch_mlp(const uint8_t* img, const float* params, int A, int 
     kern<<<grid, kStreamThreads, bytes, st>>>(img, params, A, value_net, o, n, out, out_stride, nout, err, save,
                                               second);
   } else {
-    if (second.img) return fail(PE_EINVAL, "two-network forward launches are for the streamed network");
+    if (second.img || save.loss.dz) return fail(PE_EINVAL, "PPO forward launches are for the streamed network");
     auto kern = mlp_bf16_pair_kernel<D, H>;
     const int bytes = (int)sizeof(MlpPairSmem<D, H>) + 1024;
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     const int pgrid = (int)std::min<int64_t>((tiles + 1) / 2, sms);
     ProfScope ps(prof_kind, st);
-    kern<<<pgrid, kPairThreads, bytes, st>>>(img, params, A, value_net, o, n, out, out_stride, nout, err, save);
+    kern<<<pgrid, kPairThreads, bytes, st>>>(img, params, A, value_net, o, n, out, out_stride, nout, err);
   }
   PE_CHECK_LAUNCH("bf16 MLP kernel");
   return PE_OK;
@@ -1139,23 +1141,17 @@ pe_status bf16_make_images(const pe_net& net, const float* params, uint8_t* two_
 }
 
 // forward of both networks over the same gathered minibatch rows with the PPO
-// loss in the head: the policy (image at img, loss lp, saving x, h[0], h[1])
-// and the value network (image at img + bf16_image_bytes, loss lv, saving
-// h[2], h[3]).  The streamed network runs both in one launch, its tiles
-// spread over the persistent CTAs together.
+// loss in the head, for the streamed (Stress) network: the policy (image at
+// img, loss lp, saving x, h[0], h[1]) and the value network (image at img +
+// bf16_image_bytes, loss lv, saving h[2], h[3]) in one launch, their tiles
+// spread over the persistent CTAs together.  (The 72B networks' forward is part
+// of ppo_fused_pair_kernel.)
 pe_status bf16_forward_loss(const pe_net& net, const uint8_t* img, const float* params, const void* obs,
                             const uint32_t* gather, int64_t n, const PpoHead& lp, const PpoHead& lv,
                             __nv_bfloat16* x, __nv_bfloat16* const h[4], int32_t* err, cudaStream_t st) {
   const MlpSave sp{gather, x, h[0], h[1], lp};
   const MlpSave sv{gather, nullptr, h[2], h[3], lv};
   float* out = nullptr;
-  if (net.obs_dim == 32 && net.hidden == 256) {
-    const uint8_t* img_v = img + NetKind<32, 256>::kImgPad;
-    pe_status s = launch_mlp<32, 256>(img, params, net.n_actions, 0, obs, n, out, 0, net.n_actions, err, st,
-                                      PE_PROF_PPO_GRAD, sp);
-    if (s != PE_OK) return s;
-    return launch_mlp<32, 256>(img_v, params, net.n_actions, 1, obs, n, out, 0, 1, err, st, PE_PROF_PPO_GRAD, sv);
-  }
   if (net.obs_dim == 64 && net.hidden == 512)
     return launch_mlp<64, 512>(img, params, net.n_actions, 0, obs, n, out, 0, net.n_actions, err, st,
                                PE_PROF_PPO_GRAD, sp, MlpSecond{img + NetKind<64, 512>::kImgPad, sv});
