@@ -87,12 +87,13 @@ __global__ void weight_image_kernel(const float* __restrict__ params, int A, int
 //   epilogue 2, half A (N-half 0) runs during the N-half 1 MMAs; its first
 //   results wait in registers until the N-half 1 MMAs have read h1's first
 //   four K-blocks, which h2 overwrites in place;
-//   the head accumulates in TMEM columns 256-271, so the next tile's layer-1
-//   N-half 0 can start while warps 0-3 copy the head accumulators to shared
-//   memory (they compute the loss later, during the next tile's layer-2
-//   N-half 0 MMAs) and warps 4-15 write the next tile's X (its rows fetched
-//   during the previous epilogue) into the buffer's last K-block, which only
-//   epilogue 1, half B overwrites.
+//   the next tile's X has its own buffer (written after epilogue 1), so its
+//   layer-1 N-half 0 runs during epilogue 2, half B; the head accumulates in
+//   TMEM columns 256-271 while epilogue 1, half A of the next tile computes its
+//   first results into registers (h1 overwrites the h2 that the head reads);
+//   warps 0-3 copy the head accumulators to shared memory before layer-1
+//   N-half 1 takes their columns, and compute the loss later, during the
+//   layer-2 N-half 0 MMAs.
 // The accumulation order of every accumulator is that of the serial kernel,
 // so the results are the same bits.  One launch may also cover two networks
 // over the same rows (the policy, then the value network of a PPO forward):
@@ -138,7 +139,8 @@ __global__ void weight_image_stream_kernel(const float* __restrict__ params, int
 
 template <int D, int H>
 struct MlpStreamSmem {
-  alignas(1024) uint8_t act[kTcRows * H * 2];  // X (last K-block), then h1, then h2 (in place)
+  alignas(1024) uint8_t act[kTcRows * H * 2];  // h1, then h2 (in place)
+  alignas(1024) uint8_t x[kTcRows * D * 2];
   alignas(1024) uint8_t ring[2][kStageBytes];
   float headv[kTcRows][kHeadN];                // the previous tile's head accumulators (warps 0-3)
   float b1[2][H], b2[2][H], b3[2][kHeadN];     // per network of the launch
@@ -161,9 +163,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
                            MlpSave save, MlpSecond second) {
   using I = ImgS<D, H>;
   static_assert(D == 64 && H == 512, "two 256-column halves per layer; X is one 128-byte K-block");
+  static_assert(sizeof(MlpStreamSmem<D, H>) + 1024 <= 232448, "stream kernel shared memory");
   constexpr int NJ = H / 2 / 4 / 16;                 // 16-column chunks per warp and half
   constexpr int KBH = H / 2 / 64;                    // K-blocks of h per half
-  constexpr int kXOff = (H / 64 - 1) * kTcRows * 128;  // X sits in the last K-block of the buffer
   constexpr int XCPR = D / 8;                        // 16-byte observation chunks per row
   constexpr int XCH = (kTcRows * XCPR + 383) / 384;  // per X-writing thread (warps 4-15)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -227,30 +229,35 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   };
   int last_issued = -1;  // producer: global index of its last issued stage
   if (warp == 16) {
-    // producer: every stage of every tile of this CTA, in consumption order
+    // producer: every stage of every tile of this CTA, in consumption order:
+    // W1's first half, the previous tile's head, W1's second half, W2
     if (lane == 0) {
       int gs = 0;
+      auto issue = [&](const uint8_t* timg, int st) -> bool {
+        const int slot = gs & 1;
+        if (gs >= 2 && !wt(&s.empty[slot], ((gs - 2) >> 1) & 1)) return false;
+        tc::mbar_expect_tx(&s.full[slot], (uint32_t)I::stage_bytes(st));
+        tc::bulk_g2s(s.ring[slot], timg + I::stage_off(st), (uint32_t)I::stage_bytes(st), &s.full[slot]);
+        last_issued = gs++;
+        return true;
+      };
+      const uint8_t* prev = nullptr;
       bool ok = true;
       for (int t = 0; t < my_tiles && ok; ++t) {
         int ni;
         (void)tile_of(t, ni);
         const uint8_t* timg = ni ? second.img : img;
-        for (int st = 0; st < kStreamStages && ok; ++st) {
-          const int slot = gs & 1;
-          if (gs >= 2 && !wt(&s.empty[slot], ((gs - 2) >> 1) & 1)) {
-            ok = false;
-            break;
-          }
-          tc::mbar_expect_tx(&s.full[slot], (uint32_t)I::stage_bytes(st));
-          tc::bulk_g2s(s.ring[slot], timg + I::stage_off(st), (uint32_t)I::stage_bytes(st), &s.full[slot]);
-          last_issued = gs++;
-        }
+        ok = issue(timg, 0);
+        if (t > 0) ok = ok && issue(prev, kStreamStages - 1);
+        for (int st = 1; st < kStreamStages - 1 && ok; ++st) ok = issue(timg, st);
+        prev = timg;
       }
+      if (ok && my_tiles > 0) (void)issue(prev, kStreamStages - 1);
     }
   } else if (warp == 17) {
     // MMA issuer
     if (lane == 0) {
-      const uint32_t xa = tc::smem_u32(s.act);
+      const uint32_t xa = tc::smem_u32(s.act), xb = tc::smem_u32(s.x);
       constexpr uint32_t kIdN = tc::idesc_bf16(kTcRows, 256);
       constexpr uint32_t kIdH = tc::idesc_bf16(kTcRows, kHeadN);
       int gs = 0;
@@ -276,37 +283,18 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
           stage_out();
         }
       };
-      for (int t = 0; t < my_tiles; ++t) {
-        const uint32_t par = t & 1;
-        (void)wt(&s.xin, par);
-        tc::fence_after();
-        // layer 1, N-half h; N-half 1 overwrites the columns of the previous tile's head
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          if (h == 1 && t > 0) {
-            (void)wt(&s.hd, par ^ 1);
-            tc::fence_after();
-          }
-          const uint32_t ra = stage_in();
+      // layer 1, N-half h
+      auto layer1 = [&](int h) {
+        const uint32_t ra = stage_in();
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk)
-            tc::mma_bf16(tmem + h * 256, tc::desc_kmajor(xa + kXOff + kk * 32, 1024, tc::kLayoutSW128),
-                         tc::desc_kmajor(ra + kk * 32, 1024, tc::kLayoutSW128), kIdN, kk > 0);
-          stage_out();
-          tc::mma_commit(h ? &s.m1b : &s.m1a);
-        }
-        (void)wt(&s.h1a, par);
-        tc::fence_after();
-        layer2(0, 0, KBH);
-        (void)wt(&s.h1b, par);
-        tc::fence_after();
-        layer2(0, KBH, 2 * KBH);
-        tc::mma_commit(&s.m2a);
-        layer2(1, 0, KBH);
-        tc::mma_commit(&s.n1lo);
-        layer2(1, KBH, 2 * KBH);
-        tc::mma_commit(&s.m2b);
-        // head: TMEM columns 256 .. 271 = H2 W3^T (one 16 KB stage)
+        for (int kk = 0; kk < D / 16; ++kk)
+          tc::mma_bf16(tmem + h * 256, tc::desc_kmajor(xb + kk * 32, 1024, tc::kLayoutSW128),
+                       tc::desc_kmajor(ra + kk * 32, 1024, tc::kLayoutSW128), kIdN, kk > 0);
+        stage_out();
+        tc::mma_commit(h ? &s.m1b : &s.m1a);
+      };
+      // head: TMEM columns 256 .. 271 = H2 W3^T (one 16 KB stage), once h2 is written
+      auto head = [&](uint32_t par) {
         (void)wt(&s.h2in, par);
         tc::fence_after();
         const uint32_t ra = stage_in();
@@ -319,7 +307,34 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
                          (kb | kk) != 0);
         stage_out();
         tc::mma_commit(&s.mh);
+      };
+      for (int t = 0; t < my_tiles; ++t) {
+        const uint32_t par = t & 1;
+        // N-half 0's columns: the previous tile's epilogue 2, half A has read them
+        (void)wt(&s.xin, par);
+        if (t > 0) (void)wt(&s.h2a, par ^ 1);
+        tc::fence_after();
+        layer1(0);
+        // N-half 1's: the previous tile's head, once its accumulators are out
+        if (t > 0) {
+          head(par ^ 1);
+          (void)wt(&s.hd, par ^ 1);
+          tc::fence_after();
+        }
+        layer1(1);
+        (void)wt(&s.h1a, par);
+        tc::fence_after();
+        layer2(0, 0, KBH);
+        (void)wt(&s.h1b, par);
+        tc::fence_after();
+        layer2(0, KBH, 2 * KBH);
+        tc::mma_commit(&s.m2a);
+        layer2(1, 0, KBH);
+        tc::mma_commit(&s.n1lo);
+        layer2(1, KBH, 2 * KBH);
+        tc::mma_commit(&s.m2b);
       }
+      if (my_tiles > 0) head((my_tiles - 1) & 1);
       // every MMA of this CTA completes before TMEM is released
       tc::mma_commit(&s.fin);
       if (!tc::mbar_wait(&s.fin, 0)) atomicExch(&s.err, 1);
@@ -423,64 +438,79 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
           if (j < nout) o[j] = v[j] + s.b3[0][j];
       }
     };
-    if (warp >= 4) fetch_x(0);
+    // X of this CTA's k-th tile from the registers fetch_x(k) filled (warps 4-15)
+    auto put_x = [&](int k) {
+      int ni;
+      const int64_t tl = tile_of(k, ni);
+      __nv_bfloat16* const sx = ni ? second.save.x : save.x;
+#pragma unroll
+      for (int q = 0; q < XCH; ++q) {
+        const int i = xt + q * 384;
+        if (i < kTcRows * XCPR) {
+          const uint32_t off = tc::swz_offset<128>(i / XCPR, i % XCPR * 8, kTcRows);
+          *reinterpret_cast<uint4*>(s.x + off) = xv[q];
+          if (sx)
+            *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(sx) + tl * (int64_t)(kTcRows * D * 2) + off) = xv[q];
+        }
+      }
+      handover(&s.xin);
+    };
+    if (warp >= 4 && my_tiles > 0) {
+      fetch_x(0);
+      put_x(0);
+    }
     for (int t = 0; t < my_tiles; ++t) {
       const uint32_t par = t & 1;
       int ni;
-      const int64_t tile = tile_of(t, ni);
-      __nv_bfloat16* const sx = ni ? second.save.x : save.x;
+      (void)tile_of(t, ni);
       const float* const b1 = s.b1[ni];
       const float* const b2 = s.b2[ni];
-      if (t > 0) (void)wt(&s.mh, par ^ 1);  // the previous tile's head is done
-      tc::fence_after();
-      if (warp < 4) {
-        // its accumulators out of TMEM (the loss comes later, while the
-        // layer-2 MMAs run), so that layer 1 may take the columns
-        if (t > 0) {
-          float v[16];
-          tc::tmem_ld16(lane_addr + 256u, v);
-#pragma unroll
-          for (int j = 0; j < kHeadN; j += 4)
-            *reinterpret_cast<float4*>(&s.headv[row][j]) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-          tc::fence_before();
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&s.hd);
-        }
-      } else {
-        // this tile's X (the previous tile's head MMA and the storer have read h2)
-        if (t > 0) wait_stored(&s.sb, 1);
-#pragma unroll
-        for (int q = 0; q < XCH; ++q) {
-          const int i = xt + q * 384;
-          if (i < kTcRows * XCPR) {
-            const int r = i / XCPR, c = i % XCPR;
-            const uint32_t off = tc::swz_offset<128>(r, c * 8, kTcRows);
-            *reinterpret_cast<uint4*>(s.act + kXOff + off) = xv[q];
-            if (sx)
-              *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(sx) + tile * (int64_t)(kTcRows * D * 2) + off) =
-                  xv[q];
-          }
-        }
-        handover(&s.xin);
-      }
-      // epilogue 1, half A (h1 K-blocks 0-3), then half B (K-blocks 4-7, the
-      // last of which held X: layer-1 N-half 1 is done by then)
+      // epilogue 1, half A (h1 K-blocks 0-3): the first two chunks wait in
+      // registers until the previous tile's head MMA (and the storer) have
+      // read its h2
       (void)wt(&s.m1a, par);
-      if (t > 0) wait_stored(&s.sa, 1);
       tc::fence_after();
+      {
+        const int c0 = slice * (H / 8);
+        uint32_t p0[8], p1[8];
+        chunk(c0, b1, p0);
+        chunk(c0 + 16, b1, p1);
+        if (t > 0) {
+          (void)wt(&s.mh, par ^ 1);
+          tc::fence_after();
+          if (warp < 4) {
+            // its accumulators out of TMEM (the loss comes later, while the
+            // layer-2 MMAs run), so that layer 1 may take the columns
+            float v[16];
+            tc::tmem_ld16(lane_addr + 256u, v);
+#pragma unroll
+            for (int j = 0; j < kHeadN; j += 4)
+              *reinterpret_cast<float4*>(&s.headv[row][j]) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&s.hd);
+          }
+          wait_stored(&s.sa, 1);
+        }
+        put(c0, p0);
+        put(c0 + 16, p1);
 #pragma unroll 1
-      for (int j = 0; j < NJ; ++j) {
-        const int c = slice * (H / 8) + j * 16;
-        uint32_t pk[8];
-        chunk(c, b1, pk);
-        put(c, pk);
+        for (int j = 2; j < NJ; ++j) {
+          const int c = c0 + j * 16;
+          uint32_t pk[8];
+          chunk(c, b1, pk);
+          put(c, pk);
+        }
       }
       handover(&s.h1a);
       if (losing) {  // the previous tile's inputs, in flight during half B; this tile's index
         if (t > 0) linputs(t - 1);
         lidx = lindex(t);
       }
+      if (warp >= 4) fetch_x(t + 1);
+      // epilogue 1, half B (K-blocks 4-7)
       (void)wt(&s.m1b, par);
+      if (t > 0) wait_stored(&s.sb, 1);
       tc::fence_after();
 #pragma unroll 1
       for (int j = 0; j < NJ; ++j) {
@@ -490,6 +520,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         put(c, pk);
       }
       handover(&s.h1b);
+      // the next tile's X (both halves of this tile's layer 1 are done)
+      if (warp >= 4 && t + 1 < my_tiles) put_x(t + 1);
       // the previous tile's head epilogue, while the rest of layer-2 N-half 0 runs
       if (warp < 4 && t > 0) {
         float v[16];
@@ -534,8 +566,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         put(c, pk);
       }
       handover(&s.h2in);
-      // the next tile's observation rows, fetched while its X slot waits for this tile's head MMA
-      if (warp >= 4) fetch_x(t + 1);
     }
     // the last tile's head
     if (warp < 4 && my_tiles > 0) {
