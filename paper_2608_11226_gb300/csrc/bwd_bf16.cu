@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
     if (lane == 0) {
       int gs = 0;
       bool ok = true;
+      const uint64_t keep = tc::l2_keep();
       for (int t = 0; t < my_tiles && ok; ++t) {
         int ni;
         (void)tile_of(t, ni);
@@ -204,7 +205,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
             break;
           }
           tc::mbar_expect_tx(&s.full[slot], (uint32_t)kBwStage);
-          tc::bulk_g2s(s.ring[slot], img + I::W3T + (int64_t)st * kBwStage, (uint32_t)kBwStage, &s.full[slot]);
+          tc::bulk_g2s(s.ring[slot], img + I::W3T + (int64_t)st * kBwStage, (uint32_t)kBwStage, &s.full[slot], keep);
           last_issued = gs++;
         }
       }
@@ -319,9 +320,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
       auto store = [&](uint64_t* ready, uint32_t par, uint64_t* done, uint8_t* img, int half) {
         ok = ok && wt(ready, par);
         if (!ok) return;
-        tc::bulk_s2g(img + half * kHalfBytes, s.da2 + half * kHalfBytes, (uint32_t)kHalfBytes);
-        tc::bulk_commit();
-        tc::bulk_wait_read();
+        tc::store_image(img + half * kHalfBytes, s.da2 + half * kHalfBytes, (uint32_t)kHalfBytes);
         tc::mbar_arrive(done);
       };
       for (int t = 0; t < my_tiles && ok; ++t) {

@@ -137,11 +137,12 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
     // the W2^T stages of slot 0 and of slot 1, in the issuer's order
     if (lane == 0) {
       int gs = 0;
+      const uint64_t keep = tc::l2_keep();
       auto issue = [&](const uint8_t* src, uint32_t bytes) -> bool {
         const int slot = gs & 1;
         if (gs >= 2 && !wt(&s.empty[slot], ((gs - 2) >> 1) & 1)) return false;
         tc::mbar_expect_tx(&s.full[slot], bytes);
-        tc::bulk_g2s(s.ring[slot], src, bytes, &s.full[slot]);
+        tc::bulk_g2s(s.ring[slot], src, bytes, &s.full[slot], keep);
         last_issued = gs++;
         return true;
       };
@@ -263,10 +264,8 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
           if (!ok) return;
           const int k = 2 * p + sl;
           if (k < my_tiles) {
-            tc::bulk_s2g(reinterpret_cast<uint8_t*>(img) + tile_of(k) * (int64_t)kTile, s.act[sl], (uint32_t)kTile);
-            tc::bulk_commit();
+            tc::store_image(reinterpret_cast<uint8_t*>(img) + tile_of(k) * (int64_t)kTile, s.act[sl], (uint32_t)kTile);
             if (full) tc::bulk_wait();
-            else tc::bulk_wait_read();
           }
           tc::mbar_arrive(&s.stored[sl]);
         };

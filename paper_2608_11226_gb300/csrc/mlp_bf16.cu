@@ -233,11 +233,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     // W1's first half, the previous tile's head, W1's second half, W2
     if (lane == 0) {
       int gs = 0;
+      const uint64_t keep = tc::l2_keep();
       auto issue = [&](const uint8_t* timg, int st) -> bool {
         const int slot = gs & 1;
         if (gs >= 2 && !wt(&s.empty[slot], ((gs - 2) >> 1) & 1)) return false;
         tc::mbar_expect_tx(&s.full[slot], (uint32_t)I::stage_bytes(st));
-        tc::bulk_g2s(s.ring[slot], timg + I::stage_off(st), (uint32_t)I::stage_bytes(st), &s.full[slot]);
+        tc::bulk_g2s(s.ring[slot], timg + I::stage_off(st), (uint32_t)I::stage_bytes(st), &s.full[slot], keep);
         last_issued = gs++;
         return true;
       };
@@ -347,10 +348,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       auto store = [&](uint64_t* ready, uint32_t par, uint64_t* done, __nv_bfloat16* img, int64_t tile, int half) {
         ok = ok && wt(ready, par);
         if (!ok) return;
-        tc::bulk_s2g(reinterpret_cast<uint8_t*>(img) + tile * (int64_t)(2 * kHalf) + half * kHalf,
-                     s.act + half * kHalf, kHalf);
-        tc::bulk_commit();
-        tc::bulk_wait_read();
+        tc::store_image(reinterpret_cast<uint8_t*>(img) + tile * (int64_t)(2 * kHalf) + half * kHalf,
+                        s.act + half * kHalf, kHalf);
         tc::mbar_arrive(done);
       };
       for (int t = 0; t < my_tiles && ok; ++t) {

@@ -197,6 +197,23 @@ __device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, u
       : "memory");
 }
 
+// an L2 policy that keeps the lines of a copy: for weights that every CTA
+// re-reads while the tile images stream past them
+__device__ __forceinline__ uint64_t l2_keep() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+
+__device__ __forceinline__ void bulk_g2s(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* mbar,
+                                         uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+          smem_u32(dst_smem)),
+      "l"(src_gmem), "r"(bytes), "r"(smem_u32(mbar)), "l"(policy)
+      : "memory");
+}
+
 // bulk copy shared -> global (16-byte aligned, a multiple of 16 bytes), in the
 // issuing thread's current bulk group
 __device__ __forceinline__ void bulk_s2g(void* dst_gmem, const void* src_smem, uint32_t bytes) {
@@ -209,6 +226,17 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // ... and have been written
 __device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// a tile image (bytes, a multiple of 16 KB) from shared to global memory, 16 KB
+// at a time, each read before the next is queued: a weight stage's copy then
+// waits behind 16 KB of image at most
+__device__ __forceinline__ void store_image(uint8_t* dst_gmem, const uint8_t* src_smem, uint32_t bytes) {
+  for (uint32_t o = 0; o < bytes; o += 16384) {
+    bulk_s2g(dst_gmem + o, src_smem + o, 16384);
+    bulk_commit();
+    bulk_wait_read();
+  }
+}
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
