@@ -48,7 +48,7 @@ struct FusedSmem {
   alignas(1024) uint8_t w3[Img<D, H>::W3];         // B of the head (K-major SW128)
   alignas(1024) uint8_t w3t[BwdImg<H>::W3T];       // B of dh2 = dz W3 (K-major SW32)
   alignas(1024) uint8_t dz[2][kTcRows * 32];       // A of dh2 per slot (K-major SW32)
-  float b1[H], b2[H], b3[kHeadN];
+  alignas(16) float b1[H], b2[H], b3[kHeadN];
   uint64_t bar_w, fin, full[2], empty[2];
   uint64_t mma1[2], mma2[2], head[2], mdh2[2], mdh1[2];
   uint64_t xin[2], h1in[2], h2in[2], dzin[2], d2in[2], d1in[2], stored[2];
@@ -321,16 +321,16 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
     // hidden layer: tanh(acc + bias) -> bf16 -> act[sl]
     auto hidden = [&](int sl, const float* bias) {
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        const int c = slice * (H / 4) + j * 16;
-        float v[16];
-        tc::tmem_ld16(lane_base + (uint32_t)(sl * 256 + c), v);
-        uint32_t pk[8];
-        tc::tanh16_bf16(v, bias + c, pk);
-        const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
-        const uint4 lo = make_uint4(pk[0], pk[1], pk[2], pk[3]), hi = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-        *reinterpret_cast<uint4*>(s.act[sl] + o0) = lo;
-        *reinterpret_cast<uint4*>(s.act[sl] + o1) = hi;
+      for (int j = 0; j < NJ / 2; ++j) {
+        const int c = slice * (H / 4) + j * 32;
+        float v[32];
+        tc::tmem_ld32(lane_base + (uint32_t)(sl * 256 + c), v);
+        uint32_t pk[16];
+        tc::tanh_bf16(v, bias + c, pk);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          *reinterpret_cast<uint4*>(s.act[sl] + tc::swz_offset<128>(row, c + 8 * q, kTcRows)) =
+              make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
       }
     };
     // head: the PPO loss per row, dz to its tile image and to the slot's
@@ -432,8 +432,10 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
           hv[j][0] = make_uint4(0, 0, 0, 0);
           hv[j][1] = make_uint4(0, 0, 0, 0);
           if (h1t) {
-            hv[j][0] = __ldcg(reinterpret_cast<const uint4*>(h1t + tc::swz_offset<128>(row, c, kTcRows)));
-            hv[j][1] = __ldcg(reinterpret_cast<const uint4*>(h1t + tc::swz_offset<128>(row, c + 8, kTcRows)));
+            // columns c .. c + 15 are one 32-byte sector, its halves swapped in odd rows
+            const uint32_t o = tc::swz_offset<128>(row, c, kTcRows) & ~31u;
+            if (row & 1) tc::ld_global32(h1t + o, hv[j][1], hv[j][0]);
+            else tc::ld_global32(h1t + o, hv[j][0], hv[j][1]);
           }
         }
         (void)wt(&s.mdh1[sl], par);

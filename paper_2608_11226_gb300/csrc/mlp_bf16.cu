@@ -143,7 +143,7 @@ struct MlpStreamSmem {
   alignas(1024) uint8_t x[kTcRows * D * 2];
   alignas(1024) uint8_t ring[2][kStageBytes];
   float headv[kTcRows][kHeadN];                // the previous tile's head accumulators (warps 0-3)
-  float b1[2][H], b2[2][H], b3[2][kHeadN];     // per network of the launch
+  alignas(16) float b1[2][H], b2[2][H], b3[2][kHeadN];  // per network of the launch
   uint64_t full[2], empty[2], fin;
   // one completion per tile each: X written (warps 4-15), head read out of
   // TMEM (warps 0-3), layer-1 N-halves done, h1 halves written, layer-2
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     auto chunk = [&](int c, const float* bias, uint32_t (&pk)[8]) {
       float v[16];
       tc::tmem_ld16(lane_addr + (uint32_t)c, v);
-      tc::tanh16_bf16(v, bias + c, pk);
+      tc::tanh_bf16(v, bias + c, pk);
     };
     // ... into the activation buffer (the next A operand)
     auto put = [&](int c, const uint32_t (&pk)[8]) {
@@ -621,7 +621,7 @@ struct MlpPairSmem {
   alignas(1024) uint8_t ring[2][kPairW2Stage];
   alignas(1024) uint8_t w1[Img<D, H>::W1];
   alignas(1024) uint8_t w3[Img<D, H>::W3];
-  float b1[H], b2[H], b3[kHeadN];
+  alignas(16) float b1[H], b2[H], b3[kHeadN];
   uint64_t bar_w, full[2], empty[2], mma1[2], mma2[2], head[2], xin[2], h1in[2], h2in[2];
   uint32_t tmem_base;
   int32_t err;
@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         float v[16];
         tc::tmem_ld16(lane_base + (uint32_t)(sl * 256 + c), v);
         uint32_t pk[8];
-        tc::tanh16_bf16(v, bias + c, pk);
+        tc::tanh_bf16(v, bias + c, pk);
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
         *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
