@@ -230,6 +230,12 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
         int ni;
         const int64_t tl = tile_of(t, ni);
         const uint8_t* h1 = (ni ? g.h1[1] : g.h1[0]) + tl * (int64_t)kTileBytes;
+        if (t + 1 < my_tiles) {  // the next tile's images, asked of L2 a tile ahead
+          int nn;
+          const int64_t nt = tile_of(t + 1, nn);
+          tc::bulk_prefetch_l2((nn ? g.h2[1] : g.h2[0]) + nt * (int64_t)kTileBytes, (uint32_t)kTileBytes);
+          tc::bulk_prefetch_l2((nn ? g.h1[1] : g.h1[0]) + nt * (int64_t)kTileBytes, (uint32_t)kTileBytes);
+        }
         if (!wt(&s.n1lo, par) || !wt(&s.sa, 0)) break;
         copy(2, &s.h1a, h1, 0);
         if (!wt(&s.m1b, par) || !wt(&s.sb, 0)) break;
@@ -371,15 +377,6 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
       const int64_t ntile = t + 1 < my_tiles ? tile_of(t + 1, nn) : 0;
       const int nr = (int)(g.n - tile * kBwRows < kBwRows ? g.n - tile * kBwRows : kBwRows);
       const bool valid = row < nr;
-      if (t + 1 < my_tiles) {
-        // the next tile's h1/h2 images asked of L2 a tile ahead (128-byte lines)
-        const uint8_t* h2n = (nn ? g.h2[1] : g.h2[0]) + ntile * (int64_t)kTileBytes;
-        const uint8_t* h1n = (nn ? g.h1[1] : g.h1[0]) + ntile * (int64_t)kTileBytes;
-        for (int64_t off = (int64_t)tid * 128; off < (int64_t)kTileBytes; off += (int64_t)kBwCompute * 128) {
-          tc::prefetch_l2(h2n + off);
-          tc::prefetch_l2(h1n + off);
-        }
-      }
       // dz tile (4 KB, already in the SW32 layout; the previous tile's dh2
       // MMAs have read the old one), then the next tile's into registers
       if (tid < kBwRows * 2) {

@@ -174,9 +174,9 @@ __device__ __forceinline__ bool bar_any(int id, int nthreads, bool pred) {
   return r != 0;
 }
 
-// ask L2 to fetch the 128-byte line holding p (no register result, no wait)
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+// ask L2 to fetch `bytes` (a multiple of 16) from p on (16-byte aligned; no wait)
+__device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // ---------------------------------------------------------------- mbarriers
