@@ -846,6 +846,26 @@ def test_ppo_7b_single_step_partitions(n):
     assert_stats(gs, st, n)
 
 
+@pytest.mark.parametrize("n", [4096, 4097, 16400, 70000])
+def test_ppo_advantage_statistics_clusters(n):
+    """The statistics of one minibatch are summed by a cluster of CTAs of 512
+    threads with 16 register values each: one CTA up to 4,096 samples, two
+    above, eight above 16,384, and beyond 65,536 each thread gathers the rest
+    again.  A wrong mean or deviation scales the whole first moment."""
+    wl = W.make_7b(n_envs=1152)
+    params, buf, adv, ret = _ppo_inputs(wl, 64, seed=6)
+    D = wl.net.obs_dim
+    sub = {"obs": buf["obs"].reshape(-1, D)[:n].contiguous(), "act": buf["act"].reshape(-1)[:n].contiguous(),
+           "logp": buf["logp"].reshape(-1)[:n].contiguous()}
+    a_, r_ = adv.reshape(-1)[:n].contiguous(), ret.reshape(-1)[:n].contiguous()
+    ppo = W.PPOSpec(epochs=1, minibatch=n)
+    gp, gm, gv, gs = _run_ppo(wl, ppo, params, sub, a_, r_)
+    P, m, v, t, st = _oracle_ppo(wl, ppo, params, sub, a_, r_)
+    assert t == 1 and gs[7] == 1
+    assert rel_err(gm, m) <= TOL and rel_err(gp, P) <= TOL
+    assert_stats(gs, st, n)
+
+
 # ------------------------------------------------------------------ bf16 PPO
 BF16_TOL = 2e-2
 
@@ -869,8 +889,8 @@ def test_ppo_bf16_single_step(preset, E, T):
 @pytest.mark.parametrize("preset,E,T", [("72b", 320, 128), ("stress", 160, 122)])
 def test_ppo_bf16_several_tiles_per_cta(preset, E, T):
     """One minibatch large enough that the persistent kernels take more than
-    one tile (pair) per CTA: 72B 40,960 samples = 320 tiles over 152 CTAs
-    (the first 16 run two tile pairs, the second half empty); Stress 19,520
+    one tile (pair) per CTA: 72B 40,960 samples = 320 tiles per network over
+    76 CTAs each (four or five tiles, the odd pair half empty); Stress 19,520
     samples = 153 tiles per network, whose forward and backward-data
     launches spread the 306 tiles of both networks over the 152 CTAs (two
     or three each, most CTAs crossing from a policy tile to a value tile).
@@ -883,6 +903,26 @@ def test_ppo_bf16_several_tiles_per_cta(preset, E, T):
     assert t == 1 and gs[7] == 1
     assert bf16_ok(gm, m), (np.abs(gm - m).max() / np.abs(m).max())
     assert_stats(gs, st, T * E, tol=BF16_TOL)
+
+
+@pytest.mark.parametrize("preset,n", [("72b", 60), ("72b", 200), ("stress", 60), ("stress", 330)])
+def test_ppo_bf16_few_chunks(preset, n):
+    """Minibatches of 1 to 6 chunks of 64 samples: the reduction of the 72B
+    weight gradients deals its chunks out to four threads (the last ones have
+    none below four chunks), Stress sums all in one, and the second network
+    column has fewer chunks than the first."""
+    wl = W.make_72b(n_envs=16) if preset == "72b" else W.make_stress(n_envs=16, horizon=32)
+    params, buf, adv, ret = _ppo_inputs(wl, 32, seed=2)
+    D = wl.net.obs_dim
+    sub = {"obs": buf["obs"].reshape(-1, D)[:n].contiguous(), "act": buf["act"].reshape(-1)[:n].contiguous(),
+           "logp": buf["logp"].reshape(-1)[:n].contiguous()}
+    a_, r_ = adv.reshape(-1)[:n].contiguous(), ret.reshape(-1)[:n].contiguous()
+    ppo = W.PPOSpec(epochs=1, minibatch=n, ent_coef=0.01)
+    gp, gm, gv, gs = _run_ppo(wl, ppo, params, sub, a_, r_, iteration=1)
+    P, m, v, t, st = _oracle_ppo(wl, ppo, params, sub, a_, r_, iteration=1)
+    assert t == 1 and gs[7] == 1
+    assert bf16_ok(gm, m), (np.abs(gm - m).max() / np.abs(m).max())
+    assert_stats(gs, st, n, tol=BF16_TOL)
 
 
 @pytest.mark.parametrize("preset,E,mb,clip", [("72b", 64, 1500, 0.2), ("72b", 64, 1500, 0.01),
