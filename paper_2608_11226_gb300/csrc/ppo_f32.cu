@@ -29,6 +29,8 @@
 
 #include <cstddef>
 
+#include <cooperative_groups.h>
+
 #include "mlp_f32.cuh"
 #include "tc.cuh"
 
@@ -59,24 +61,58 @@ __device__ __forceinline__ float block_sum_f(float v, float* red) {
   return t;
 }
 
-// advantage mean and 1/(std + 1e-8) (unbiased std) of every minibatch
-__global__ void ppo_advstats_kernel(const float* __restrict__ adv, int64_t N, int M, int nmb,
-                                    FeistelSet perms, float2* __restrict__ out) {
+// advantage mean and 1/(std + 1e-8) (unbiased std) of every (minibatch, epoch),
+// two passes by a cluster of CTAs each: thread t of CTA r takes the positions
+// t + 512 (r + CL i), the cluster's sums are added in CTA order.  A position
+// costs its permutation (a serial chain of integer operations) and a gather
+// from L2, so the launch is bound by the longest thread: the
+// first kAdvKeep values stay in registers for the second pass, and CL (a power
+// of two up to 8, the portable limit) is the least that gives a thread at most
+// 8 values, as long as that is met.  With one CTA of 1024 per minibatch and
+// both passes gathered, the 32 of a 72B update took 263 us and now 42; the
+// 7B update's went from 80 to 16.
+constexpr int kAdvNT = 512, kAdvKeep = 16;
+__global__ void __launch_bounds__(kAdvNT) ppo_advstats_kernel(const float* __restrict__ adv, int64_t N, int M, int nmb,
+                                                              FeistelSet perms, float2* __restrict__ out) {
+  namespace cg = cooperative_groups;
   __shared__ float red[32];
-  const int mb = blockIdx.x, ep = blockIdx.y;
+  __shared__ float csum[2];
+  const cg::cluster_group cl = cg::this_cluster();
+  const int CL = (int)cl.num_blocks(), r = (int)cl.block_rank();
+  const int mb = blockIdx.x / CL, ep = blockIdx.y;
   const Feistel& f = perms.f[ep];
   const int64_t start = (int64_t)mb * M;
   const int cnt = (int)(N - start < (int64_t)M ? N - start : (int64_t)M);
-  float s = 0.0f;
-  for (int j = threadIdx.x; j < cnt; j += blockDim.x) s += __ldg(adv + feistel_index(f, start + j));
-  const float mean = block_sum_f(s, red) / (float)cnt;
+  const int j0 = r * kAdvNT + threadIdx.x, step = CL * kAdvNT;
+  auto value = [&](int64_t j) { return __ldg(adv + feistel_index(f, start + j)); };
+  auto cluster_sum = [&](float v, int k) -> float {
+    const float b = block_sum_f(v, red);
+    if (CL == 1) return b;
+    if (threadIdx.x == 0) csum[k] = b;
+    cl.sync();
+    float t = 0.0f;
+    for (int q = 0; q < CL; ++q) t += *cl.map_shared_rank(&csum[k], q);
+    return t;
+  };
+  float keep[kAdvKeep], s = 0.0f;
+#pragma unroll
+  for (int i = 0; i < kAdvKeep; ++i) keep[i] = j0 + (int64_t)i * step < cnt ? value(j0 + (int64_t)i * step) : 0.0f;
+#pragma unroll
+  for (int i = 0; i < kAdvKeep; ++i) s += keep[i];
+  for (int64_t j = j0 + (int64_t)kAdvKeep * step; j < cnt; j += step) s += value(j);
+  const float mean = cluster_sum(s, 0) / (float)cnt;
   float q = 0.0f;
-  for (int j = threadIdx.x; j < cnt; j += blockDim.x) {
-    const float a = __ldg(adv + feistel_index(f, start + j)) - mean;
+#pragma unroll
+  for (int i = 0; i < kAdvKeep; ++i) {
+    const float a = keep[i] - mean;
+    if (j0 + (int64_t)i * step < cnt) q = fmaf(a, a, q);
+  }
+  for (int64_t j = j0 + (int64_t)kAdvKeep * step; j < cnt; j += step) {
+    const float a = value(j) - mean;
     q = fmaf(a, a, q);
   }
-  const float ss = block_sum_f(q, red);
-  if (threadIdx.x == 0) {
+  const float ss = cluster_sum(q, 1);
+  if (r == 0 && threadIdx.x == 0) {
     if (cnt > 1) {
       const float sd = sqrtf(ss / (float)(cnt - 1));
       out[ep * nmb + mb] = make_float2(mean, 1.0f / (sd + 1e-8f));
@@ -84,6 +120,7 @@ __global__ void ppo_advstats_kernel(const float* __restrict__ adv, int64_t N, in
       out[ep * nmb + mb] = make_float2(0.0f, 1.0f);  // a 1-sample minibatch is not normalised
     }
   }
+  if (CL > 1) cl.sync();  // the other CTAs have read this one's sum
 }
 
 // Dense-layer register tiles for the sample slices: a thread owns RT
@@ -1054,9 +1091,22 @@ pe_status launch_advstats(const float* adv, int64_t N, int M, int nmb, int epoch
   if (epochs < 1 || epochs > kPpoMaxEpochs) return fail(PE_EINVAL, "epochs must be in [1, %d]", kPpoMaxEpochs);
   FeistelSet perms{};
   for (int ep = 0; ep < epochs; ++ep) perms.f[ep] = make_feistel((uint64_t)N, seed, ep, iteration);
+  const int64_t cnt = std::min<int64_t>(M, N);
+  unsigned cl = 1;
+  while (cl < 8 && (int64_t)cl * kAdvNT * 8 < cnt) cl *= 2;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cl;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3((unsigned)nmb * cl, epochs);
+  lc.blockDim = dim3(kAdvNT);
+  lc.stream = st;
+  lc.attrs = &at;
+  lc.numAttrs = 1;
   {
     ProfScope ps(PE_PROF_PPO_OTHER, st);
-    ppo_advstats_kernel<<<dim3(nmb, epochs), 1024, 0, st>>>(adv, N, M, nmb, perms, out);
+    PE_TRY_CUDA(cudaLaunchKernelEx(&lc, ppo_advstats_kernel, adv, N, M, nmb, perms, out));
   }
   PE_CHECK_LAUNCH("ppo_advstats_kernel");
   return PE_OK;
@@ -1084,11 +1134,9 @@ static pe_status ppo_run(const pe_net& net, float* params, float* m, float* v, i
   PE_TRY_CUDA(cudaMemsetAsync(acc, 0, 8 * sizeof(double) + 16, st));
   FeistelSet perms{};
   for (int ep = 0; ep < cfg.epochs; ++ep) perms.f[ep] = make_feistel((uint64_t)N, cfg.seed, ep, cfg.iteration);
-  {
-    ProfScope ps(PE_PROF_PPO_OTHER, st);
-    ppo_advstats_kernel<<<dim3(pl.nmb, cfg.epochs), 256, 0, st>>>(adv, N, cfg.minibatch, pl.nmb, perms, advstat);
-  }
-  PE_CHECK_LAUNCH("ppo_advstats_kernel");
+  if (const pe_status e = launch_advstats(adv, N, cfg.minibatch, pl.nmb, cfg.epochs, cfg.seed, cfg.iteration, advstat, st);
+      e != PE_OK)
+    return e;
   {
     ProfScope ps(PE_PROF_PPO_OTHER, st);
     PE_TRY_CUDA(cudaMemsetAsync(img, 0, 2 * img_floats(net) * sizeof(float), st));  // zero the w2t padding
