@@ -28,6 +28,8 @@
 // overwrites it waits for that.  (Stored by the epilogue threads, 16 bytes of
 // a 128-byte row each, every warp-wide store touched 32 lines.
 // 72B update of 32 minibatch steps: 8.07 and 7.25 ms.)
+// One launch covers both networks: the even CTAs take the policy's tiles, the
+// odd ones the value's.
 // The loss epilogue of slot s runs on the four warps of column slice s (one
 // per TMEM lane quadrant), so the two slots' losses run side by side.  The
 // last epilogue of a tile reads h1 back from its tile image, from L2.
@@ -56,21 +58,25 @@ struct FusedSmem {
   int32_t err;
 };
 
-struct FusedArgs {
+struct FusedNet {
   const uint8_t* img;    // forward weight image of the network (W1 | W2 | W3)
   const uint8_t* bimg;   // backward weight image (W3^T | W2^T stages)
-  const float* params;
-  int A, value_net;
-  const __nv_bfloat16* obs;
-  int64_t n;             // valid samples (rows gathered through save.gather)
   MlpSave save;          // gather; x (policy only), h1, h2 tile images; the loss (dz images, partial rows)
   uint8_t* da2;          // out: da2 tile images
   uint8_t* da1;          // out: da1 tile images
+};
+
+struct FusedArgs {
+  FusedNet net[2];       // policy, value: the even and the odd CTAs
+  const float* params;
+  int A;
+  const __nv_bfloat16* obs;
+  int64_t n;             // valid samples (rows gathered through save.gather)
   int32_t* err;
 };
 
 template <int D, int H>
-__global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs g) {
+__global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __grid_constant__ FusedArgs args) {
   using I = Img<D, H>;
   using Bw = BwdImg<H>;
   static_assert(H == 256 && Bw::NH == 1 && Bw::KB == 4, "two tiles in flight need 2 x 256 TMEM columns");
@@ -85,8 +91,10 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   FusedSmem<D, H>& s = *reinterpret_cast<FusedSmem<D, H>*>(base);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const MlpLayout Lp = mlp_layout(D, H, g.A);
-  const int nout = g.value_net ? 1 : g.A;
+  const int value_net = blockIdx.x & 1, cta = blockIdx.x >> 1, ctas = gridDim.x >> 1;  // of this network
+  const FusedNet& g = args.net[value_net];
+  const MlpLayout Lp = mlp_layout(D, H, args.A);
+  const int nout = value_net ? 1 : args.A;
   if (tid == 0) {
     s.err = 0;
     tc::mbar_init(&s.bar_w, 1);
@@ -111,16 +119,16 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
   }
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, 512);
   for (int i = tid; i < H; i += blockDim.x) {
-    s.b1[i] = __ldg(g.params + (g.value_net ? Lp.c1 : Lp.b1) + i);
-    s.b2[i] = __ldg(g.params + (g.value_net ? Lp.c2 : Lp.b2) + i);
+    s.b1[i] = __ldg(args.params + (value_net ? Lp.c1 : Lp.b1) + i);
+    s.b2[i] = __ldg(args.params + (value_net ? Lp.c2 : Lp.b2) + i);
   }
-  if (tid < kHeadN) s.b3[tid] = tid < nout ? __ldg(g.params + (g.value_net ? Lp.c3 : Lp.b3) + tid) : 0.0f;
+  if (tid < kHeadN) s.b3[tid] = tid < nout ? __ldg(args.params + (value_net ? Lp.c3 : Lp.b3) + tid) : 0.0f;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = s.tmem_base;
-  const int64_t tiles = (g.n + kTcRows - 1) / kTcRows;
-  const int my_tiles = (int)((tiles - blockIdx.x + gridDim.x - 1) / gridDim.x);
+  const int64_t tiles = (args.n + kTcRows - 1) / kTcRows;
+  const int my_tiles = (int)((tiles - cta + ctas - 1) / ctas);
   const int npairs = (my_tiles + 1) / 2;
   // a bounded wait that is skipped once the CTA has an error (so that a
   // failed CTA does not spend one time-out per remaining hand-over)
@@ -130,7 +138,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
     atomicExch(&s.err, 1);
     return false;
   };
-  auto tile_of = [&](int k) { return (int64_t)blockIdx.x + (int64_t)k * gridDim.x; };
+  auto tile_of = [&](int k) { return (int64_t)cta + (int64_t)k * ctas; };
   int last_issued = -1;
   if (warp == 16) {
     // producer: per tile pair W1, the W2 K-blocks of slot 0 and of slot 1,
@@ -283,7 +291,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
     const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16);
     auto rows_of = [&](int k) {
       if (k >= my_tiles) return 0;
-      const int64_t left = g.n - tile_of(k) * kTcRows;
+      const int64_t left = args.n - tile_of(k) * kTcRows;
       return (int)(left < kTcRows ? left : kTcRows);
     };
     uint4 xv[2][XCH];
@@ -294,9 +302,9 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
         const int i = tid + q * kTcThreads, r = i / CPR, c = i % CPR;
         const int64_t rr = tl * kTcRows + r;
         dst[q] = make_uint4(0, 0, 0, 0);
-        if (k < my_tiles && rr < g.n) {
+        if (k < my_tiles && rr < args.n) {
           const int64_t src = g.save.gather ? (int64_t)__ldg(g.save.gather + rr) : rr;
-          dst[q] = __ldg(reinterpret_cast<const uint4*>(g.obs + src * D) + c);
+          dst[q] = __ldg(reinterpret_cast<const uint4*>(args.obs + src * D) + c);
         }
       }
     };
@@ -340,7 +348,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
     LossIn lin{0.0f, 0.0f, 0.0f, 0};
     auto lindex = [&](int p) -> uint32_t {  // this thread's sample of pair p (slices 0 and 1: one slot each)
       const int k = 2 * p + slice;
-      return slice < 2 && k < my_tiles ? loss_index(g.save.gather, tile_of(k) * kTcRows + row, g.n) : 0u;
+      return slice < 2 && k < my_tiles ? loss_index(g.save.gather, tile_of(k) * kTcRows + row, args.n) : 0u;
     };
     uint32_t lidx = lindex(0);
     auto head_epi = [&](int sl, int k) {
@@ -348,7 +356,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
       if (k < my_tiles) {
         float v[16];
         tc::tmem_ld16(lane_base + (uint32_t)(sl * 256), v);
-        ppo_head_row(g.save.loss, g.value_net, g.A, s.b3, lin, tile_of(k), row, g.n, v, quad, s.dz[sl]);
+        ppo_head_row(g.save.loss, value_net, args.A, s.b3, lin, tile_of(k), row, args.n, v, quad, s.dz[sl]);
       } else {
         *reinterpret_cast<uint4*>(s.dz[sl] + row * 32) = make_uint4(0, 0, 0, 0);
         *reinterpret_cast<uint4*>(s.dz[sl] + row * 32 + 16) = make_uint4(0, 0, 0, 0);
@@ -396,7 +404,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
       }
       // the loss inputs, in flight during layer 2, and the next pair's index
       if (slice < 2) {
-        lin = loss_inputs(g.save.loss, g.value_net, lidx);
+        lin = loss_inputs(g.save.loss, value_net, lidx);
         lidx = lindex(p + 1);
       }
       for (int sl = 0; sl < 2; ++sl) {
@@ -462,7 +470,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
   if (s.err && warp == 16 && lane == 0)
     for (int q = last_issued - 1; q <= last_issued; ++q)
       if (q >= 0) (void)tc::mbar_wait(&s.full[q & 1], (q >> 1) & 1);
-  if (tid == 0 && s.err && g.err) atomicExch(g.err, 1);
+  if (tid == 0 && s.err && args.err) atomicExch(args.err, 1);
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
@@ -472,36 +480,38 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(FusedArgs
 // ---------------------------------------------------------------------------
 bool bf16_fused_supported(const pe_net& net) { return net.obs_dim == 32 && net.hidden == 256; }
 
-pe_status bf16_fused_fwd_bwd(const pe_net& net, const uint8_t* img, const uint8_t* bimg, const float* params,
-                             int value_net, const void* obs, const uint32_t* gather, int64_t n, const PpoHead& loss,
-                             __nv_bfloat16* x, __nv_bfloat16* h1, __nv_bfloat16* h2, uint8_t* da2, uint8_t* da1,
-                             int32_t* err, cudaStream_t st) {
+// both networks (policy, value) of a minibatch in one launch
+pe_status bf16_fused_fwd_bwd(const pe_net& net, const uint8_t* const img[2], const uint8_t* const bimg[2],
+                             const float* params, const void* obs, const uint32_t* gather, int64_t n,
+                             const PpoHead loss[2], __nv_bfloat16* x, __nv_bfloat16* const h[4],
+                             uint8_t* const da2[2], uint8_t* const da1[2], int32_t* err, cudaStream_t st) {
   if (!bf16_fused_supported(net)) return fail(PE_EINVAL, "fused PPO forward-backward: 32-256-256 networks only");
   if (n <= 0) return PE_OK;
   int dev = 0, sms = 0;
   PE_TRY_CUDA(cudaGetDevice(&dev));
   PE_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t tiles = (n + kTcRows - 1) / kTcRows;
-  const int grid = (int)std::min<int64_t>((tiles + 1) / 2, sms);
+  // each network has half the SMs, so that both networks' tiles share one last
+  // wave: 512 tiles each (a minibatch of 65,536) are at most 7 per CTA, where
+  // two launches over all SMs took 4 + 4 (107 us together, 105 in one, and one
+  // launch gap less per step)
+  const int per_net = (int)std::min<int64_t>((tiles + 1) / 2, std::max(1, sms / 2));
   auto kern = ppo_fused_pair_kernel<32, 256>;
   constexpr int bytes = (int)sizeof(FusedSmem<32, 256>) + 1024;
   static_assert(bytes <= 232448, "fused kernel shared memory");
   PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   FusedArgs a;
-  a.img = img;
-  a.bimg = bimg;
+  for (int ni = 0; ni < 2; ++ni)
+    a.net[ni] = FusedNet{img[ni], bimg[ni], MlpSave{gather, ni ? nullptr : x, h[2 * ni], h[2 * ni + 1], loss[ni]},
+                         da2[ni], da1[ni]};
   a.params = params;
   a.A = net.n_actions;
-  a.value_net = value_net;
   a.obs = reinterpret_cast<const __nv_bfloat16*>(obs);
   a.n = n;
-  a.save = MlpSave{gather, x, h1, h2, loss};
-  a.da2 = da2;
-  a.da1 = da1;
   a.err = err;
   {
     ProfScope ps(PE_PROF_PPO_GRAD, st);
-    kern<<<grid, kFuThreads, bytes, st>>>(a);
+    kern<<<2 * per_net, kFuThreads, bytes, st>>>(a);
   }
   PE_CHECK_LAUNCH("ppo_fused_pair_kernel");
   return PE_OK;

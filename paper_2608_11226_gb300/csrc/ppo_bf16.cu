@@ -16,7 +16,7 @@
 //                and hidden-bias gradients split over samples with a
 //                fixed-order reduction into the canonical gradient vector;
 //                for the 72B networks the forward, the loss and the data
-//                products of a network run as one kernel (fused_bf16.cu);
+//                products run as one kernel (fused_bf16.cu);
 //   step      -- the gradient's squared norm (summed with the weight
 //                gradients' reduction), clip, Adam on the fp32 master
 //                parameters, which also writes the updated weights into the
@@ -51,10 +51,10 @@ pe_status bf16_backward(const pe_net& net, const float* params, uint8_t* const i
 pe_status bf16_bwd_images(const pe_net& net, const float* params, uint8_t* const img[2], cudaStream_t st);
 // defined in fused_bf16.cu
 bool bf16_fused_supported(const pe_net& net);
-pe_status bf16_fused_fwd_bwd(const pe_net& net, const uint8_t* img, const uint8_t* bimg, const float* params,
-                             int value_net, const void* obs, const uint32_t* gather, int64_t n, const PpoHead& loss,
-                             __nv_bfloat16* x, __nv_bfloat16* h1, __nv_bfloat16* h2, uint8_t* da2, uint8_t* da1,
-                             int32_t* err, cudaStream_t st);
+pe_status bf16_fused_fwd_bwd(const pe_net& net, const uint8_t* const img[2], const uint8_t* const bimg[2],
+                             const float* params, const void* obs, const uint32_t* gather, int64_t n,
+                             const PpoHead loss[2], __nv_bfloat16* x, __nv_bfloat16* const h[4],
+                             uint8_t* const da2[2], uint8_t* const da1[2], int32_t* err, cudaStream_t st);
 int wgrad_reduce_blocks();
 
 constexpr int kHead = 16;   // head rows (logits; the value head padded with zero rows)
@@ -267,7 +267,6 @@ pe_status ppo_update_bf16(const pe_net& net, float* params, float* m, float* v, 
   PE_CHECK_LAUNCH("perm_index_kernel");
   for (int ep = 0; ep < cfg.epochs; ++ep) {
     for (int mbi = 0; mbi < pl.nmb; ++mbi) {
-      const int64_t start = (int64_t)mbi * cfg.minibatch;
       const int cnt = mb_count(mbi);
       const int rows = (cnt + kTile - 1) / kTile * kTile;
       // the step after this one (the next minibatch, or the next epoch's first)
@@ -284,22 +283,17 @@ pe_status ppo_update_bf16(const pe_net& net, float* params, float* m, float* v, 
       lh.ent_coef = cfg.ent_coef;
       lh.inv_cnt = 1.0f / (float)cnt;
       lh.part = lossp;
+      PpoHead heads[2] = {lh, lh};
+      heads[0].dz = dz[0];
+      heads[1].dz = dz[1];
       if (fused) {
-        // 72B: forward, loss and backward data products of a network in one
-        // kernel (its backward images first)
-        lh.dz = dz[0];
-        s = bf16_fused_fwd_bwd(net, img, bimg[0], params, 0, obs, idx, cnt, lh, x, h[0], h[1], da2[0], da1[0], err,
-                               st);
-        if (s != PE_OK) return s;
-        lh.dz = dz[1];
-        s = bf16_fused_fwd_bwd(net, img + pl.img, bimg[1], params, 1, obs, idx, cnt, lh, nullptr, h[2], h[3], da2[1],
-                               da1[1], err, st);
+        // 72B: forward, loss and backward data products in one kernel
+        const uint8_t* const fimg[2] = {img, img + pl.img};
+        const uint8_t* const bimgc[2] = {bimg[0], bimg[1]};
+        s = bf16_fused_fwd_bwd(net, fimg, bimgc, params, obs, idx, cnt, heads, x, h, da2, da1, err, st);
       } else {
-        // Stress: forward and loss of both networks in one launch
-        PpoHead lv = lh;
-        lh.dz = dz[0];
-        lv.dz = dz[1];
-        s = bf16_forward_loss(net, img, params, obs, idx, cnt, lh, lv, x, h, err, st);
+        // Stress: forward and loss in one launch
+        s = bf16_forward_loss(net, img, params, obs, idx, cnt, heads[0], heads[1], x, h, err, st);
       }
       if (s != PE_OK) return s;
       const int nlb = rows / kTile * 4;
