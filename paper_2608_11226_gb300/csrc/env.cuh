@@ -256,16 +256,24 @@ __device__ void env_reset_at(const EnvDev& env, Acc& a, int o) {
   rebuild_history<C>(env, a, env.level_init);
 }
 
-// new episode at a random offset (Sec. 4.1); with several trace families,
-// word 1 of the draw picks the episode's family (Sec. 4.2 G2) and word 0
-// the offset inside that family's trace
+// where a new episode starts (Sec. 4.1): with several trace families, word 1
+// of the draw picks the episode's family (Sec. 4.2 G2), and word 0 the offset
+// inside that family's trace
+__device__ __forceinline__ int reset_offset(const EnvDev& env, const u32x4& w, int& fam) {
+  fam = env.F > 1 ? (int)__umulhi(w.y, (uint32_t)env.F) : 0;
+  const uint32_t span = (uint32_t)(fam_of(env, fam).L - env.span - kWLong + 1);
+  return kWLong + (int)__umulhi(w.x, span);
+}
+
+// new episode at a random offset
 template <int C, class Acc>
 __device__ void env_reset(const EnvDev& env, Acc& a, uint32_t eg, uint32_t t, uint32_t it,
                           uint32_t purpose) {
   const u32x4 w = philox10(u32x4{eg, t, it, purpose}, (uint32_t)env.seed, (uint32_t)(env.seed >> 32));
-  a.fam() = env.F > 1 ? (int)__umulhi(w.y, (uint32_t)env.F) : 0;
-  const uint32_t span = (uint32_t)(fam_of(env, a.fam()).L - env.span - kWLong + 1);
-  env_reset_at<C>(env, a, kWLong + (int)__umulhi(w.x, span));
+  int fam;
+  const int o = reset_offset(env, w, fam);
+  a.fam() = fam;
+  env_reset_at<C>(env, a, o);
 }
 
 template <int C, class Acc>
@@ -451,13 +459,10 @@ struct StepOut {
   int32_t q, v1, v60, done, samples;
 };
 
-// Apply action act and consume one sample (Sec. 4.1 actuator and action set
-// with the Sec. 4.2 floor g_min; Eqs. 1-3; G1 or Eq. 6 reward).
-// ONE: every step consumes one sample (no cadence table); `next`: that
-// sample, when the caller has fetched it ahead.
-template <int C, bool ONE = false, class Acc>
-__device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, float lambda,
-                                            const Samp<C>* next = nullptr) {
+// the action's effect on the actuator (Sec. 4.1 actuator and action set with
+// the Sec. 4.2 floor g_min); returns the new level
+template <class Acc>
+__device__ __forceinline__ int apply_action(const EnvDev& env, Acc& a, int act) {
   int nl = a.level();
   if (env.act_kind == PE_ACT_INCDEC) {
     if (act == 1 && nl > env.g_min) --nl;
@@ -470,13 +475,38 @@ __device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, 
   a.til() = (nl != a.level()) ? 0 : a.til() + 1;
   a.prev() = a.level();
   a.level() = nl;
+  return nl;
+}
+
+// tokens per generation sample at a level whose table entry is `rate`
+template <class Acc>
+__device__ __forceinline__ float token_rate(const EnvDev& env, Acc& a, float rate) {
+  if (env.act_kind == PE_ACT_INCDEC) rate = __fdiv_rn(rate * (float)a.b(), (float)env.b_init);
+  return rate;
+}
+
+// a step's reward from its sums, its largest 30 s excess and the fixed-reward sum
+__device__ __forceinline__ float step_reward(const EnvDev& env, const StepOut& o, float lambda, float peak_w,
+                                             float fixed) {
+  return env.reward_kind == PE_REWARD_LAGRANGE
+             ? o.tokens / 1000.0f - lambda * o.excess - 2.0f * lambda * peak_w  // Eq. 6
+             : fixed;
+}
+
+// Apply action act and consume one sample (Sec. 4.1 actuator and action set
+// with the Sec. 4.2 floor g_min; Eqs. 1-3; G1 or Eq. 6 reward).
+// ONE: every step consumes one sample (no cadence table); `next`: that
+// sample, when the caller has fetched it ahead.
+template <int C, bool ONE = false, class Acc>
+__device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, float lambda,
+                                            const Samp<C>* next = nullptr) {
+  const int nl = apply_action(env, a, act);
   // consume the step's samples (one, or a generation batch with a cadence
   // table): windows, violations and excess per sample; tokens and excess
   // summed; the Eq. 6 peak term is the batch's largest 30 s excess
   const Fam fm = fam_of(env, a.fam());
   const int64_t B60 = (int64_t)kWLong * fm.B;
-  float rate = a.tab.tokens[nl];
-  if (env.act_kind == PE_ACT_INCDEC) rate = __fdiv_rn(rate * (float)a.b(), (float)env.b_init);
+  const float rate = token_rate(env, a, a.tab.tokens[nl]);
   StepOut o;
   o.q = 0;
   o.v1 = 0;
@@ -537,9 +567,7 @@ __device__ __forceinline__ StepOut env_step(const EnvDev& env, Acc& a, int act, 
     for (; i < n; ++i) consume(std::integral_constant<int, 1>());
   }
   o.samples = n;
-  o.reward = env.reward_kind == PE_REWARD_LAGRANGE
-                 ? o.tokens / 1000.0f - lambda * o.excess - 2.0f * lambda * peak_w  // Eq. 6
-                 : fixed;
+  o.reward = step_reward(env, o, lambda, peak_w, fixed);
   a.k() += 1;
   o.done = a.k() == env.ep_len;
   return o;

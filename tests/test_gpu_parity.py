@@ -496,6 +496,44 @@ def test_replay_four_channel_traces(cadence):
     env.close()
 
 
+@pytest.mark.parametrize("preset,n_envs", [("72b", 61), ("72b", 1), ("mixed", 37), ("tiny", 50)])
+@pytest.mark.parametrize("rule", ["replay", "random", "threshold", "hysteresis"])
+def test_rule_rollout_batch_groups(preset, n_envs, rule):
+    """Steps of 8 or more samples without observations run on eight lanes per
+    env, every remainder of the batch included; with observations one thread
+    runs the env.  Both give the same bits over several episodes and calls,
+    and leave the same state (the last call observes both)."""
+    wl = {"72b": W.make_72b, "mixed": W.make_72b_mixed, "tiny": W.make_tiny}[preset](n_envs=n_envs)
+    spec = wl.env
+    spec.level_samples = [8 + (5 * l) % 17 for l in range(spec.n_levels)]
+    spec.episode_len = 9
+    kind = None if rule == "replay" else {"random": W.random_rule, "threshold": lambda: W.threshold_rule(spec.budget_q),
+                                          "hysteresis": lambda: W.hysteresis_rule(spec.budget_q)}[rule]()
+    envs = [pe.Env(spec, torch.from_numpy(wl.trace), torch.from_numpy(wl.phase)) for _ in range(2)]
+    rng = np.random.default_rng(5)
+    for it, T, obs in ((0, 20, (True, False)), (1, 7, (True, False)), (2, 3, (True, True))):
+        acts = torch.from_numpy(rng.integers(0, spec.n_actions, (T, n_envs)).astype(np.uint8)).cuda()
+        out = []
+        for env, ob in zip(envs, obs):
+            buf = pe.alloc_rule_rollout(spec, T, obs=True)
+            last = buf["obs_last"]
+            if not ob:
+                buf["obs"] = None
+            if kind is None:
+                pe.rollout_replay(env, acts, T, it, buf, lam=0.5)
+            else:
+                pe.rollout_rule(env, kind, T, it, buf, lam=0.5)
+            out.append({k: cpu(v) for k, v in buf.items() if v is not None})
+            assert buf["obs_last"] is last
+        for k in ("obs_last", "act", "done", "viol", "energy_q", "samples", "q", "reward", "tokens", "excess"):
+            assert np.array_equal(out[0][k], out[1][k]), (it, k)
+        if it == 0:
+            assert out[0]["done"].sum() == 2 * n_envs
+    assert np.array_equal(out[0]["obs"], out[1]["obs"])
+    for env in envs:
+        env.close()
+
+
 def test_rollout_parity_7b_sampled():
     wl = W.make_7b()
     rng = np.random.default_rng(3)
