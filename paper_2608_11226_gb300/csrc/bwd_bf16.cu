@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, H);
+  pdl_enter();
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -519,6 +520,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
   }
   for (int i = tid; i < 512 / 4; i += kWgThreads) reinterpret_cast<uint32_t*>(s.ones)[i] = 0x3F803F80u;
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, 512);
+  pdl_enter();
   tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
@@ -669,6 +671,7 @@ __global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const
   using R = WgReduce<H>;
   constexpr int NCH = H / 256, MB = H / 128;
   __shared__ float red[kWgReduceThreads / 32];
+  pdl_enter();
   const MlpLayout Lp = mlp_layout(D, H, A);
   float q = 0.0f;
   if (blockIdx.x < kWgReduceBlocks) {
@@ -815,7 +818,7 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     a.n = n;
     a.err = err;
     ProfScope ps(PE_PROF_PPO_GRAD, st);
-    kern<<<grid, kBwThreads, bytes, st>>>(a);
+    PE_TRY_CUDA(launch_pdl(kern, grid, kBwThreads, bytes, st, true, a));
   }
   PE_CHECK_LAUNCH("bwd_data_kernel");
   {
@@ -854,10 +857,10 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     const int bytes = (int)sizeof(WgSmem) + 1024;
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     ProfScope ps(PE_PROF_PPO_GRAD, st);
-    kern<<<ctas, kWgThreads, bytes, st>>>(a);
+    PE_TRY_CUDA(launch_pdl(kern, ctas, kWgThreads, bytes, st, true, a));
     PE_CHECK_LAUNCH("wgrad_kernel");
-    wgrad_reduce_kernel<D, H><<<wgrad_reduce_blocks(), kWgReduceThreads, 0, st>>>(part, a.S[0], a.S[1], A, grad, lossp,
-                                                                              nlb, stat5, sq);
+    PE_TRY_CUDA(launch_pdl(wgrad_reduce_kernel<D, H>, wgrad_reduce_blocks(), kWgReduceThreads, 0, st, true, part, a.S[0],
+                           a.S[1], A, grad, lossp, nlb, stat5, sq));
     PE_CHECK_LAUNCH("wgrad_reduce_kernel");
   }
   return PE_OK;

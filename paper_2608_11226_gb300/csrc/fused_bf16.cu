@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, 512);
+  pdl_enter();
   for (int i = tid; i < H; i += blockDim.x) {
     s.b1[i] = __ldg(args.params + (value_net ? Lp.c1 : Lp.b1) + i);
     s.b2[i] = __ldg(args.params + (value_net ? Lp.c2 : Lp.b2) + i);
@@ -511,7 +512,7 @@ pe_status bf16_fused_fwd_bwd(const pe_net& net, const uint8_t* const img[2], con
   a.err = err;
   {
     ProfScope ps(PE_PROF_PPO_GRAD, st);
-    kern<<<2 * per_net, kFuThreads, bytes, st>>>(a);
+    PE_TRY_CUDA(launch_pdl(kern, 2 * per_net, kFuThreads, bytes, st, true, a));
   }
   PE_CHECK_LAUNCH("ppo_fused_pair_kernel");
   return PE_OK;

@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, 512);
+  pdl_enter();
   for (int k = 0; k < nnet; ++k) {
     const int vn = two ? k : value_net;
     const int no = two ? (k ? 1 : A) : nout;
@@ -991,8 +992,11 @@ static pe_status launch_mlp(const uint8_t* img, const float* params, int A, int 
     const int bytes = (int)sizeof(MlpStreamSmem<D, H>) + 1024;
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     ProfScope ps(prof_kind, st);
-    kern<<<grid, kStreamThreads, bytes, st>>>(img, params, A, value_net, o, n, out, out_stride, nout, err, save,
-                                              second);
+    // early in an update's chain of kernels; a rollout's policy launches gain
+    // nothing (their blocks would sit waiting beside the env step: a Stress
+    // rollout of 262,144 envs x 8 steps took 4.00 ms so, and takes 3.90)
+    PE_TRY_CUDA(launch_pdl(kern, grid, kStreamThreads, bytes, st, second.img != nullptr, img, params, A, value_net, o, n,
+                           out, out_stride, nout, err, save, second));
   } else {
     if (second.img || save.loss.dz) return fail(PE_EINVAL, "PPO forward launches are for the streamed network");
     auto kern = mlp_bf16_pair_kernel<D, H>;

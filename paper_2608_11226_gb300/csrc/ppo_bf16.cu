@@ -100,6 +100,7 @@ struct AdamBf16Args {
 template <int D, int H>
 __global__ void adam_bf16_kernel(AdamBf16Args a) {
   __shared__ float s_norm;
+  pdl_enter();
   if (threadIdx.x < 32) {
     float t = 0.0f;
     for (int b = threadIdx.x; b < a.nsq; b += 32) t += a.sq[b];
@@ -332,9 +333,9 @@ pe_status ppo_update_bf16(const pe_net& net, float* params, float* m, float* v, 
       {
         ProfScope ps(PE_PROF_PPO_ADAM, st);
         if (pl.D == 32 && pl.H == 256)
-          adam_bf16_kernel<32, 256><<<ceil_div(pl.P, 256), 256, 0, st>>>(ad);
+          PE_TRY_CUDA(launch_pdl(adam_bf16_kernel<32, 256>, ceil_div(pl.P, 256), 256, 0, st, true, ad));
         else
-          adam_bf16_kernel<64, 512><<<ceil_div(pl.P, 256), 256, 0, st>>>(ad);
+          PE_TRY_CUDA(launch_pdl(adam_bf16_kernel<64, 512>, ceil_div(pl.P, 256), 256, 0, st, true, ad));
       }
       PE_CHECK_LAUNCH("ppo bf16 step kernels");
     }
