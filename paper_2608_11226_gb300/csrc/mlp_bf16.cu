@@ -392,11 +392,21 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(bar);
     };
-    // columns c .. c + 15 of this thread's row: tanh(acc + bias), packed bf16
-    auto chunk = [&](int c, const float* bias, uint32_t (&pk)[8]) {
-      float v[16];
-      tc::tmem_ld16(lane_addr + (uint32_t)c, v);
-      tc::tanh_bf16(v, bias + c, pk);
+    // a half of a hidden layer from column c0 on: tanh(acc + bias) of the
+    // thread's row, 16 columns at a time, each chunk's accumulators loaded while
+    // the one before is computed; done(j, c, packed bf16) takes them
+    auto half = [&](int c0, const float* bias, auto done) {
+      float v[2][16];
+      tc::tmem_get16(lane_addr + (uint32_t)c0, v[0]);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
+        const int c = c0 + j * 16;
+        tc::tmem_got16(v[j & 1]);
+        if (j + 1 < NJ) tc::tmem_get16(lane_addr + (uint32_t)(c + 16), v[(j + 1) & 1]);
+        uint32_t pk[8];
+        tc::tanh_bf16(v[j & 1], bias + c, pk);
+        done(j, c, pk);
+      }
     };
     // ... into the activation buffer (the next A operand)
     auto put = [&](int c, const uint32_t (&pk)[8]) {
@@ -471,36 +481,35 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       (void)wt(&s.m1a, par);
       tc::fence_after();
       {
-        const int c0 = slice * (H / 8);
-        uint32_t p0[8], p1[8];
-        chunk(c0, b1, p0);
-        chunk(c0 + 16, b1, p1);
-        if (t > 0) {
-          (void)wt(&s.mh, par ^ 1);
-          tc::fence_after();
-          if (warp < 4) {
-            // its accumulators out of TMEM (the loss comes later, while the
-            // layer-2 MMAs run), so that layer 1 may take the columns
-            float v[16];
-            tc::tmem_ld16(lane_addr + 256u, v);
+        uint32_t p0[8];
+        half(slice * (H / 8), b1, [&](int j, int c, const uint32_t (&pk)[8]) {
+          if (j == 0) {
 #pragma unroll
-            for (int j = 0; j < kHeadN; j += 4)
-              *reinterpret_cast<float4*>(&s.headv[row][j]) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&s.hd);
+            for (int q = 0; q < 8; ++q) p0[q] = pk[q];
+            return;
           }
-          wait_stored(&s.sa, 1);
-        }
-        put(c0, p0);
-        put(c0 + 16, p1);
-#pragma unroll 1
-        for (int j = 2; j < NJ; ++j) {
-          const int c = c0 + j * 16;
-          uint32_t pk[8];
-          chunk(c, b1, pk);
+          if (j == 1) {
+            if (t > 0) {
+              (void)wt(&s.mh, par ^ 1);
+              tc::fence_after();
+              if (warp < 4) {
+                // its accumulators out of TMEM (the loss comes later, while the
+                // layer-2 MMAs run), so that layer 1 may take the columns
+                float v[16];
+                tc::tmem_ld16(lane_addr + 256u, v);
+#pragma unroll
+                for (int q = 0; q < kHeadN; q += 4)
+                  *reinterpret_cast<float4*>(&s.headv[row][q]) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+                tc::fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&s.hd);
+              }
+              wait_stored(&s.sa, 1);
+            }
+            put(c - 16, p0);
+          }
           put(c, pk);
-        }
+        });
       }
       handover(&s.h1a);
       if (losing) {  // the previous tile's inputs, in flight during half B; this tile's index
@@ -512,13 +521,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       (void)wt(&s.m1b, par);
       if (t > 0) wait_stored(&s.sb, 1);
       tc::fence_after();
-#pragma unroll 1
-      for (int j = 0; j < NJ; ++j) {
-        const int c = H / 2 + slice * (H / 8) + j * 16;
-        uint32_t pk[8];
-        chunk(c, b1, pk);
-        put(c, pk);
-      }
+      half(H / 2 + slice * (H / 8), b1, [&](int, int c, const uint32_t (&pk)[8]) { put(c, pk); });
       handover(&s.h1b);
       // the next tile's X (both halves of this tile's layer 1 are done)
       if (warp >= 4 && t + 1 < my_tiles) put_x(t + 1);
@@ -537,34 +540,27 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
       (void)wt(&s.m2a, par);
       tc::fence_after();
       {
-        const int c0 = slice * (H / 8);
-        uint32_t p0[8], p1[8];
-        chunk(c0, b2, p0);
-        chunk(c0 + 16, b2, p1);
-        (void)wt(&s.n1lo, par);
-        wait_stored(&s.sa, 0);
-        tc::fence_after();
-        put(c0, p0);
-        put(c0 + 16, p1);
-#pragma unroll 1
-        for (int j = 2; j < NJ; ++j) {
-          const int c = c0 + j * 16;
-          uint32_t pk[8];
-          chunk(c, b2, pk);
+        uint32_t p0[8];
+        half(slice * (H / 8), b2, [&](int j, int c, const uint32_t (&pk)[8]) {
+          if (j == 0) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) p0[q] = pk[q];
+            return;
+          }
+          if (j == 1) {
+            (void)wt(&s.n1lo, par);
+            wait_stored(&s.sa, 0);
+            tc::fence_after();
+            put(c - 16, p0);
+          }
           put(c, pk);
-        }
+        });
       }
       handover(&s.h2a);
       (void)wt(&s.m2b, par);
       wait_stored(&s.sb, 0);
       tc::fence_after();
-#pragma unroll 1
-      for (int j = 0; j < NJ; ++j) {
-        const int c = H / 2 + slice * (H / 8) + j * 16;
-        uint32_t pk[8];
-        chunk(c, b2, pk);
-        put(c, pk);
-      }
+      half(H / 2 + slice * (H / 8), b2, [&](int, int c, const uint32_t (&pk)[8]) { put(c, pk); });
       handover(&s.h2in);
     }
     // the last tile's head
