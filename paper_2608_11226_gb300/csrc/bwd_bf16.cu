@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
   };
   // a bounded wait that is skipped once the CTA has an error
   auto wt = [&](uint64_t* b, uint32_t par) -> bool {
+    if (tc::mbar_try_wait(b, par)) return true;
     if (*reinterpret_cast<volatile int32_t*>(&s.err)) return false;
     if (tc::mbar_wait(b, par)) return true;
     atomicExch(&s.err, 1);
@@ -349,18 +350,16 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
     // d = bf16(TMEM (1 - h^2)) over this thread's chunks of half hf, in place
     // over h in the shared buffer
     auto epi = [&](int hf, bool valid) {
-#pragma unroll 2
-      for (int j = 0; j < NJ; ++j) {
-        const int c = hf * (H / 2) + slice * (H / 8) + j * 16;
-        float v[16];
-        tc::tmem_ld16(lane_addr + (uint32_t)c, v);
+      const int c0 = hf * (H / 2) + slice * (H / 8);
+      tc::tmem_chunks<NJ>(lane_addr + (uint32_t)c0, [&](int j, const float (&v)[16]) {
+        const int c = c0 + j * 16;
         const uint32_t o0 = tc::swz_offset<128>(row, c, kBwRows), o1 = tc::swz_offset<128>(row, c + 8, kBwRows);
         const uint4 hb[2] = {*reinterpret_cast<const uint4*>(s.da2 + o0), *reinterpret_cast<const uint4*>(s.da2 + o1)};
         uint32_t pk[8];
         tanh_grad16(v, hb, valid, pk);
         *reinterpret_cast<uint4*>(s.da2 + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.da2 + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      }
+      });
     };
     auto handover = [&](uint64_t* bar) {
       tc::fence_async_smem();

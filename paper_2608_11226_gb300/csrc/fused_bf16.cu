@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
   // a bounded wait that is skipped once the CTA has an error (so that a
   // failed CTA does not spend one time-out per remaining hand-over)
   auto wt = [&](uint64_t* b, uint32_t par) -> bool {
+    if (tc::mbar_try_wait(b, par)) return true;
     if (*reinterpret_cast<volatile int32_t*>(&s.err)) return false;
     if (tc::mbar_wait(b, par)) return true;
     atomicExch(&s.err, 1);
@@ -329,18 +330,15 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
     };
     // hidden layer: tanh(acc + bias) -> bf16 -> act[sl]
     auto hidden = [&](int sl, const float* bias) {
-#pragma unroll
-      for (int j = 0; j < NJ / 2; ++j) {
-        const int c = slice * (H / 4) + j * 32;
-        float v[32];
-        tc::tmem_ld32(lane_base + (uint32_t)(sl * 256 + c), v);
-        uint32_t pk[16];
+      const int c0 = slice * (H / 4);
+      tc::tmem_chunks<NJ>(lane_base + (uint32_t)(sl * 256 + c0), [&](int j, const float (&v)[16]) {
+        const int c = c0 + j * 16;
+        uint32_t pk[8];
         tc::tanh_bf16(v, bias + c, pk);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-          *reinterpret_cast<uint4*>(s.act[sl] + tc::swz_offset<128>(row, c + 8 * q, kTcRows)) =
-              make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-      }
+        const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
+        *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+      });
     };
     // head: the PPO loss per row, dz to its tile image and to the slot's
     // shared dz tile (zeros for a slot without a tile); slot s by the four
@@ -367,11 +365,9 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
     // place), or da1 with h1 from registers (hv, this thread's own h1 chunks)
     auto grad_epi = [&](int sl, int k, const uint4 (*hv)[2]) {
       const bool valid = row < rows_of(k);
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
-        const int c = slice * (H / 4) + j * 16;
-        float v[16];
-        tc::tmem_ld16(lane_base + (uint32_t)(sl * 256 + c), v);
+      const int c0 = slice * (H / 4);
+      tc::tmem_chunks<NJ>(lane_base + (uint32_t)(sl * 256 + c0), [&](int j, const float (&v)[16]) {
+        const int c = c0 + j * 16;
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
         uint4 hb[2];
         if (hv) {
@@ -385,7 +381,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
         tanh_grad16(v, hb, valid, pk);
         *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      }
+      });
     };
     fetch_x(0, xv[0]);
     fetch_x(1, xv[1]);

@@ -223,6 +223,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
   };
   // a bounded wait that is skipped once the CTA has an error
   auto wt = [&](uint64_t* b, uint32_t par) -> bool {
+    if (tc::mbar_try_wait(b, par)) return true;
     if (*reinterpret_cast<volatile int32_t*>(&s.err)) return false;
     if (tc::mbar_wait(b, par)) return true;
     atomicExch(&s.err, 1);
@@ -396,17 +397,12 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     // thread's row, 16 columns at a time, each chunk's accumulators loaded while
     // the one before is computed; done(j, c, packed bf16) takes them
     auto half = [&](int c0, const float* bias, auto done) {
-      float v[2][16];
-      tc::tmem_get16(lane_addr + (uint32_t)c0, v[0]);
-#pragma unroll
-      for (int j = 0; j < NJ; ++j) {
+      tc::tmem_chunks<NJ>(lane_addr + (uint32_t)c0, [&](int j, const float (&v)[16]) {
         const int c = c0 + j * 16;
-        tc::tmem_got16(v[j & 1]);
-        if (j + 1 < NJ) tc::tmem_get16(lane_addr + (uint32_t)(c + 16), v[(j + 1) & 1]);
         uint32_t pk[8];
-        tc::tanh_bf16(v[j & 1], bias + c, pk);
+        tc::tanh_bf16(v, bias + c, pk);
         done(j, c, pk);
-      }
+      });
     };
     // ... into the activation buffer (the next A operand)
     auto put = [&](int c, const uint32_t (&pk)[8]) {
@@ -775,17 +771,15 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     };
     // hidden layer epilogue of slot sl: tanh(acc + bias) -> bf16 -> act[sl]
     auto hidden = [&](int sl, const float* bias) {
-#pragma unroll
-      for (int j = 0; j < H / 64; ++j) {
-        const int c = slice * (H / 4) + j * 16;
-        float v[16];
-        tc::tmem_ld16(lane_base + (uint32_t)(sl * 256 + c), v);
+      const int c0 = slice * (H / 4);
+      tc::tmem_chunks<H / 64>(lane_base + (uint32_t)(sl * 256 + c0), [&](int j, const float (&v)[16]) {
+        const int c = c0 + j * 16;
         uint32_t pk[8];
         tc::tanh_bf16(v, bias + c, pk);
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
         *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      }
+      });
     };
     auto handover = [&](uint64_t* bar) {
       tc::fence_async_smem();

@@ -148,27 +148,25 @@ __device__ __forceinline__ void tmem_got16(float (&v)[16]) {
                : "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// N chunks of 16 columns from taddr on, each loaded while f(j, values) works on
+// the one before
+template <int N, class F>
+__device__ __forceinline__ void tmem_chunks(uint32_t taddr, F f) {
+  float v[2][16];
+  tmem_get16(taddr, v[0]);
 #pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+  for (int j = 0; j < N; ++j) {
+    tmem_got16(v[j & 1]);
+    if (j + 1 < N) tmem_get16(taddr + (uint32_t)(16 * (j + 1)), v[(j + 1) & 1]);
+    f(j, v[j & 1]);
+  }
 }
 
 // 32 bytes of global memory in one load from L2 (32-byte aligned): a warp whose
 // lanes read 32 different lines takes 32 L1 cycles per request of either
 // width, so half as many as with 16-byte loads.  In the 72B PPO kernel issuing
-// the h1 chunks took 4-5 k clk of a tile's 58 k; with this and 32-column TMEM
-// loads a 72B update of 262,144 samples x 2 epochs went from 6.84 to 6.57 ms.
+// the h1 chunks took 4-5 k clk of a tile's 58 k; a 72B update of 32 steps went
+// from 6.84 to 6.57 ms.
 __device__ __forceinline__ void ld_global32(const void* p, uint4& lo, uint4& hi) {
   asm volatile("ld.relaxed.gpu.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
@@ -226,6 +224,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* b, uint32_t parity) {
 
 // bounded wait for phase `parity` of the barrier: false after ~`cycles` SM cycles
 __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, long long cycles = 4000000000LL) {
+  if (mbar_try_wait(b, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_try_wait(b, parity)) {
     if (clock64() - t0 > cycles) return false;
