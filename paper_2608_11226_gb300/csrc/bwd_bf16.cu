@@ -42,7 +42,7 @@
 //   is not a multiple of the SM count.
 // wgrad_kernel (split over samples): each CTA owns 128 output rows (one
 //   block of layer outputs o) of one network and one 256-column chunk, and
-//   accumulates over its share of the minibatch, 64 samples per stage:
+//   accumulates over its share of the minibatch, 32 samples per stage:
 //   [dW2 | db2] = da2^T [h1 | 1], and for column chunk 0 also
 //   [dW1 | db1] = da1^T [x | 1] and dW3^T = h2^T dz; it writes its fp32
 //   accumulators as one partial block.  Column chunk 0's stages bring more
@@ -428,17 +428,25 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
 }
 
 // ---------------------------------------------------------------------------
-// weight gradients: split over samples, 64 samples per stage
+// weight gradients: split over samples, 32 samples per stage
 // ---------------------------------------------------------------------------
-constexpr int kWgSamples = 64;
+constexpr int kWgSamples = 32;
 constexpr int kWgThreads = 128;
 // stage layout (bytes): A da2 | A da1 | A h2 (each 2 blocks of 64 features x
-// 64 samples), B h1 (4 blocks: 256 columns), B x (64 samples x D), B dz
-constexpr int kWgA = 2 * kWgSamples * 128;  // 16 KB
+// 32 samples), B h1 (4 blocks: 256 columns), B x (32 samples x D), B dz; the
+// second column chunk's stages hold da2 and h1 alone.  The kernel is bound by
+// the bytes it keeps in flight, so the stages are small and fill the shared
+// memory: 4 of 45 KB, or 8 of 24 KB.  With two slots of 90 KB for either, of
+// which column chunk 1 used 48, a Stress update took 6.55 ms and a 72B update
+// 5.73 ms; now 6.35 and 5.67.  (5 and 9 slots: 6.37 and 5.79 ms, the next
+// kernel's blocks then find no shared memory beside this one's.)
+constexpr int kWgA = 2 * kWgSamples * 128;  // 8 KB
 constexpr int kWgDa2 = 0, kWgDa1 = kWgA, kWgH2 = 2 * kWgA, kWgH1 = 3 * kWgA;
-constexpr int kWgX = kWgH1 + 4 * kWgSamples * 128;        // 80 KB
-constexpr int kWgDz = kWgX + kWgSamples * 128;            // x takes at most 8 KB
-constexpr int kWgStageBytes = kWgDz + kWgSamples * 32;    // 90 KB
+constexpr int kWgX = kWgH1 + 4 * kWgSamples * 128;        // 40 KB
+constexpr int kWgDz = kWgX + kWgSamples * 128;            // x takes at most 4 KB
+constexpr int kWgStageBytes = kWgDz + kWgSamples * 32;    // 45 KB
+constexpr int kWgStageBytes1 = kWgA + 4 * kWgSamples * 128;  // 24 KB
+constexpr int kWgSlots = 4, kWgSlots1 = 8;                // powers of two
 constexpr int kWgMaxCols = 256 + 16 + 64 + 16 + 16;       // dW2 | db2 | dW1 | db1 | dW3^T
 
 template <int D>
@@ -447,9 +455,9 @@ struct WgCols {  // TMEM / partial-block column of each product
 };
 
 struct WgSmem {
-  alignas(1024) uint8_t st[2][kWgStageBytes];
+  alignas(1024) uint8_t st[std::max(kWgSlots * kWgStageBytes, kWgSlots1 * kWgStageBytes1)];
   alignas(1024) uint8_t ones[512];  // 16 samples x 16 columns of bf16 ones (B of the bias sums)
-  uint64_t full[2], empty[2], bar_mma;
+  uint64_t full[kWgSlots1], empty[kWgSlots1], bar_mma;
   uint32_t tmem_base;
   int32_t err;
 };
@@ -462,7 +470,7 @@ struct WgArgs {
   WgNet net[2];
   const uint8_t* x;   // shared input tile images
   int64_t n;          // valid samples
-  int nstages;        // ceil(n / 64)
+  int nstages;        // ceil(n / 32)
   int spc[2];         // stages per CTA, per column chunk
   int S[2];           // sample chunks (CTAs per group), per column chunk
   float* part;        // one [128][kWgMaxCols] partial block per CTA, in CTA order
@@ -510,7 +518,7 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
   const int k0 = chunk * spc, k1 = min(k0 + spc, g.nstages);
   if (tid == 0) {
     s.err = 0;
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kWgSlots1; ++i) {
       tc::mbar_init(&s.full[i], 1);
       tc::mbar_init(&s.empty[i], 1);
     }
@@ -525,23 +533,26 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = s.tmem_base;
-  const int64_t hb = (int64_t)kWgSamples * 128;  // bytes of one 64-sample half of a 128-row block
+  const int64_t hb = (int64_t)kWgSamples * 128;  // bytes of one 32-sample quarter of a 128-row block
+  const int lslots = first ? 2 : 3, nslots = 1 << lslots;
+  const int stage_bytes = first ? kWgStageBytes : kWgStageBytes1, h1_off = first ? kWgH1 : kWgA;
+  static_assert(kWgSlots == 4 && kWgSlots1 == 8 && kBwRows == 4 * kWgSamples, "slots and stages per tile");
   int last_issued = -1;
   if (warp == 0) {
     if (lane == 0) {
       for (int k = k0; k < k1; ++k) {
-        const int j = k - k0, slot = j & 1;
-        if (j >= 2 && !tc::mbar_wait(&s.empty[slot], ((j - 2) >> 1) & 1)) {
+        const int j = k - k0, slot = j & (nslots - 1);
+        if (j >= nslots && !tc::mbar_wait(&s.empty[slot], ((j >> lslots) - 1) & 1)) {
           atomicExch(&s.err, 1);
           break;
         }
-        const int64_t tile = k >> 1, half = k & 1;
+        const int64_t tile = k >> 2, part = k & 3;
         const int64_t tb = tile * (int64_t)(kBwRows * H * 2);  // tile image base of a hidden-width operand
-        uint8_t* d = s.st[slot];
+        uint8_t* d = s.st + slot * stage_bytes;
         const uint32_t bytes = (uint32_t)(2 * hb + 4 * hb + (first ? 4 * hb + kWgSamples * XB + kWgSamples * 32 : 0));
         tc::mbar_expect_tx(&s.full[slot], bytes);
         for (int q = 0; q < 2; ++q) {
-          const int64_t off = tb + (int64_t)(2 * mb + q) * kBwRows * 128 + half * hb;
+          const int64_t off = tb + (int64_t)(2 * mb + q) * kBwRows * 128 + part * hb;
           tc::bulk_g2s(d + kWgDa2 + q * hb, nt.da2 + off, (uint32_t)hb, &s.full[slot]);
           if (first) {
             tc::bulk_g2s(d + kWgDa1 + q * hb, nt.da1 + off, (uint32_t)hb, &s.full[slot]);
@@ -549,13 +560,13 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
           }
         }
         for (int q = 0; q < 4; ++q) {
-          const int64_t off = tb + (int64_t)(4 * nc + q) * kBwRows * 128 + half * hb;
-          tc::bulk_g2s(d + kWgH1 + q * hb, nt.h1 + off, (uint32_t)hb, &s.full[slot]);
+          const int64_t off = tb + (int64_t)(4 * nc + q) * kBwRows * 128 + part * hb;
+          tc::bulk_g2s(d + h1_off + q * hb, nt.h1 + off, (uint32_t)hb, &s.full[slot]);
         }
         if (first) {
-          tc::bulk_g2s(d + kWgX, g.x + tile * (int64_t)(kBwRows * XB) + half * kWgSamples * XB,
+          tc::bulk_g2s(d + kWgX, g.x + tile * (int64_t)(kBwRows * XB) + part * kWgSamples * XB,
                        (uint32_t)(kWgSamples * XB), &s.full[slot]);
-          tc::bulk_g2s(d + kWgDz, nt.dz + tile * (int64_t)(kBwRows * 32) + half * kWgSamples * 32,
+          tc::bulk_g2s(d + kWgDz, nt.dz + tile * (int64_t)(kBwRows * 32) + part * kWgSamples * 32,
                        (uint32_t)(kWgSamples * 32), &s.full[slot]);
         }
         last_issued = j;
@@ -571,18 +582,18 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
       constexpr uint32_t kXAtom = D == 32 ? 512 : 1024;
       const uint64_t ones = tc::desc_strided(onea, 16, 256, tc::kLayoutSW32);
       for (int k = k0; k < k1; ++k) {
-        const int j = k - k0, slot = j & 1;
-        if (!tc::mbar_wait(&s.full[slot], (j >> 1) & 1)) {
+        const int j = k - k0, slot = j & (nslots - 1);
+        if (!tc::mbar_wait(&s.full[slot], (j >> lslots) & 1)) {
           atomicExch(&s.err, 1);
           break;
         }
         tc::fence_after();
-        const uint32_t sa = tc::smem_u32(s.st[slot]);
+        const uint32_t sa = tc::smem_u32(s.st + slot * stage_bytes);
 #pragma unroll
         for (int kk = 0; kk < kWgSamples / 16; ++kk) {
           const uint32_t acc = (j | kk) != 0;
           const uint64_t a2 = tc::desc_strided(sa + kWgDa2 + kk * 2048, (uint32_t)hb, 1024, tc::kLayoutSW128);
-          tc::mma_bf16(tmem + Cn::DW2, a2, tc::desc_strided(sa + kWgH1 + kk * 2048, (uint32_t)hb, 1024, tc::kLayoutSW128),
+          tc::mma_bf16(tmem + Cn::DW2, a2, tc::desc_strided(sa + h1_off + kk * 2048, (uint32_t)hb, 1024, tc::kLayoutSW128),
                        kIdW2, acc);
           if (first) {
             tc::mma_bf16(tmem + Cn::DB2, a2, ones, kId16, acc);
@@ -622,8 +633,10 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
   }
   tc::fence_before();
   __syncthreads();
-  if (s.err && warp == 0 && lane == 0 && last_issued >= 0)
-    (void)tc::mbar_wait(&s.full[last_issued & 1], (last_issued >> 1) & 1);
+  // on an error, the copies that may still be in flight
+  if (s.err && warp == 0 && lane == 0)
+    for (int j = std::max(0, last_issued - nslots + 1); j <= last_issued; ++j)
+      (void)tc::mbar_wait(&s.full[j & (nslots - 1)], (j >> lslots) & 1);
   if (tid == 0 && s.err && g.err) atomicExch(g.err, 1);
   __syncthreads();
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
@@ -829,7 +842,7 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     a.nstages = (int)((n + kWgSamples - 1) / kWgSamples);
     // CTAs per (network, row block), split between the column chunks in
     // proportion to the bytes a stage brings in: chunk 0 also loads da1, h2,
-    // x and dz (for the Stress networks 90 KB per stage against 48 KB), so
+    // x and dz (for the Stress networks 45 KB per stage against 24 KB), so
     // with equal shares its CTAs would set the launch's length
     constexpr int NCH = H / 256;
     const int cap = std::max(NCH, std::min(sms, kWgMaxCtas) / (groups / NCH));
@@ -853,7 +866,8 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     a.part = part;
     a.err = err;
     auto kern = wgrad_kernel<D, H>;
-    const int bytes = (int)sizeof(WgSmem) + 1024;
+    constexpr int bytes = (int)sizeof(WgSmem) + 1024;
+    static_assert(bytes <= 232448, "weight-gradient shared memory");
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     ProfScope ps(PE_PROF_PPO_GRAD, st);
     PE_TRY_CUDA(launch_pdl(kern, ctas, kWgThreads, bytes, st, true, a));
