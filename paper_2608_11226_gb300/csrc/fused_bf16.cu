@@ -366,8 +366,11 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
     auto grad_epi = [&](int sl, int k, const uint4 (*hv)[2]) {
       const bool valid = row < rows_of(k);
       const int c0 = slice * (H / 4);
-      tc::tmem_chunks<NJ>(lane_base + (uint32_t)(sl * 256 + c0), [&](int j, const float (&v)[16]) {
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) {
         const int c = c0 + j * 16;
+        float v[16];
+        tc::tmem_ld16(lane_base + (uint32_t)(sl * 256 + c), v);
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
         uint4 hb[2];
         if (hv) {
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
         tanh_grad16(v, hb, valid, pk);
         *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
-      });
+      }
     };
     fetch_x(0, xv[0]);
     fetch_x(1, xv[1]);
