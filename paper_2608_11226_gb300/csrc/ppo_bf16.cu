@@ -101,8 +101,14 @@ template <int D, int H>
 __global__ void adam_bf16_kernel(AdamBf16Args a) {
   __shared__ float s_norm;
   pdl_enter();
+  // this thread's parameter and moments, in flight while the norm is summed
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool mine = p < a.P;
+  float g0 = 0.0f, m0 = 0.0f, v0 = 0.0f, p0 = 0.0f;
+  if (mine) g0 = a.grad[p], m0 = a.m[p], v0 = a.v[p], p0 = a.params[p];
   if (threadIdx.x < 32) {
     float t = 0.0f;
+#pragma unroll 4
     for (int b = threadIdx.x; b < a.nsq; b += 32) t += a.sq[b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -111,27 +117,27 @@ __global__ void adam_bf16_kernel(AdamBf16Args a) {
   __syncthreads();
   const float norm = s_norm;
   const float coef = fminf(1.0f, a.max_norm / (norm + 1e-6f));
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.P; p += (int64_t)gridDim.x * blockDim.x) {
-    const float gp = a.grad[p] * coef;
-    const float mp = a.beta1 * a.m[p] + (1.0f - a.beta1) * gp;
-    const float vp = a.beta2 * a.v[p] + (1.0f - a.beta2) * gp * gp;
+  if (mine) {
+    const float gp = g0 * coef;
+    const float mp = a.beta1 * m0 + (1.0f - a.beta1) * gp;
+    const float vp = a.beta2 * v0 + (1.0f - a.beta2) * gp * gp;
     a.m[p] = mp;
     a.v[p] = vp;
-    const float pn = a.params[p] - a.step_size * mp / (sqrtf(vp) * a.inv_sqrt_bc2 + a.eps);
+    const float pn = p0 - a.step_size * mp / (sqrtf(vp) * a.inv_sqrt_bc2 + a.eps);
     a.params[p] = pn;
     // the weight's place in the images: network, layer, row, column
     const MlpLayout L = mlp_layout(D, H, a.A);
     int net = -1, mat = 0;
-    int64_t q = 0;
-    if (p < L.b1) net = 0, mat = 1, q = p - L.w1;
-    else if (p >= L.w2 && p < L.b2) net = 0, mat = 2, q = p - L.w2;
-    else if (p >= L.w3 && p < L.b3) net = 0, mat = 3, q = p - L.w3;
-    else if (p >= L.v1 && p < L.c1) net = 1, mat = 1, q = p - L.v1;
-    else if (p >= L.v2 && p < L.c2) net = 1, mat = 2, q = p - L.v2;
-    else if (p >= L.v3 && p < L.c3) net = 1, mat = 3, q = p - L.v3;
+    int q = 0;
+    if (p < L.b1) net = 0, mat = 1, q = (int)(p - L.w1);
+    else if (p >= L.w2 && p < L.b2) net = 0, mat = 2, q = (int)(p - L.w2);
+    else if (p >= L.w3 && p < L.b3) net = 0, mat = 3, q = (int)(p - L.w3);
+    else if (p >= L.v1 && p < L.c1) net = 1, mat = 1, q = (int)(p - L.v1);
+    else if (p >= L.v2 && p < L.c2) net = 1, mat = 2, q = (int)(p - L.v2);
+    else if (p >= L.v3 && p < L.c3) net = 1, mat = 3, q = (int)(p - L.v3);
     if (net >= 0) {
       const int cols = mat == 1 ? D : H;
-      const int r = (int)(q / cols), k = (int)(q % cols);
+      const int r = q / cols, k = q % cols;
       const __nv_bfloat16 b = __float2bfloat16_rn(pn);
       *reinterpret_cast<__nv_bfloat16*>(a.fimg + net * a.fstride + fwd_img_offset<D, H>(mat, r, k)) = b;
       if (mat >= 2) *reinterpret_cast<__nv_bfloat16*>(a.bimg[net] + bwd_img_offset<H>(mat, r, k)) = b;
