@@ -513,12 +513,12 @@ def run_fleet(args, world, tr=None, roofs=None):
                        "n": N, "horizon": H},
             "kernel_ms_per_launch": wms / wn if wn else None,
             "composed_samples_per_s": composed / (wms / wn / 1e3) if wn else None,
-            "logical_l2_gbs": 4.0 * fw.n_jobs * composed / (wms / wn / 1e3) / 1e9 if wn else None,
-            "roofline": ({"kernel": "fleet_windows_v4_kernel", "bound": "l2",
-                          "achieved": 4.0 * fw.n_jobs * composed / (wms / wn / 1e3) / 1e9,
+            "logical_l2_gbs": 2.0 * fw.n_jobs * composed / (wms / wn / 1e3) / 1e9 if wn else None,
+            "roofline": ({"kernel": "fleet_windows_h16_kernel", "bound": "l2",
+                          "achieved": 2.0 * fw.n_jobs * composed / (wms / wn / 1e3) / 1e9,
                           "peak": roofs["l2_read"]["value"], "unit": "GB/s",
-                          "frac": 4.0 * fw.n_jobs * composed / (wms / wn / 1e3) / 1e9 / roofs["l2_read"]["value"],
-                          "note": "logical bytes: 4 B per job per composed sample, against the measured "
+                          "frac": 2.0 * fw.n_jobs * composed / (wms / wn / 1e3) / 1e9 / roofs["l2_read"]["value"],
+                          "note": "logical bytes: 2 B per job per composed sample, against the measured "
                                   "L2-read roof (32 MB resident buffer)"}
                          if (wn and roofs) else None),
             "violation_fraction_mean": [float(c[:, i].mean() / (H - w + 1)) for i, w in enumerate(windows)],
@@ -1069,19 +1069,19 @@ def per_config_table(out):
 def gae_kernel_name(E: int) -> str:
     """The GAE kernel the library picks for a batch of E envs (its dispatch
     by width): streamed per env column for wide batches, chunked below."""
-    if E >= 196608 and E % 4 == 0:
-        return "gae_stream_kernel<4, 8>"
+    if E >= 196608:
+        return "gae_stream_kernel<32, 128>"
     if E >= 49152:
-        return "gae_stream_kernel<1, 16>"
+        return "gae_stream_kernel<16, 64>"
     if E >= 32768:
-        return "gae_stream_kernel<1, 32>"
+        return "gae_stream_kernel<32, 128>"
     return "gae_kernel_v (chunked)"
 
 
 def gae_traffic(env_steps: int, E: int):
     """DRAM bytes of one GAE launch larger than L2, scaled from the committed
     capture's bytes per env-step of the same kernel."""
-    key = "traffic_bytes_per_env_step_v4" if E >= 196608 and E % 4 == 0 else "traffic_bytes_per_env_step_v1"
+    key = "traffic_bytes_per_env_step_v4" if E >= 196608 else "traffic_bytes_per_env_step_v1"
     b = load_traffic_per_unit("gae_stream_kernel", key) if E >= 32768 else None
     return None if b is None else b * env_steps
 
@@ -1230,9 +1230,9 @@ def run_ncu_case(name: str):
         for _ in range(3):
             pe.gae(r, v, d, lv, 0.99, 0.95, adv, ret)
     elif name == "gae":
-        # the two streamed launch shapes: 1,024 x 65,536 (one env per thread,
-        # the 72B rollout's shape, 1.1 GB of algorithmic traffic) and
-        # 512 x 262,144 (four envs per thread, the Stress width, 2.3 GB)
+        # the two streamed launch shapes: 1,024 x 65,536 (the 72B rollout's, 64
+        # threads per CTA, 1.1 GB of algorithmic traffic) and 512 x 262,144
+        # (the Stress width, 128 threads, 2.3 GB)
         for T, E in ((1024, 65536), (512, 262144)):
             g = torch.Generator(device="cuda").manual_seed(0)
             r = torch.randn(T, E, device="cuda", generator=g)

@@ -345,10 +345,11 @@ pe_status pe_ppo_update(const pe_net* net, float* params, float* adam_m, float* 
  *  (all device memory); windows: [W] HOST array, W in [1, 4], each w in [1, 992];
  *  counts, peaks: [N][W] int32 (device).
  *  workspace: pe_fleet_workspace_bytes(J, L, H) bytes.  For J <= 8 that size
- *  holds four copies of the per-job prefix sums, each shifted by one sample,
- *  so that the counts use 16-byte loads; a smaller workspace, down to the one
- *  copy of J * (L + H + 128) words plus 1 KiB, gives the same results through
- *  4-byte loads.
+ *  holds eight shifted copies of the jobs' samples in 16 bits (where their
+ *  ranges allow it) or four of their prefix sums, so that the counts use
+ *  16-byte loads; a smaller workspace, down to the one copy of
+ *  J * (L + H + 128) words plus 1 KiB, gives the same results through 4-byte
+ *  loads.
  * The call validates the traces on the device and waits for that check
  * (one small device-to-host read on `stream`) before launching the counts.
  * Errors: PE_EINVAL (sizes, pointers, job map or offsets out of range),

@@ -123,13 +123,6 @@ __device__ __forceinline__ float ratio_i(int32_t num, int32_t den) {
   return __fdiv_rn(__int2float_rn(num), __int2float_rn(den));
 }
 
-__device__ __forceinline__ float bf16r(float x) {
-  // round-to-nearest-even to bf16, returned as fp32
-  uint32_t u = __float_as_uint(x);
-  u += 0x7FFFu + ((u >> 16) & 1u);
-  return __uint_as_float(u & 0xFFFF0000u);
-}
-
 // Approximate KL term of one sample, (rho - 1) - log rho with
 // rho = exp(x) (Schulman's k3 estimator), without the cancellation of the
 // literal fp32 form: for |x| < 1/8 the Taylor series of e^x - 1 - x,

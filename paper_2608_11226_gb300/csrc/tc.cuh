@@ -174,22 +174,6 @@ __device__ __forceinline__ void ld_global32(const void* p, uint4& lo, uint4& hi)
                : "memory");
 }
 
-// named barrier `id` over `nthreads` threads that also ORs a predicate across
-// them: every thread gets the same answer, so a loop can stop uniformly
-__device__ __forceinline__ bool bar_any(int id, int nthreads, bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "bar.red.or.pred q, %2, %3, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t"
-      "}\n"
-      : "=r"(r)
-      : "r"((uint32_t)pred), "r"(id), "r"(nthreads)
-      : "memory");
-  return r != 0;
-}
-
 // ask L2 to fetch `bytes` (a multiple of 16) from p on (16-byte aligned; no wait)
 __device__ __forceinline__ void bulk_prefetch_l2(const void* p, uint32_t bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
