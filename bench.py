@@ -1069,12 +1069,17 @@ def per_config_table(out):
 def gae_kernel_name(E: int) -> str:
     """The GAE kernel the library picks for a batch of E envs (its dispatch
     by width): streamed per env column for wide batches, chunked below."""
-    if E >= 196608:
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if E > 920 * sms:
         return "gae_stream_kernel<32, 128>"
-    if E >= 49152:
+    if E > 400 * sms:
         return "gae_stream_kernel<16, 64>"
+    if E > 250 * sms and E % 4 == 0:
+        return "gae_stream_kernel<32, 64>"
     if E >= 32768:
         return "gae_stream_kernel<32, 128>"
+    if E > 128 * sms:
+        return "gae_stream_kernel<64, 64>"
     return "gae_kernel_v (chunked)"
 
 

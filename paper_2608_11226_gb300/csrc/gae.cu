@@ -10,7 +10,7 @@
 // through shared memory, and each thread then re-runs its chunk with the
 // right carry-in and streams A and R out.  Longer horizons loop over
 // super-chunks of CL*NW steps from the end.  That time-parallel form serves
-// narrow batches; batches of 32,768 envs or more take the barrier-free
+// narrow batches; wider ones (the rule is in gae_launch) take the barrier-free
 // per-column kernel below.
 #include <type_traits>
 
@@ -128,8 +128,8 @@ __global__ void __launch_bounds__(32 * NW)
 }
 
 
-// Wide batches (E >= 32,768): one thread per env walks the whole horizon
-// backwards, A_t = delta_t + gamma lambda (1 - d_t) A_{t+1} in the same
+// Batches too wide for the chunked kernels: one thread per env walks the whole
+// horizon backwards, A_t = delta_t + gamma lambda (1 - d_t) A_{t+1} in the same
 // order as the recursion, with no barrier and no shared memory.  The loads of
 // the next P steps are kept in flight in a register ring, so each SM holds
 // enough outstanding bytes to cover HBM latency; every warp streams
@@ -210,16 +210,29 @@ pe_status gae_launch(const float* r, const float* v, const uint8_t* d, const flo
                                       reinterpret_cast<uintptr_t>(adv) | reinterpret_cast<uintptr_t>(ret) |
                                       reinterpret_cast<uintptr_t>(last_v)) % 8 == 0) &&
                    reinterpret_cast<uintptr_t>(d) % 2 == 0;
-  if (E >= 196608) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (E >= 49152) return gae_stream_run<16, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (E >= 32768) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (n >= ((int64_t)1 << 28) && al4) return gae_run<4, 8, 4>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (E >= 16384 && al2) return gae_run<4, 16, 2>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  // one CTA of 1,024 threads fills an SM: beyond one per SM, CTAs of 512 (800
-  // steps of 7,766 envs: 32.8 against 41.2 us)
   int dev = 0, sms = 0;
   PE_TRY_CUDA(cudaGetDevice(&dev));
   PE_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  // The streaming kernels by what the SMs hold at once: with 32 steps in flight
+  // 512 envs per SM, with 16 steps 1,024; a partly filled second wave costs more
+  // than the shallower ring.  Measured on 152 SMs, with 54M env-steps: 56,000
+  // envs 169 us (16 steps: 183), 85,000 envs 180 (32 steps: 199), 150,000 envs
+  // 175 (181), 262,144 envs 171.
+  // Blocks of 64 spread more evenly over the SMs (42,000 envs: 193 against 201
+  // us); where a row does not start on a 16-byte boundary, neighbouring blocks
+  // share more lines (49,151 envs: 201 against 195).
+  if (E > 920 * sms) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E > 400 * sms) return gae_stream_run<16, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E > 250 * sms && E % 4 == 0) return gae_stream_run<32, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E >= 32768) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  // The chunked kernels while their CTAs fit the SMs at once (one of 1,024
+  // threads per 32 envs, two of 512 per 32 or 64 envs); beyond that the
+  // streaming kernel with 64 steps in flight.  2,048 steps of 10,000 envs: 140
+  // us (179 with CTAs of 32 envs), of 20,000 envs 181 (281 with CTAs of 64).
+  if (E > 128 * sms || (E > 64 * sms && !al2))
+    return gae_stream_run<64, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (n >= ((int64_t)1 << 28) && al4) return gae_run<4, 8, 4>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E > 64 * sms) return gae_run<4, 16, 2>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (E > 32 * sms) return gae_run<8, 16, 1>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   return gae_run<8, 32, 1>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
 }

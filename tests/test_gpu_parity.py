@@ -71,6 +71,32 @@ def test_gae_parity(T, E):
     assert rel_err(cpu(ret), rr) <= TOL
 
 
+@pytest.mark.parametrize("T", [1, 70, 130])
+@pytest.mark.parametrize("per_sm,extra", [(32, 0), (32, 1), (64, 0), (64, 1), (64, 2), (128, 0), (128, 1), (128, 2),
+                                          (250, 0), (250, 4), (400, 0), (400, 1), (920, 0), (920, 1)])
+def test_gae_parity_batch_widths(per_sm, extra, T):
+    """Both sides of the widths at which another kernel takes over (envs per
+    SM: one chunked CTA, two, two of 64 envs, then the streaming kernels, of
+    64, 32, 16 and 32 steps in flight), odd widths included, with horizons
+    shorter than the load ring and ending inside its second or third turn."""
+    E = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    g = torch.Generator(device="cuda").manual_seed(E + T)
+    r = torch.randn(T, E, device="cuda", generator=g)
+    v = torch.randn(T, E, device="cuda", generator=g)
+    d = (torch.rand(T, E, device="cuda", generator=g) < 0.02).to(torch.uint8)
+    lv = torch.randn(E, device="cuda", generator=g)
+    adv = torch.full((T, E), 7e7, device="cuda")
+    ret = torch.full((T, E), 7e7, device="cuda")
+    pe.gae(r, v, d, lv, 0.99, 0.95, adv, ret)
+    cols = np.unique(np.concatenate([[0, 31, 32, 63, 64, E - 65, E - 33, E - 2, E - 1],
+                                     np.random.default_rng(T).choice(E, 40, replace=False)]))
+    ci = torch.from_numpy(cols).cuda()
+    ra, rr = O.gae(cpu(r[:, ci]), cpu(v[:, ci]), cpu(d[:, ci]), cpu(lv[ci]), 0.99, 0.95)
+    assert rel_err(cpu(adv[:, ci]), ra) <= TOL
+    assert rel_err(cpu(ret[:, ci]), rr) <= TOL
+    assert float(adv.abs().max()) < 1e6 and float(ret.abs().max()) < 1e6
+
+
 @pytest.mark.parametrize("T,E", [(64, 16384), (2048, 131072), (1024, 65536), (37, 32771), (300, 131074),
                                  (5, 262144)])
 def test_gae_parity_vector_paths(T, E):
