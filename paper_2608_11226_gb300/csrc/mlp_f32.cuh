@@ -39,6 +39,7 @@ __host__ __device__ __forceinline__ MlpLayout mlp_layout(int D, int H, int A) {
 // alone put a warp's stores into one bank.)
 __device__ __forceinline__ void load_transposed(const float* __restrict__ W, float* dst, int N, int K) {
   const int lane = threadIdx.x & 31, nt = N / 8;
+#pragma unroll 8
   for (int t = threadIdx.x >> 5; t < nt * (K / 4); t += blockDim.x >> 5) {
     const int n = (t % nt) * 8 + (lane & 7), k = (t / nt) * 4 + (lane >> 3);
     dst[k * N + n] = __ldg(W + (int64_t)n * K + k);

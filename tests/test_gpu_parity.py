@@ -604,6 +604,21 @@ def test_rollout_parity_stress_full_size_sampled():
     _rollout_case(wl, 2048, iters=1, sample_envs=ids)
 
 
+@pytest.mark.parametrize("D,H,A", [(8, 64, 3), (16, 128, 5)])
+def test_value_fp32_row_tiles(D, H, A):
+    """The fp32 value network's row tile follows the batch (16, 32 or 64 rows):
+    both sides of each limit, one row, and a last tile of one row."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    net = W.NetSpec(D, H, A, pe.PE_F32)
+    params = W.init_params(net, seed=6, bias_scale=0.1)
+    for n in (1, 17, 32 * sms, 32 * sms + 1, 64 * sms, 64 * sms + 1):
+        obs = torch.randn(n, D, generator=torch.Generator().manual_seed(n))
+        out = torch.full((n,), 7e7, device="cuda")
+        pe.value(net, torch.from_numpy(params).cuda(), obs.cuda(), out)
+        _, ov = O.mlp_forward(net, params, obs.numpy())
+        assert rel_err(cpu(out), ov) <= TOL, n
+
+
 def test_value_bf16_stress_ragged():
     net = W.NetSpec(64, 512, 16, pe.PE_BF16)
     params = W.init_params(net, seed=6, bias_scale=0.1)
