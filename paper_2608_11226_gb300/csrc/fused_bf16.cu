@@ -331,14 +331,16 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
     // hidden layer: tanh(acc + bias) -> bf16 -> act[sl]
     auto hidden = [&](int sl, const float* bias) {
       const int c0 = slice * (H / 4);
+      uint32_t least[NJ];
       tc::tmem_chunks<NJ>(lane_base + (uint32_t)(sl * 256 + c0), [&](int j, const float (&v)[16]) {
         const int c = c0 + j * 16;
         uint32_t pk[8];
-        tc::tanh_bf16(v, bias + c, pk);
+        tc::tanh_bf16(v, bias + c, pk, least[j]);
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
         *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
       });
+      tc::tanh_exact<kTcRows>(least, lane_base + (uint32_t)(sl * 256 + c0), bias, s.act[sl], quad * 32, c0);
     };
     // head: the PPO loss per row, dz to its tile image and to the slot's
     // shared dz tile (zeros for a slot without a tile); slot s by the four

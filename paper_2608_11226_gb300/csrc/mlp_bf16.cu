@@ -397,12 +397,14 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     // thread's row, 16 columns at a time, each chunk's accumulators loaded while
     // the one before is computed; done(j, c, packed bf16) takes them
     auto half = [&](int c0, const float* bias, auto done) {
+      uint32_t least[NJ];
       tc::tmem_chunks<NJ>(lane_addr + (uint32_t)c0, [&](int j, const float (&v)[16]) {
         const int c = c0 + j * 16;
         uint32_t pk[8];
-        tc::tanh_bf16(v, bias + c, pk);
+        tc::tanh_bf16(v, bias + c, pk, least[j]);
         done(j, c, pk);
       });
+      tc::tanh_exact<kTcRows>(least, lane_addr + (uint32_t)c0, bias, s.act, quad * 32, c0);
     };
     // ... into the activation buffer (the next A operand)
     auto put = [&](int c, const uint32_t (&pk)[8]) {
@@ -772,14 +774,16 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     // hidden layer epilogue of slot sl: tanh(acc + bias) -> bf16 -> act[sl]
     auto hidden = [&](int sl, const float* bias) {
       const int c0 = slice * (H / 4);
+      uint32_t least[H / 64];
       tc::tmem_chunks<H / 64>(lane_base + (uint32_t)(sl * 256 + c0), [&](int j, const float (&v)[16]) {
         const int c = c0 + j * 16;
         uint32_t pk[8];
-        tc::tanh_bf16(v, bias + c, pk);
+        tc::tanh_bf16(v, bias + c, pk, least[j]);
         const uint32_t o0 = tc::swz_offset<128>(row, c, kTcRows), o1 = tc::swz_offset<128>(row, c + 8, kTcRows);
         *reinterpret_cast<uint4*>(s.act[sl] + o0) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
         *reinterpret_cast<uint4*>(s.act[sl] + o1) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
       });
+      tc::tanh_exact<kTcRows>(least, lane_base + (uint32_t)(sl * 256 + c0), bias, s.act[sl], quad * 32, c0);
     };
     auto handover = [&](uint64_t* bar) {
       tc::fence_async_smem();

@@ -271,19 +271,21 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* b) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
 }
 
-// tanh of a pair of fp32 pre-activations whose results are rounded to bf16:
-// x P(x^2) / Q(x^2) with P and Q cubic, fitted to tanh on |x| <= 3.5 by
-// weighted least squares (relative error of the fit 1.8e-9; of the fp32
-// evaluation at most 2.8e-7 and 6e-8 rms over [1e-6, 3.5], as tanhf's).  The
-// argument is clamped to +-3.5 first: tanh(3.5) = 0.99818 lies above the
-// midpoint 0.99805 between the two largest bf16 values below and at one, so
-// every |x| >= 3.5 rounds to +-1 as tanh does; infinities clamp and NaN
-// passes.  Nine packed or plain FMA-pipe operations, a reciprocal and a clamp
-// per value, without a branch, where tanhf takes about 18 issue slots and
-// both sides of its branch: the hidden epilogues are bound by instruction
-// issue.  Measured with tanhf and with this: a 72B rollout of 65,536 envs x 64
-// steps 4.91 and 4.18 ms, a Stress rollout of 262,144 x 8 5.44 and 4.56 ms.
-__device__ __forceinline__ float2 tanh2_for_bf16(float2 x) {
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// tanh of a pair of fp32 pre-activations to within kTanhUlps fp32 steps of
+// tanhf: x P(x^2) / Q(x^2) with P and Q cubic, fitted to tanh on |x| <= 3.5 by
+// weighted least squares.  The argument is clamped to +-3.5 first: tanh(3.5) =
+// 0.99818 lies above the midpoint 0.99805 between the two largest bf16 values
+// below and at one, so every |x| >= 3.5 rounds to +-1 as tanhf's result does;
+// infinities clamp and NaN passes.  Over all 1.08e9 floats in [0, 3.5) it
+// equals tanhf for 94%, differs by one step for 5%, by more than three for 16
+// in a million, by kTanhUlps at most.
+constexpr int kTanhUlps = 5;
+__device__ __forceinline__ float2 tanh2_rational(float2 x) {
   asm("min.NaN.xorsign.abs.f32 %0, %0, 0f40600000;" : "+f"(x.x));  // 3.5 with x's sign
   asm("min.NaN.xorsign.abs.f32 %0, %0, 0f40600000;" : "+f"(x.y));
   const float2 s = __fmul2_rn(x, x);
@@ -300,25 +302,73 @@ __device__ __forceinline__ float2 tanh2_for_bf16(float2 x) {
   return __fmul2_rn(__fmul2_rn(x, p), r);
 }
 
-// tanh of N hidden pre-activations (v + bias, one TMEM chunk of a thread's
-// row; bias 16-byte aligned), rounded to bf16 and packed in pairs; the bias is
-// added with the packed two-lane fp32 add (the same rounding as two adds).
+// tanh(v + bias) of N hidden pre-activations (one TMEM chunk of a thread's row;
+// bias 16-byte aligned), rounded to bf16 and packed in pairs; the bias is added
+// with the packed two-lane fp32 add (the same rounding as two adds).  A result
+// can differ from bf16(tanhf(v + bias)) only where its fp32 value lies within
+// kTanhUlps steps of a midpoint between two bf16 values, low half 0x8000 +-
+// kTanhUlps: 11 of 65,536.  `least` takes the least of (low half - 0x8000 +
+// kTanhUlps) mod 2^16 of the even and of the odd columns; tanh_exact settles
+// the chunks where one is at most 2 kTanhUlps.
 template <int N>
-__device__ __forceinline__ void tanh_bf16(const float (&v)[N], const float* bias, uint32_t (&pk)[N / 2]) {
+__device__ __forceinline__ void tanh_bf16(const float (&v)[N], const float* bias, uint32_t (&pk)[N / 2],
+                                          uint32_t& least) {
+  constexpr uint32_t kShift = (0x8000u + kTanhUlps) * 0x10001u;
+  least = 0xFFFFFFFFu;
 #pragma unroll
   for (int i = 0; i < N; i += 4) {
     const float4 b = *reinterpret_cast<const float4*>(bias + i);
-    const float2 t = tanh2_for_bf16(__fadd2_rn(make_float2(v[i], v[i + 1]), make_float2(b.x, b.y)));
-    const float2 u = tanh2_for_bf16(__fadd2_rn(make_float2(v[i + 2], v[i + 3]), make_float2(b.z, b.w)));
-    __nv_bfloat162 r = __floats2bfloat162_rn(t.x, t.y), q = __floats2bfloat162_rn(u.x, u.y);
-    pk[i / 2] = *reinterpret_cast<uint32_t*>(&r);
-    pk[i / 2 + 1] = *reinterpret_cast<uint32_t*>(&q);
+    const float2 t = tanh2_rational(__fadd2_rn(make_float2(v[i], v[i + 1]), make_float2(b.x, b.y)));
+    const float2 u = tanh2_rational(__fadd2_rn(make_float2(v[i + 2], v[i + 3]), make_float2(b.z, b.w)));
+    pk[i / 2] = pack_bf16(t.x, t.y);
+    pk[i / 2 + 1] = pack_bf16(u.x, u.y);
+    least = __viaddmin_u16x2(__byte_perm(__float_as_uint(t.x), __float_as_uint(t.y), 0x5410), kShift, least);
+    least = __viaddmin_u16x2(__byte_perm(__float_as_uint(u.x), __float_as_uint(u.y), 0x5410), kShift, least);
   }
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&v);
+__device__ __forceinline__ bool near_midpoint(uint32_t least) {
+  return min(least & 0xFFFFu, least >> 16) <= 2 * kTanhUlps;
+}
+
+// Makes the activations of a warp's 32 rows (from row0 on; NJ chunks of 16
+// accumulators from taddr, columns from c0 on) in the K-major buffer `act` those
+// of tanhf; least[j]: tanh_bf16's of the thread's chunk j.  8% of a warp's chunks
+// need it, and all warps of a tile wait for the last one, so the latency of a
+// pass and the code it fetches count: two rows of a chunk at a time, a lane per
+// column, in one loop for all chunks.  A 72B rollout of 65,536 envs x 64 steps
+// takes 3.79 ms, a Stress rollout of 262,144 x 8 4.23 ms; with tanhf for every
+// value, about 18 issue slots and both sides of its branch, 4.20 and 4.63; with
+// the rational alone, whose results are not tanhf's, 3.36 and 3.76.  (Settling
+// each chunk before the next, 4.05 and 4.51.)
+template <int R, int NJ>
+__device__ __forceinline__ void tanh_exact(const uint32_t (&least)[NJ], uint32_t taddr, const float* bias, uint8_t* act,
+                                           int row0, int c0) {
+  uint32_t m = least[0];
+#pragma unroll
+  for (int j = 1; j < NJ; ++j) m = __vminu2(m, least[j]);
+  if (!__any_sync(0xffffffffu, near_midpoint(m))) return;
+  const int lane = threadIdx.x & 31;
+  uint32_t near = 0;  // the thread's chunks to settle
+#pragma unroll
+  for (int j = 0; j < NJ; ++j) near |= near_midpoint(least[j]) ? 1u << j : 0u;
+  while (const uint32_t any = __ballot_sync(0xffffffffu, near != 0)) {
+    const int j = __ffs(__shfl_sync(0xffffffffu, near, __ffs(any) - 1)) - 1;
+    const uint32_t rows = __ballot_sync(0xffffffffu, (near >> j) & 1u), rest = rows & (rows - 1);
+    const int ra = __ffs(rows) - 1, rb = rest ? __ffs(rest) - 1 : ra;
+    const int r = lane < 16 ? ra : rb, c = c0 + 16 * j + (lane & 15);
+    float v[16], z = 0.0f;
+    tmem_ld16(taddr + (uint32_t)(16 * j), v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float x = __shfl_sync(0xffffffffu, v[i], r);
+      if ((lane & 15) == i) z = x;
+    }
+    const __nv_bfloat16 h = __float2bfloat16_rn(tanhf(z + bias[c]));
+    __syncwarp();  // after the rows' own stores
+    *reinterpret_cast<__nv_bfloat16*>(act + swz_offset<128>(row0 + r, c, R)) = h;
+    if (lane == ra || lane == rb) near &= ~(1u << j);
+  }
 }
 
 }  // namespace tc

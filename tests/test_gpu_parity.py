@@ -647,9 +647,10 @@ def test_value_bf16_parity_ragged():
 def test_bf16_tanh_pointwise(D, H):
     """The hidden layers' tanh at chosen arguments: one-hot observations
     saturate one hidden unit of layer 1 to exactly 1, so that unit 0 of layer
-    2 sees W2[0][d] + b2[0] and the head returns its bf16 activation.  The fp32
-    value is within 3e-7 (relative) of tanh, so after rounding it may differ
-    only next to a rounding midpoint, by one bf16 step; +-inf gives +-1 and
+    2 sees W2[0][d] + b2[0] and the head returns its bf16 activation, tanhf
+    rounded to bf16.  tanhf lies within two fp32 steps of tanh, so of 65,536
+    results about four may differ from tanh rounded to bf16, by one bf16 step (0.02
+    of the 384 here; tests/test_gpu_tanh.py has every argument); +-inf gives +-1 and
     NaN stays NaN."""
     net = W.NetSpec(D, H, 16, pe.PE_BF16)
     pol = H * D + H + H * H + H + 16 * H + 16
@@ -675,7 +676,7 @@ def test_bf16_tanh_pointwise(D, H):
         step = np.maximum(np.abs(want), 1e-37) * 2.0 ** -7
         assert np.all(np.abs(got - want) <= step), (call, got, want)
         seen, off = seen + 32, off + int((got != want).sum())
-    assert off <= seen // 50, (off, seen)
+    assert off <= 1, (off, seen)
     for b2, want in ((np.inf, 1.0), (-np.inf, -1.0), (np.nan, np.nan)):
         p[o + H * H] = b2
         pe.value(net, torch.from_numpy(p).cuda(), obs, out)
