@@ -39,7 +39,7 @@ struct LossIn {
 };
 
 __device__ __forceinline__ uint32_t loss_index(const uint32_t* gather, int64_t j, int64_t n) {
-  return j < n ? __ldg(gather + j) : 0u;
+  return j < n ? __ldcg(gather + j) : 0u;
 }
 
 __device__ __forceinline__ LossIn loss_inputs(const PpoHead& L, int value_net, uint32_t i) {

@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
     };
     uint4 dzv = make_uint4(0, 0, 0, 0);
     if (tid < kBwRows * 2 && my_tiles > 0)
-      dzv = __ldg(reinterpret_cast<const uint4*>((ni0 ? g.dz[1] : g.dz[0]) + tile_of(0, ni0) * (kBwRows * 32)) + tid);
+      dzv = __ldcg(reinterpret_cast<const uint4*>((ni0 ? g.dz[1] : g.dz[0]) + tile_of(0, ni0) * (kBwRows * 32)) + tid);
     for (int t = 0; t < my_tiles; ++t) {
       const uint32_t par = t & 1;
       int ni, nn = 0;
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
       if (tid < kBwRows * 2) {
         reinterpret_cast<uint4*>(s.dz)[tid] = dzv;
         if (t + 1 < my_tiles)
-          dzv = __ldg(reinterpret_cast<const uint4*>((nn ? g.dz[1] : g.dz[0]) + ntile * (kBwRows * 32)) + tid);
+          dzv = __ldcg(reinterpret_cast<const uint4*>((nn ? g.dz[1] : g.dz[0]) + ntile * (kBwRows * 32)) + tid);
       }
       handover(&s.dzin);
       // da2 = bf16(dh2 (1 - h2^2)) per half, in place over h2 (the next A operand)
@@ -674,9 +674,9 @@ static_assert(WgReduce<512>::BLOCKS == kWgReduceBlocks && kWgReduceBlocks * WgRe
 constexpr int kLossPartW = 32;  // loss-kernel partial row: pg, ent, kl, clip, vl, db3[16], dc3
 
 template <int D, int H>
-__global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const float* __restrict__ part, int S0, int S1,
+__global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const float* part, int S0, int S1,
                                                            int A,
-                                                           float* __restrict__ grad, const float* __restrict__ lossp,
+                                                           float* __restrict__ grad, const float* lossp,
                                                            int nlb, double* __restrict__ stat5,
                                                            float* __restrict__ sq) {
   using Cn = WgCols<D>;
@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const
     const int col = w < 5 ? w : (w - 5 < A ? 5 + (w - 5) : 21);
     double t = 0.0;
 #pragma unroll 4
-    for (int b = threadIdx.x; b < nlb; b += blockDim.x) t += (double)lossp[(int64_t)b * kLossPartW + col];
+    for (int b = threadIdx.x; b < nlb; b += blockDim.x) t += (double)__ldcg(lossp + (int64_t)b * kLossPartW + col);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     if (lane == 0) redd[warp] = t;
@@ -815,7 +815,8 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     return fail(PE_EINVAL, "the 72B data products run in the fused forward-backward kernel");
   } else {
     auto kern = bwd_data_kernel<H>;
-    const int bytes = (int)sizeof(BwdSmem<H>) + 1024;
+    constexpr int bytes = (int)sizeof(BwdSmem<H>) + 1024;
+    static_assert(bytes > kPdlTmemSmem, "one CTA per SM");
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     const int grid = (int)std::min<int64_t>(2 * tiles, sms);
     BwdArgs a;
@@ -867,7 +868,7 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     a.err = err;
     auto kern = wgrad_kernel<D, H>;
     constexpr int bytes = (int)sizeof(WgSmem) + 1024;
-    static_assert(bytes <= 232448, "weight-gradient shared memory");
+    static_assert(bytes <= 232448 && bytes > kPdlTmemSmem, "weight-gradient shared memory: one CTA per SM");
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     ProfScope ps(PE_PROF_PPO_GRAD, st);
     PE_TRY_CUDA(launch_pdl(kern, ctas, kWgThreads, bytes, st, true, a));

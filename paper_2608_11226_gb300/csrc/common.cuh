@@ -172,6 +172,17 @@ inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 // that an earlier kernel writes or reads may be touched before.  pdl_enter
 // then lets the next kernel start in turn: a kernel begins at the earliest
 // when the one before last is complete.
+// What the kernels of a step write for one another (parameters, gather
+// indices, dz, partial sums) is written within the lifetime of the kernel that
+// reads it, so it is not read-only there: it is loaded behind pdl_enter with
+// coherent loads (__ldcg or plain ones), through pointers without const
+// __restrict__.  __ldg and const __restrict__, which allow a load ahead of
+// pdl_enter and a stale line of the L1, are for what no kernel of the step
+// writes: obs, act, logp, adv, ret and the advantage statistics.
+// A kernel that allocates tensor memory may let the next one start before its
+// own allocation is through; the next one cannot take the memory from it, for
+// two such kernels need more shared memory than an SM has (a static_assert at
+// each launch: above half).
 // Used between the five kernels of a bf16 update step, where the launch gaps
 // and prologues were 3% of a 72B update (5.91 to 5.74 ms) and 1.6% of a Stress
 // update (6.68 to 6.58 ms).
@@ -179,6 +190,8 @@ __device__ __forceinline__ void pdl_enter() {
   cudaGridDependencySynchronize();
   cudaTriggerProgrammaticLaunchCompletion();
 }
+
+constexpr int kPdlTmemSmem = 116 * 1024;  // dynamic shared memory of a launch_pdl kernel with tensor memory: above this
 
 template <class... P, class... A>
 inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool early,

@@ -120,10 +120,10 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
   if (warp == 0) tc::tmem_alloc(&s.tmem_base, 512);
   pdl_enter();
   for (int i = tid; i < H; i += blockDim.x) {
-    s.b1[i] = __ldg(args.params + (value_net ? Lp.c1 : Lp.b1) + i);
-    s.b2[i] = __ldg(args.params + (value_net ? Lp.c2 : Lp.b2) + i);
+    s.b1[i] = __ldcg(args.params + (value_net ? Lp.c1 : Lp.b1) + i);
+    s.b2[i] = __ldcg(args.params + (value_net ? Lp.c2 : Lp.b2) + i);
   }
-  if (tid < kHeadN) s.b3[tid] = tid < nout ? __ldg(args.params + (value_net ? Lp.c3 : Lp.b3) + tid) : 0.0f;
+  if (tid < kHeadN) s.b3[tid] = tid < nout ? __ldcg(args.params + (value_net ? Lp.c3 : Lp.b3) + tid) : 0.0f;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kFuThreads, 1) ppo_fused_pair_kernel(const __g
         const int64_t rr = tl * kTcRows + r;
         dst[q] = make_uint4(0, 0, 0, 0);
         if (k < my_tiles && rr < args.n) {
-          const int64_t src = g.save.gather ? (int64_t)__ldg(g.save.gather + rr) : rr;
+          const int64_t src = g.save.gather ? (int64_t)__ldcg(g.save.gather + rr) : rr;
           dst[q] = __ldg(reinterpret_cast<const uint4*>(args.obs + src * D) + c);
         }
       }
@@ -500,7 +500,7 @@ pe_status bf16_fused_fwd_bwd(const pe_net& net, const uint8_t* const img[2], con
   const int per_net = (int)std::min<int64_t>((tiles + 1) / 2, std::max(1, sms / 2));
   auto kern = ppo_fused_pair_kernel<32, 256>;
   constexpr int bytes = (int)sizeof(FusedSmem<32, 256>) + 1024;
-  static_assert(bytes <= 232448, "fused kernel shared memory");
+  static_assert(bytes <= 232448 && bytes > kPdlTmemSmem, "fused kernel shared memory: one CTA per SM");
   PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   FusedArgs a;
   for (int ni = 0; ni < 2; ++ni)

@@ -157,7 +157,7 @@ struct MlpStreamSmem {
 
 template <int D, int H>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-    mlp_bf16_stream_kernel(const uint8_t* __restrict__ img, const float* __restrict__ params, int A,
+    mlp_bf16_stream_kernel(const uint8_t* img, const float* params, int A,
                            int value_net, const __nv_bfloat16* __restrict__ obs, int64_t n,
                            float* __restrict__ out, int out_stride, int nout, int32_t* __restrict__ err,
                            MlpSave save, MlpSecond second) {
@@ -204,10 +204,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     const int vn = two ? k : value_net;
     const int no = two ? (k ? 1 : A) : nout;
     for (int i = tid; i < H; i += blockDim.x) {
-      s.b1[k][i] = __ldg(params + (vn ? Lp.c1 : Lp.b1) + i);
-      s.b2[k][i] = __ldg(params + (vn ? Lp.c2 : Lp.b2) + i);
+      s.b1[k][i] = __ldcg(params + (vn ? Lp.c1 : Lp.b1) + i);
+      s.b2[k][i] = __ldcg(params + (vn ? Lp.c2 : Lp.b2) + i);
     }
-    if (tid < kHeadN) s.b3[k][tid] = tid < no ? __ldg(params + (vn ? Lp.c3 : Lp.b3) + tid) : 0.0f;
+    if (tid < kHeadN) s.b3[k][tid] = tid < no ? __ldcg(params + (vn ? Lp.c3 : Lp.b3) + tid) : 0.0f;
   }
   tc::fence_before();
   __syncthreads();
@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
         const int64_t rr = tl * kTcRows + r;
         xv[q] = make_uint4(0, 0, 0, 0);
         if (k < my_tiles && i < kTcRows * XCPR && rr < n) {
-          const int64_t src = gather ? (int64_t)__ldg(gather + rr) : rr;
+          const int64_t src = gather ? (int64_t)__ldcg(gather + rr) : rr;
           xv[q] = __ldg(reinterpret_cast<const uint4*>(obs + src * D) + c);
         }
       }
@@ -983,7 +983,8 @@ static pe_status launch_mlp(const uint8_t* img, const float* params, int A, int 
     const int64_t all = second.img ? 2 * tiles : tiles;
     const int grid = (int)(all < sms ? all : sms);
     auto kern = mlp_bf16_stream_kernel<D, H>;
-    const int bytes = (int)sizeof(MlpStreamSmem<D, H>) + 1024;
+    constexpr int bytes = (int)sizeof(MlpStreamSmem<D, H>) + 1024;
+    static_assert(bytes > kPdlTmemSmem, "one CTA per SM");
     PE_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
     ProfScope ps(prof_kind, st);
     // early in an update's chain of kernels; a rollout's policy launches gain

@@ -1033,6 +1033,33 @@ def test_ppo_bf16_ragged_epochs(preset, E, mb, clip):
         assert st[4] > 0.05
 
 
+@pytest.mark.parametrize("preset,E", [("72b", 64), ("stress", 32)])
+def test_ppo_bf16_params_at_any_offset(preset, E):
+    """Two epochs of three minibatches with the parameters and moments as views
+    that start 1, 3 and 5 floats into their storage: sectors and cache lines
+    then straddle the Adam blocks that write them and the kernels that read
+    them next, and every output keeps the bits of the aligned run."""
+    T = 64
+    wl = W.make_72b(n_envs=E) if preset == "72b" else W.make_stress(n_envs=E, horizon=T)
+    params, buf, adv, ret = _ppo_inputs(wl, T, seed=4)
+    ppo = W.PPOSpec(epochs=2, minibatch=T * E // 3 + 1, ent_coef=0.01)
+    want = None
+    for off in (0, 1, 3, 5):
+        p, m, v = (torch.zeros(params.size + off, device="cuda")[off:] for _ in range(3))
+        p.copy_(torch.from_numpy(params))
+        stats = torch.zeros(8, device="cuda")
+        ws = torch.empty(pe.ppo_workspace_bytes(wl.net, ppo, T * E), dtype=torch.uint8, device="cuda")
+        pe.ppo_update(wl.net, ppo, p, m, v, 0, buf["obs"], buf["act"], buf["logp"], adv, ret, stats, ws,
+                      seed=7, iteration=3)
+        torch.cuda.synchronize()
+        got = (p, m, v, stats)
+        if want is None:
+            want = got
+            assert float(stats[7]) == 6 and not torch.equal(p, torch.from_numpy(params).cuda())
+        for g, w in zip(got, want):
+            assert torch.equal(g, w), off
+
+
 # ------------------------------------------------------- baseline rule policies
 def _rule_for(kind, preset, B):
     if kind == 1:
