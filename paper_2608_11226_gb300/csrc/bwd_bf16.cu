@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(kBwThreads, 1) bwd_data_kernel(BwdArgs g) {
 // weight gradients: split over samples, 32 samples per stage
 // ---------------------------------------------------------------------------
 constexpr int kWgSamples = 32;
+constexpr int kWgUnit = 64;  // samples that a CTA's share is a multiple of (it fixes the sums' order)
 constexpr int kWgThreads = 128;
 // stage layout (bytes): A da2 | A da1 | A h2 (each 2 blocks of 64 features x
 // 32 samples), B h1 (4 blocks: 256 columns), B x (32 samples x D), B dz; the
@@ -642,112 +643,43 @@ __global__ void __launch_bounds__(kWgThreads, 1) wgrad_kernel(WgArgs g) {
   if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
-// The rest of the minibatch gradient and its squared norm, in one launch (all
-// orders fixed, so the result is deterministic):
+// The rest of the minibatch gradient and its squared norm, in one launch of
+// kWgReduceBlocks blocks (all orders fixed, so the result is deterministic):
 //   - every weight and hidden-bias entry: the sum over the S sample chunks of
-//     its partial blocks.  A thread takes four adjacent columns of one partial
-//     block row and one in KS of the chunks, in order; the KS sums are then
-//     added in order.  KS is 4 for the 72B networks (38 chunks, 512 rows) and
-//     1 for Stress (11 and 8 chunks, 2048 rows): either way one wave of
-//     kWgReduceBlocks blocks, each thread with at most a dozen 16-byte loads,
-//     four in flight.  The launch is bound by that latency: with one column
-//     per thread, up to 38 loads in a row and 1.3 waves, it took 20.0 us (72B)
-//     and 23.3 us (Stress); it takes 9.2 and 9.1.
-//   - kWgLossBlocks more blocks sum the loss partial rows, one quantity per
+//     its partial blocks, in chunk order;
+//   - blocks 0 .. 5 + A also sum the loss partial rows, one quantity per
 //     block (the five minibatch statistics, then the head-bias gradients
 //     from the unrounded dz): thread t takes rows t, t + 512, ... in order,
 //     then a fixed shuffle tree and the warps in order;
 //   - each block writes the fp32 sum of squares of the entries it wrote
-//     (threads in order of a fixed tree), the Adam kernel sums the blocks.
+//     (a thread's entries in order, then a fixed tree), the Adam kernel sums
+//     the blocks.
+// A thread takes one entry in 131,072.  What bounds the launch is the latency
+// of its loads, so two entries and kWgReduceDepth of their chunks are in flight
+// at a time: 11.3 us (72B: 38 chunks, 188,416 entries) and 12.4 us (Stress: 11
+// and 8 chunks, 753,664 entries) per step, with one entry and eight loads in
+// flight 20.0 and 23.3.  (Four columns per 16-byte load and the 72B chunks dealt
+// out to four threads took 9.2 and 9.1, but added in another order.)
+constexpr int kWgReduceBlocks = 256;
 constexpr int kWgReduceThreads = 512;
-constexpr int kWgQuads = kWgMaxCols / 4;  // column quads per partial-block row
-template <int H>
-struct WgReduce {
-  static constexpr int KS = H == 256 ? 4 : 1;
-  static constexpr int QB = kWgReduceThreads / KS;  // quads per block
-  static constexpr int BLOCKS = 2 * (H / 128) * (H / 256) * 128 * kWgQuads / QB;
-};
-constexpr int kWgReduceBlocks = WgReduce<256>::BLOCKS;
-constexpr int kWgLossBlocks = 22;  // 5 statistics, up to 16 policy head biases, the value's
-static_assert(WgReduce<512>::BLOCKS == kWgReduceBlocks && kWgReduceBlocks * WgReduce<256>::QB == 512 * kWgQuads,
-              "one quad per thread group");
+constexpr int kWgReduceDepth = 10;
 constexpr int kLossPartW = 32;  // loss-kernel partial row: pg, ent, kl, clip, vl, db3[16], dc3
 
 template <int D, int H>
-__global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const float* part, int S0, int S1,
-                                                           int A,
-                                                           float* __restrict__ grad, const float* lossp,
-                                                           int nlb, double* __restrict__ stat5,
-                                                           float* __restrict__ sq) {
+__global__ void __launch_bounds__(kWgReduceThreads, 2) wgrad_reduce_kernel(const float* part, int S0, int S1, int A,
+                                                           float* __restrict__ grad, const float* lossp, int nlb,
+                                                           double* __restrict__ stat5, float* __restrict__ sq) {
   using Cn = WgCols<D>;
-  using R = WgReduce<H>;
-  constexpr int NCH = H / 256, MB = H / 128;
+  constexpr int NCH = H / 256, MB = H / 128, U = 2, KB = kWgReduceDepth;
+  constexpr int kTotal = 2 * MB * NCH * 128 * kWgMaxCols, kStep = kWgReduceBlocks * kWgReduceThreads;
   __shared__ float red[kWgReduceThreads / 32];
+  __shared__ double redd[kWgReduceThreads / 32];
   pdl_enter();
   const MlpLayout Lp = mlp_layout(D, H, A);
-  float q = 0.0f;
-  if (blockIdx.x < kWgReduceBlocks) {
-    __shared__ float4 ksum[R::KS][R::KS > 1 ? R::QB : 1];
-    const int tq = threadIdx.x % R::QB, kp = threadIdx.x / R::QB;
-    const int i = (int)blockIdx.x * R::QB + tq;
-    const int col = i % kWgQuads * 4, row = i / kWgQuads % 128, grp = i / (kWgQuads * 128);
-    const int ni = grp / (MB * NCH), mb = (grp / NCH) % MB, nc = grp % NCH;
-    const int o = mb * 128 + row, nout = ni ? 1 : A;
-    // the quad's entries: the first one's place, their stride and their count
-    // (every product's columns start at a multiple of 16)
-    int64_t dst = 0;
-    int step = 1, m = 0;
-    if (col < 256) {
-      dst = (ni ? Lp.v2 : Lp.w2) + (int64_t)o * H + nc * 256 + col, m = 4;
-    } else if (nc == 0) {
-      if (col == Cn::DB2) dst = (ni ? Lp.c2 : Lp.b2) + o, m = 1;
-      else if (col >= Cn::DW1 && col < Cn::DW1 + D) dst = (ni ? Lp.v1 : Lp.w1) + (int64_t)o * D + (col - Cn::DW1), m = 4;
-      else if (col == Cn::DB1) dst = (ni ? Lp.c1 : Lp.b1) + o, m = 1;
-      else if (col >= Cn::DW3 && col < Cn::DW3 + nout)
-        dst = (ni ? Lp.v3 : Lp.w3) + (int64_t)(col - Cn::DW3) * H + o, step = H, m = min(4, Cn::DW3 + nout - col);
-    }
-    float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (m) {
-      const int S[2] = {S0, S1};
-      const int nch = nc ? S1 : S0;
-      const float* p = part + ((int64_t)wg_first_cta<NCH>(grp, S) * 128 + row) * kWgMaxCols + col;
-      for (int k0 = kp; k0 < nch; k0 += 4 * R::KS) {
-        float4 v[4];
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const int k = k0 + b * R::KS;
-          v[b] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-          if (k < nch) v[b] = __ldcg(reinterpret_cast<const float4*>(p + (int64_t)k * 128 * kWgMaxCols));
-        }
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-          acc = make_float4(acc.x + v[b].x, acc.y + v[b].y, acc.z + v[b].z, acc.w + v[b].w);
-      }
-    }
-    if (R::KS > 1) {
-      ksum[kp][tq] = acc;
-      __syncthreads();
-      if (kp == 0)
-#pragma unroll
-        for (int k = 1; k < R::KS; ++k) {
-          const float4 v = ksum[k][tq];
-          acc = make_float4(acc.x + v.x, acc.y + v.y, acc.z + v.z, acc.w + v.w);
-        }
-    }
-    if (kp == 0) {
-      const float a[4] = {acc.x, acc.y, acc.z, acc.w};
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (c < m) {
-          grad[dst + (int64_t)c * step] = a[c];
-          q = fmaf(a[c], a[c], q);
-        }
-    }
-  }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __shared__ double redd[kWgReduceThreads / 32];
-  const int w = (int)blockIdx.x - kWgReduceBlocks;  // statistic w (w < 5), then head-bias sum j = w - 5 (policy j < A, then the value's)
-  if (w >= 0 && w < 5 + A + 1) {
+  float bias = 0.0f;  // thread 0: the block's head-bias entry
+  const int w = (int)blockIdx.x;  // statistic w (w < 5), then head-bias sum j = w - 5 (policy j < A, then the value's)
+  if (w < 5 + A + 1) {
     const int col = w < 5 ? w : (w - 5 < A ? 5 + (w - 5) : 21);
     double t = 0.0;
 #pragma unroll 4
@@ -763,12 +695,59 @@ __global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const
         stat5[w] = u;
       } else {
         const int j = w - 5;
-        const float g = (float)u;
-        grad[j < A ? Lp.b3 + j : Lp.c3] = g;
-        q = fmaf(g, g, q);
+        bias = (float)u;
+        grad[j < A ? Lp.b3 + j : Lp.c3] = bias;
       }
     }
   }
+  const int S[2] = {S0, S1};
+  float q = 0.0f;
+  for (int i0 = (int)blockIdx.x * kWgReduceThreads + (int)threadIdx.x; i0 < kTotal; i0 += U * kStep) {
+    int64_t dst[U];
+    const float* p[U];
+    int n[U];  // chunks to sum (0: no entry)
+    float acc[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = i0 + u * kStep;
+      const int col = i % kWgMaxCols, row = i / kWgMaxCols % 128, grp = i / (kWgMaxCols * 128);
+      const int ni = grp / (MB * NCH), mb = (grp / NCH) % MB, nc = grp % NCH;
+      const int o = mb * 128 + row, nout = ni ? 1 : A;
+      dst[u] = -1;
+      if (col < 256) {
+        dst[u] = (ni ? Lp.v2 : Lp.w2) + (int64_t)o * H + nc * 256 + col;
+      } else if (nc == 0) {
+        if (col == Cn::DB2) dst[u] = (ni ? Lp.c2 : Lp.b2) + o;
+        else if (col >= Cn::DW1 && col < Cn::DW1 + D) dst[u] = (ni ? Lp.v1 : Lp.w1) + (int64_t)o * D + (col - Cn::DW1);
+        else if (col == Cn::DB1) dst[u] = (ni ? Lp.c1 : Lp.b1) + o;
+        else if (col >= Cn::DW3 && col < Cn::DW3 + nout) dst[u] = (ni ? Lp.v3 : Lp.w3) + (int64_t)(col - Cn::DW3) * H + o;
+      }
+      if (i >= kTotal) dst[u] = -1;
+      n[u] = dst[u] < 0 ? 0 : nc ? S1 : S0;
+      p[u] = part;
+      if (n[u]) p[u] += ((int64_t)wg_first_cta<NCH>(grp, S) * 128 + row) * kWgMaxCols + col;
+      acc[u] = 0.0f;
+    }
+    for (int k0 = 0; k0 < max(n[0], n[1]); k0 += KB) {
+      float v[U][KB];
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int b = 0; b < KB; ++b)
+          v[u][b] = k0 + b < n[u] ? __ldcg(p[u] + (int64_t)(k0 + b) * (128 * kWgMaxCols)) : 0.0f;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int b = 0; b < KB; ++b) acc[u] += v[u][b];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (n[u]) {
+        grad[dst[u]] = acc[u];
+        q = fmaf(acc[u], acc[u], q);
+      }
+  }
+  q = fmaf(bias, bias, q);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) q += __shfl_xor_sync(0xffffffffu, q, off);
   if (lane == 0) red[warp] = q;
@@ -780,7 +759,7 @@ __global__ void __launch_bounds__(kWgReduceThreads, 3) wgrad_reduce_kernel(const
   }
 }
 
-int wgrad_reduce_blocks() { return kWgReduceBlocks + kWgLossBlocks; }
+int wgrad_reduce_blocks() { return kWgReduceBlocks; }
 
 // ---------------------------------------------------------------------------
 // host side
@@ -841,6 +820,7 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     a.x = x;
     a.n = n;
     a.nstages = (int)((n + kWgSamples - 1) / kWgSamples);
+    const int units = (int)((n + kWgUnit - 1) / kWgUnit);
     // CTAs per (network, row block), split between the column chunks in
     // proportion to the bytes a stage brings in: chunk 0 also loads da1, h2,
     // x and dz (for the Stress networks 45 KB per stage against 24 KB), so
@@ -858,9 +838,10 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
     for (int c = 0; c < 2; ++c) {
       a.spc[c] = a.S[c] = 0;
       if (c >= NCH) continue;
-      const int s_want = std::max(1, std::min(want[c], a.nstages));
-      a.spc[c] = (a.nstages + s_want - 1) / s_want;
-      a.S[c] = (a.nstages + a.spc[c] - 1) / a.spc[c];
+      const int s_want = std::max(1, std::min(want[c], units));
+      const int per = (units + s_want - 1) / s_want;
+      a.spc[c] = per * (kWgUnit / kWgSamples);
+      a.S[c] = (units + per - 1) / per;
       ctas += a.S[c];
     }
     ctas *= groups / NCH;
@@ -882,7 +863,7 @@ static pe_status bwd_launch(const float* params, int A, uint8_t* const img[2], c
 
 // the whole backward of both networks of a bf16 PPO minibatch step: writes
 // every entry of the gradient vector (the head biases from the loss kernel's
-// partials), the five minibatch statistics, and wgrad_reduce_blocks() partial sums
+// partials), the five minibatch statistics, and kWgReduceBlocks partial sums
 // of squares of the gradient
 pe_status bf16_backward(const pe_net& net, const float* params, uint8_t* const img[2], const uint8_t* x,
                         const uint8_t* const dz[2], const uint8_t* const h1[2], const uint8_t* const h2[2],

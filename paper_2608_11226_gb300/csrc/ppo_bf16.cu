@@ -119,7 +119,7 @@ __global__ void adam_bf16_kernel(AdamBf16Args a) {
   const float coef = fminf(1.0f, a.max_norm / (norm + 1e-6f));
   if (mine) {
     const float gp = g0 * coef;
-    const float mp = a.beta1 * m0 + (1.0f - a.beta1) * gp;
+    const float mp = fmaf(1.0f - a.beta1, gp, a.beta1 * m0);  // spelled out: a compiler may fuse either product
     const float vp = a.beta2 * v0 + (1.0f - a.beta2) * gp * gp;
     a.m[p] = mp;
     a.v[p] = vp;

@@ -62,57 +62,69 @@ __device__ __forceinline__ float block_sum_f(float v, float* red) {
 }
 
 // advantage mean and 1/(std + 1e-8) (unbiased std) of every (minibatch, epoch),
-// two passes by a cluster of CTAs each: thread t of CTA r takes the positions
-// t + 512 (r + CL i), the cluster's sums are added in CTA order.  A position
-// costs its permutation (a serial chain of integer operations) and a gather
-// from L2, so the launch is bound by the longest thread: the
-// first kAdvKeep values stay in registers for the second pass, and CL (a power
-// of two up to 8, the portable limit) is the least that gives a thread at most
-// 8 values, as long as that is met.  With one CTA of 1024 per minibatch and
-// both passes gathered, the 32 of a 72B update took 263 us and now 42; the
-// 7B update's went from 80 to 16.
-constexpr int kAdvNT = 512, kAdvKeep = 16;
+// two passes by a cluster of CL CTAs each.  The order of the sums is that of one
+// block of VT threads: thread t of it adds the positions t, t + VT, ... in
+// order, a fixed shuffle tree its warps, and the warps follow in order.  CTA r
+// takes the threads [r W, (r + 1) W), W = VT / CL.  A position costs its
+// permutation (a serial chain of integer operations) and a gather from L2, so
+// all of a CTA's threads fetch the values of its W into shared memory, kAdvCap at
+// a time (fetched once where that is all of them), and W threads add them up.
+// CL (a power of two up to 8, the portable limit) is the least that gives a
+// thread at most 8 values to fetch, as long as that is met.  One block per
+// minibatch that gathered for both passes took 263 us for the 32 of a 72B update,
+// 66 for the 16 of Stress and 80 for a 7B update's; this takes 46, 18 and 17.
+constexpr int kAdvNT = 512, kAdvCap = 8192;
+template <int VT>
 __global__ void __launch_bounds__(kAdvNT) ppo_advstats_kernel(const float* __restrict__ adv, int64_t N, int M, int nmb,
                                                               FeistelSet perms, float2* __restrict__ out) {
   namespace cg = cooperative_groups;
-  __shared__ float red[32];
-  __shared__ float csum[2];
+  constexpr int VW = VT / 32;
+  __shared__ float val[kAdvCap];
+  __shared__ float mine[2][VW], all[2][VW];  // per pass: this CTA's warp sums, then the cluster's
   const cg::cluster_group cl = cg::this_cluster();
-  const int CL = (int)cl.num_blocks(), r = (int)cl.block_rank();
+  const int CL = (int)cl.num_blocks(), r = (int)cl.block_rank(), W = VT / CL, tid = threadIdx.x;
   const int mb = blockIdx.x / CL, ep = blockIdx.y;
   const Feistel& f = perms.f[ep];
   const int64_t start = (int64_t)mb * M;
   const int cnt = (int)(N - start < (int64_t)M ? N - start : (int64_t)M);
-  const int j0 = r * kAdvNT + threadIdx.x, step = CL * kAdvNT;
-  auto value = [&](int64_t j) { return __ldg(adv + feistel_index(f, start + j)); };
-  auto cluster_sum = [&](float v, int k) -> float {
-    const float b = block_sum_f(v, red);
-    if (CL == 1) return b;
-    if (threadIdx.x == 0) csum[k] = b;
+  const int rows = (cnt - 1) / VT + 1, most = kAdvCap / W;  // values per thread; at a time
+  float mean = 0.0f;
+  auto pass = [&](int k, auto add) -> float {
+    float s = 0.0f;
+    for (int i0 = 0; i0 < rows; i0 += most) {
+      const int ni = min(most, rows - i0);
+      if (k == 0 || rows > most) {
+        __syncthreads();
+#pragma unroll 8
+        for (int x = tid; x < ni * W; x += kAdvNT) {
+          const int64_t j = (int64_t)(i0 + x / W) * VT + r * W + x % W;
+          val[x] = j < cnt ? __ldg(adv + feistel_index(f, start + j)) : 0.0f;
+        }
+        __syncthreads();
+      }
+      if (tid < W) {
+        const int n = min(ni, (int)(((int64_t)cnt - (r * W + tid) + VT - 1) / VT) - i0);
+#pragma unroll 8
+        for (int i = 0; i < n; ++i) s = add(s, val[i * W + tid]);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (tid < W && (tid & 31) == 0) mine[k][tid >> 5] = s;
     cl.sync();
+    if (tid < VW) all[k][tid] = *cl.map_shared_rank(&mine[k][tid % (W / 32)], tid / (W / 32));
+    __syncthreads();
     float t = 0.0f;
-    for (int q = 0; q < CL; ++q) t += *cl.map_shared_rank(&csum[k], q);
+#pragma unroll
+    for (int i = 0; i < VW; ++i) t += all[k][i];
     return t;
   };
-  float keep[kAdvKeep], s = 0.0f;
-#pragma unroll
-  for (int i = 0; i < kAdvKeep; ++i) keep[i] = j0 + (int64_t)i * step < cnt ? value(j0 + (int64_t)i * step) : 0.0f;
-#pragma unroll
-  for (int i = 0; i < kAdvKeep; ++i) s += keep[i];
-  for (int64_t j = j0 + (int64_t)kAdvKeep * step; j < cnt; j += step) s += value(j);
-  const float mean = cluster_sum(s, 0) / (float)cnt;
-  float q = 0.0f;
-#pragma unroll
-  for (int i = 0; i < kAdvKeep; ++i) {
-    const float a = keep[i] - mean;
-    if (j0 + (int64_t)i * step < cnt) q = fmaf(a, a, q);
-  }
-  for (int64_t j = j0 + (int64_t)kAdvKeep * step; j < cnt; j += step) {
-    const float a = value(j) - mean;
-    q = fmaf(a, a, q);
-  }
-  const float ss = cluster_sum(q, 1);
-  if (r == 0 && threadIdx.x == 0) {
+  mean = pass(0, [](float s, float v) { return s + v; }) / (float)cnt;
+  const float ss = pass(1, [&](float s, float v) {
+    const float a = v - mean;
+    return fmaf(a, a, s);
+  });
+  if (r == 0 && tid == 0) {
     if (cnt > 1) {
       const float sd = sqrtf(ss / (float)(cnt - 1));
       out[ep * nmb + mb] = make_float2(mean, 1.0f / (sd + 1e-8f));
@@ -120,7 +132,7 @@ __global__ void __launch_bounds__(kAdvNT) ppo_advstats_kernel(const float* __res
       out[ep * nmb + mb] = make_float2(0.0f, 1.0f);  // a 1-sample minibatch is not normalised
     }
   }
-  if (CL > 1) cl.sync();  // the other CTAs have read this one's sum
+  cl.sync();  // the other CTAs have read this one's sums
 }
 
 // Dense-layer register tiles for the sample slices: a thread owns RT
@@ -1085,14 +1097,15 @@ static PpoPlan ppo_plan(const pe_net& net, const pe_ppo_config& cfg, int64_t N) 
   return p;
 }
 
-// advantage statistics of every (epoch, minibatch), shared with the bf16 update
-pe_status launch_advstats(const float* adv, int64_t N, int M, int nmb, int epochs, uint64_t seed,
-                          uint32_t iteration, float2* out, cudaStream_t st) {
+// advantage statistics of every (epoch, minibatch), in the order of a block of VT threads
+template <int VT>
+static pe_status advstats_run(const float* adv, int64_t N, int M, int nmb, int epochs, uint64_t seed,
+                              uint32_t iteration, float2* out, cudaStream_t st) {
   if (epochs < 1 || epochs > kPpoMaxEpochs) return fail(PE_EINVAL, "epochs must be in [1, %d]", kPpoMaxEpochs);
   FeistelSet perms{};
   for (int ep = 0; ep < epochs; ++ep) perms.f[ep] = make_feistel((uint64_t)N, seed, ep, iteration);
   const int64_t cnt = std::min<int64_t>(M, N);
-  unsigned cl = 1;
+  unsigned cl = VT > kAdvNT ? VT / kAdvNT : 1;
   while (cl < 8 && (int64_t)cl * kAdvNT * 8 < cnt) cl *= 2;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeClusterDimension;
@@ -1106,10 +1119,16 @@ pe_status launch_advstats(const float* adv, int64_t N, int M, int nmb, int epoch
   lc.numAttrs = 1;
   {
     ProfScope ps(PE_PROF_PPO_OTHER, st);
-    PE_TRY_CUDA(cudaLaunchKernelEx(&lc, ppo_advstats_kernel, adv, N, M, nmb, perms, out));
+    PE_TRY_CUDA(cudaLaunchKernelEx(&lc, ppo_advstats_kernel<VT>, adv, N, M, nmb, perms, out));
   }
   PE_CHECK_LAUNCH("ppo_advstats_kernel");
   return PE_OK;
+}
+
+// for the bf16 update
+pe_status launch_advstats(const float* adv, int64_t N, int M, int nmb, int epochs, uint64_t seed,
+                          uint32_t iteration, float2* out, cudaStream_t st) {
+  return advstats_run<1024>(adv, N, M, nmb, epochs, seed, iteration, out, st);
 }
 
 int64_t ppo_ws_bytes_f32(const pe_net& net, const pe_ppo_config& cfg, int64_t N) {
@@ -1134,7 +1153,7 @@ static pe_status ppo_run(const pe_net& net, float* params, float* m, float* v, i
   PE_TRY_CUDA(cudaMemsetAsync(acc, 0, 8 * sizeof(double) + 16, st));
   FeistelSet perms{};
   for (int ep = 0; ep < cfg.epochs; ++ep) perms.f[ep] = make_feistel((uint64_t)N, cfg.seed, ep, cfg.iteration);
-  if (const pe_status e = launch_advstats(adv, N, cfg.minibatch, pl.nmb, cfg.epochs, cfg.seed, cfg.iteration, advstat, st);
+  if (const pe_status e = advstats_run<256>(adv, N, cfg.minibatch, pl.nmb, cfg.epochs, cfg.seed, cfg.iteration, advstat, st);
       e != PE_OK)
     return e;
   {

@@ -6,6 +6,8 @@ that near-zero entries do not fail a pure relative test; sampled actions
 agree on >= 99.9% of steps under teacher forcing (the oracle steps with the
 GPU's actions, so one flipped sample cannot cascade).
 """
+import hashlib
+
 import numpy as np
 import pytest
 import torch
@@ -928,10 +930,10 @@ def test_ppo_7b_single_step_partitions(n):
 
 @pytest.mark.parametrize("n", [4096, 4097, 16400, 70000])
 def test_ppo_advantage_statistics_clusters(n):
-    """The statistics of one minibatch are summed by a cluster of CTAs of 512
-    threads with 16 register values each: one CTA up to 4,096 samples, two
-    above, eight above 16,384, and beyond 65,536 each thread gathers the rest
-    again.  A wrong mean or deviation scales the whole first moment."""
+    """The statistics of one minibatch are summed by a cluster of CTAs that fetch
+    up to 8,192 values each: one CTA up to 4,096 samples, two above, eight above
+    16,384, and beyond 65,536 in two rounds per pass, the second partly empty.
+    A wrong mean or deviation scales the whole first moment."""
     wl = W.make_7b(n_envs=1152)
     params, buf, adv, ret = _ppo_inputs(wl, 64, seed=6)
     D = wl.net.obs_dim
@@ -987,10 +989,9 @@ def test_ppo_bf16_several_tiles_per_cta(preset, E, T):
 
 @pytest.mark.parametrize("preset,n", [("72b", 20), ("72b", 60), ("72b", 200), ("stress", 60), ("stress", 330)])
 def test_ppo_bf16_few_chunks(preset, n):
-    """Minibatches of 1 to 11 chunks of 32 samples: the reduction of the 72B
-    weight gradients deals its chunks out to four threads (the last ones have
-    none below four chunks), Stress sums all in one, and the second network
-    column has fewer chunks than the first."""
+    """Minibatches of 1 to 6 shares of 64 samples in the weight gradients' split:
+    the reduction sums as many partial blocks, fewer than it has loads in
+    flight, and the second network column of Stress has fewer than the first."""
     wl = W.make_72b(n_envs=16) if preset == "72b" else W.make_stress(n_envs=16, horizon=32)
     params, buf, adv, ret = _ppo_inputs(wl, 32, seed=2)
     D = wl.net.obs_dim
@@ -1031,6 +1032,40 @@ def test_ppo_bf16_ragged_epochs(preset, E, mb, clip):
     assert st[3] > 0.0
     if clip < 0.1:
         assert st[4] > 0.05
+
+
+BF16_UPDATE_SHA1 = {"72b": "9de9ceaad4b2d68e9a9084e73b71eb4e3ea1ef8b",
+                    "stress": "8d8b7d3878f684f7ce7f683f2f5e7ecacfbd9e71"}
+
+
+@pytest.mark.parametrize("preset", ["72b", "stress"])
+def test_ppo_bf16_update_keeps_its_bits(preset):
+    """Two epochs of two ragged minibatches against the digest of the same update
+    by the kernels of the first release.  Adam's first steps are +-lr whatever
+    the gradient's size, so any change of a rounding or of the order of a sum
+    (a tanh, a chunk sum, the norm, the advantage statistics) moves parameters
+    by up to 1e-3 and shows here, where tolerances cannot tell it from an error.
+    The split of the weight gradients follows the SM count."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the digests are for 152 SMs")
+    net = (W.make_72b(n_envs=4) if preset == "72b" else W.make_stress(n_envs=4, horizon=32)).net
+    rng = np.random.default_rng(3)
+    N, D = 8192, net.obs_dim
+
+    def uniform(lo, hi, *shape):  # multiples of 2^-16: no libm in the inputs
+        return torch.from_numpy((rng.integers(0, 1 << 16, shape) * ((hi - lo) / 65536) + lo).astype(np.float32)).cuda()
+
+    p = uniform(-0.125, 0.125, W.param_count(D, net.hidden, net.n_actions))
+    m, v, stats = torch.zeros_like(p), torch.zeros_like(p), torch.zeros(8, device="cuda")
+    obs = uniform(-1, 1, N, D).bfloat16()
+    act = torch.from_numpy(rng.integers(0, net.n_actions, N).astype(np.uint8)).cuda()
+    logp, adv, ret = uniform(-3, -2.5, N), uniform(-2, 2, N), uniform(-1, 1, N)
+    ppo = W.PPOSpec(epochs=2, minibatch=5000, ent_coef=0.01)
+    ws = torch.empty(pe.ppo_workspace_bytes(net, ppo, N), dtype=torch.uint8, device="cuda")
+    pe.ppo_update(net, ppo, p, m, v, 0, obs, act, logp, adv, ret, stats, ws, seed=7, iteration=1)
+    torch.cuda.synchronize()
+    got = hashlib.sha1(b"".join(cpu(t).tobytes() for t in (p, m, v, stats))).hexdigest()
+    assert got == BF16_UPDATE_SHA1[preset], got
 
 
 @pytest.mark.parametrize("preset,E", [("72b", 64), ("stress", 32)])
