@@ -1067,8 +1067,9 @@ def per_config_table(out):
 
 
 def gae_kernel_name(E: int) -> str:
-    """The GAE kernel the library picks for a batch of E envs (its dispatch
-    by width): streamed per env column for wide batches, chunked below."""
+    """The GAE kernel the library picks for a batch of E envs in aligned buffers
+    (its dispatch by width): streamed per env column for wide batches, chunked
+    below."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     if E > 920 * sms:
         return "gae_stream_kernel<32, 128>"
@@ -1076,18 +1077,19 @@ def gae_kernel_name(E: int) -> str:
         return "gae_stream_kernel<16, 64>"
     if E > 250 * sms and E % 4 == 0:
         return "gae_stream_kernel<32, 64>"
-    if E >= 32768:
+    if E > 230 * sms:
         return "gae_stream_kernel<32, 128>"
-    if E > 128 * sms:
+    if E > 128 * sms or (E > 64 * sms and E % 2 == 1):
         return "gae_stream_kernel<64, 64>"
     return "gae_kernel_v (chunked)"
 
 
 def gae_traffic(env_steps: int, E: int):
     """DRAM bytes of one GAE launch larger than L2, scaled from the committed
-    capture's bytes per env-step of the same kernel."""
-    key = "traffic_bytes_per_env_step_v4" if E >= 196608 else "traffic_bytes_per_env_step_v1"
-    b = load_traffic_per_unit("gae_stream_kernel", key) if E >= 32768 else None
+    capture's bytes per env-step of the same kernel (None for those without one)."""
+    key = {"gae_stream_kernel<16, 64>": "traffic_bytes_per_env_step_16_64",
+           "gae_stream_kernel<32, 128>": "traffic_bytes_per_env_step_32_128"}.get(gae_kernel_name(E))
+    b = load_traffic_per_unit("gae_stream_kernel", key) if key else None
     return None if b is None else b * env_steps
 
 

@@ -2,7 +2,7 @@
 // buffer (Sec. 4.2: gamma 0.99, lambda 0.95):
 //   delta_t = r_t + gamma (1 - d_t) V_{t+1} - V_t,  A_t = delta_t + gamma lambda (1 - d_t) A_{t+1}.
 //
-// HBM-bound: 9 bytes in and 8 bytes out per env-step.  A thread owns V
+// HBM-bound: 9 bytes in and 8 bytes out per env-step.  A thread owns V = 1 or 2
 // consecutive envs (vector loads/stores; a warp covers 32*V envs of one row)
 // and one time chunk of CL steps held in registers; the NW warps of a CTA
 // cover NW consecutive chunks.  Each thread first reduces its chunk to the
@@ -23,8 +23,8 @@ __global__ void __launch_bounds__(32 * NW)
     gae_kernel_v(const float* __restrict__ r, const float* __restrict__ v,
                  const uint8_t* __restrict__ d, const float* __restrict__ last_v, int T, int E,
                  float gamma, float lam, float* __restrict__ adv, float* __restrict__ ret) {
-  using FV = typename std::conditional<V == 4, float4, typename std::conditional<V == 2, float2, float>::type>::type;
-  using BV = typename std::conditional<V == 4, uchar4, typename std::conditional<V == 2, uchar2, unsigned char>::type>::type;
+  using FV = typename std::conditional<V == 2, float2, float>::type;
+  using BV = typename std::conditional<V == 2, uchar2, unsigned char>::type;
   __shared__ float sa[NW][32 * V], sb[NW][32 * V], cin[NW + 1][32 * V];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int e0 = (blockIdx.x * 32 + lane) * V;   // first env of this thread
@@ -134,10 +134,10 @@ __global__ void __launch_bounds__(32 * NW)
 // the next P steps are kept in flight in a register ring, so each SM holds
 // enough outstanding bytes to cover HBM latency; every warp streams
 // 32 consecutive envs of a row (coalesced).  Measured: 2,048 steps of 262,144
-// envs with 32 steps in flight 1.59 ms, 85% of the HBM copy peak (16 steps
-// 1.62, two envs per thread 1.63, four 1.72); 1,024 x 65,536 with 16 steps and
-// blocks of 64, which spread evenly over the SMs, 197 us, 85% (blocks of 128:
-// 207 us).
+// envs with 32 steps in flight 1.66 ms, 81% of the HBM copy peak (16 steps take
+// 2% longer, two envs per thread 3%, four 8%); 1,024 x 65,536 with 16 steps and
+// blocks of 64, which spread evenly over the SMs, 0.21 ms, 80% (blocks of 128
+// take 5% longer).
 template <int P, int NT>
 __global__ void __launch_bounds__(NT)
     gae_stream_kernel(const float* __restrict__ r, const float* __restrict__ v, const uint8_t* __restrict__ d,
@@ -201,11 +201,6 @@ static pe_status gae_run(const float* r, const float* v, const uint8_t* d, const
 pe_status gae_launch(const float* r, const float* v, const uint8_t* d, const float* last_v,
                      int T, int E, float gamma, float lam, float* adv, float* ret,
                      cudaStream_t st) {
-  const int64_t n = (int64_t)T * E;
-  const bool al4 = (E % 4 == 0) && ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(v) |
-                                      reinterpret_cast<uintptr_t>(adv) | reinterpret_cast<uintptr_t>(ret) |
-                                      reinterpret_cast<uintptr_t>(last_v)) % 16 == 0) &&
-                   reinterpret_cast<uintptr_t>(d) % 4 == 0;
   const bool al2 = (E % 2 == 0) && ((reinterpret_cast<uintptr_t>(r) | reinterpret_cast<uintptr_t>(v) |
                                       reinterpret_cast<uintptr_t>(adv) | reinterpret_cast<uintptr_t>(ret) |
                                       reinterpret_cast<uintptr_t>(last_v)) % 8 == 0) &&
@@ -217,21 +212,23 @@ pe_status gae_launch(const float* r, const float* v, const uint8_t* d, const flo
   // 512 envs per SM, with 16 steps 1,024; a partly filled second wave costs more
   // than the shallower ring.  Measured on 152 SMs, with 54M env-steps: 56,000
   // envs 169 us (16 steps: 183), 85,000 envs 180 (32 steps: 199), 150,000 envs
-  // 175 (181), 262,144 envs 171.
+  // 175 (181), 262,144 envs 171; 64 steps in flight below 230 envs per SM: 32,768
+  // envs 186 us (32 steps: 193), 34,000 envs 191 (193), 36,000 envs 194 (191).
   // Blocks of 64 spread more evenly over the SMs (42,000 envs: 193 against 201
   // us); where a row does not start on a 16-byte boundary, neighbouring blocks
   // share more lines (49,151 envs: 201 against 195).
   if (E > 920 * sms) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (E > 400 * sms) return gae_stream_run<16, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (E > 250 * sms && E % 4 == 0) return gae_stream_run<32, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (E >= 32768) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
+  if (E > 230 * sms) return gae_stream_run<32, 128>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   // The chunked kernels while their CTAs fit the SMs at once (one of 1,024
   // threads per 32 envs, two of 512 per 32 or 64 envs); beyond that the
   // streaming kernel with 64 steps in flight.  2,048 steps of 10,000 envs: 140
-  // us (179 with CTAs of 32 envs), of 20,000 envs 181 (281 with CTAs of 64).
+  // us (179 with CTAs of 32 envs), of 20,000 envs 181 (281 with CTAs of 64).  Long
+  // horizons change nothing: of 2^28 env-steps 4,096 envs take 1.75 ms, 16,384
+  // envs 1.24 (CTAs of 128 envs with 16-byte loads: 8.0 and 2.2).
   if (E > 128 * sms || (E > 64 * sms && !al2))
     return gae_stream_run<64, 64>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
-  if (n >= ((int64_t)1 << 28) && al4) return gae_run<4, 8, 4>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (E > 64 * sms) return gae_run<4, 16, 2>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   if (E > 32 * sms) return gae_run<8, 16, 1>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);
   return gae_run<8, 32, 1>(r, v, d, last_v, T, E, gamma, lam, adv, ret, st);

@@ -75,7 +75,8 @@ def test_gae_parity(T, E):
 
 @pytest.mark.parametrize("T", [1, 70, 130])
 @pytest.mark.parametrize("per_sm,extra", [(32, 0), (32, 1), (64, 0), (64, 1), (64, 2), (128, 0), (128, 1), (128, 2),
-                                          (250, 0), (250, 4), (400, 0), (400, 1), (920, 0), (920, 1)])
+                                          (230, 0), (230, 1), (250, 0), (250, 4), (400, 0), (400, 1), (920, 0),
+                                          (920, 1)])
 def test_gae_parity_batch_widths(per_sm, extra, T):
     """Both sides of the widths at which another kernel takes over (envs per
     SM: one chunked CTA, two, two of 64 envs, then the streaming kernels, of
@@ -102,12 +103,12 @@ def test_gae_parity_batch_widths(per_sm, extra, T):
 @pytest.mark.parametrize("T,E", [(64, 16384), (2048, 131072), (1024, 65536), (37, 32771), (300, 131074),
                                  (5, 262144)])
 def test_gae_parity_vector_paths(T, E):
-    """The wide-batch kernels: the 2-env-per-thread chunked kernel
-    (16,384 <= E < 32,768) and the per-column streaming kernel (E >= 32,768;
-    2 envs per thread from 131,072 when aligned, else 1), with ragged CTA
-    spans (32,771 and 131,074 envs), horizons shorter than, equal to and not a
-    multiple of its 16- or 12-step load ring.  Envs are independent, so the
-    oracle checks sampled columns including both ends of a CTA span."""
+    """Wide batches at fixed widths (on 152 SMs: 16,384 envs in the chunked kernel
+    with two envs per thread, the others in the streaming kernels with one),
+    with ragged CTA spans (32,771 and 131,074 envs), horizons shorter than, equal
+    to and not a multiple of their load rings of 16 to 64 steps.  Envs are
+    independent, so the oracle checks sampled columns including both ends of a
+    CTA span."""
     g = torch.Generator(device="cuda").manual_seed(E)
     r = torch.randn(T, E, device="cuda", generator=g)
     v = torch.randn(T, E, device="cuda", generator=g)

@@ -33,8 +33,8 @@ def test_profile_names_its_command(name):
     ("ppo_persistent_kernel", "traffic_bytes_per_launch"),
     ("fleet_windows_kernel", "traffic_bytes_per_launch"),
     ("mlp_bf16_pair_kernel", "traffic_bytes_per_launch"),
-    ("gae_stream_kernel", "traffic_bytes_per_env_step_v1"),
-    ("gae_stream_kernel", "traffic_bytes_per_env_step_v4"),
+    ("gae_stream_kernel", "traffic_bytes_per_env_step_16_64"),
+    ("gae_stream_kernel", "traffic_bytes_per_env_step_32_128"),
 ])
 def test_bench_traffic_figures(kernel, key):
     """bench.py reads these keys (bench.load_traffic / load_traffic_per_unit)."""
