@@ -347,9 +347,10 @@ pe_status pe_ppo_update(const pe_net* net, float* params, float* adam_m, float* 
  *  workspace: pe_fleet_workspace_bytes(J, L, H) bytes.  For J <= 8 that size
  *  holds eight shifted copies of the jobs' samples in 16 bits (where their
  *  ranges allow it) or four of their prefix sums, so that the counts use
- *  16-byte loads; a smaller workspace, down to the one copy of
- *  J * (L + H + 128) words plus 1 KiB, gives the same results through 4-byte
- *  loads.
+ *  16-byte loads; a smaller workspace gives the same results through 4-byte
+ *  loads, down to one copy: J rows of L + H + 128 words (rounded up to a
+ *  multiple of 4) and J * ceil((L + H) / 8192) words, each of the two rounded
+ *  up to a multiple of 256 bytes, and 512 bytes.
  * The call validates the traces on the device and waits for that check
  * (one small device-to-host read on `stream`) before launching the counts.
  * Errors: PE_EINVAL (sizes, pointers, job map or offsets out of range),

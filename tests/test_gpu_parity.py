@@ -205,6 +205,23 @@ def test_fleet_parity_window_alignments(windows):
         assert np.array_equal(c, oc) and np.array_equal(p, op)
 
 
+@pytest.mark.parametrize("L,H", [(2999, 1502), (380_000, 380_000)])
+def test_fleet_least_workspace(L, H):
+    """The least workspace the header states is taken, gives the counts of the
+    full one, and a byte less is refused."""
+    fw = W.make_fleet(n_compositions=3, length=L, windows=(1, 60, 600))
+    fw.horizon = H
+    J, up = fw.n_jobs, lambda n, k: (n + k - 1) // k * k  # noqa: E731
+    least = up(4 * J * up(L + H + 128, 4), 256) + up(4 * J * -(-(L + H) // 8192), 256) + 512
+    full = pe.fleet_workspace_bytes(J, L, H)
+    want = _fleet_gpu(fw, [1, 60, 600])
+    got = _fleet_gpu(fw, [1, 60, 600], ws_short=full - least)
+    assert all(np.array_equal(g, w) for g, w in zip(got, want))
+    with pytest.raises(pe.PEError) as e:
+        _fleet_gpu(fw, [1, 60, 600], ws_short=full - least + 1)
+    assert e.value.status == pe.PE_EINVAL
+
+
 def test_fleet_parity_more_than_eight_jobs():
     """Twelve jobs over the sixteen traces: the path for fleets of more than
     eight jobs (one prefix copy, stream bases in shared memory)."""
