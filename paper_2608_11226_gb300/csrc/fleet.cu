@@ -1047,9 +1047,12 @@ pe_status fleet_stagger_launch(const float* traces, int G, int L, const int32_t*
   const int64_t xmax = (int64_t)L + H - w;                     // last window of an unrolled job
   const int64_t per = (M + stride - 1) / stride, residues = std::min<int64_t>(stride, M);
   const int64_t tiles = (nc + kStTile - 1) / kStTile;
-  // items short enough to give every SM several blocks (64 samples at least:
-  // an item stages 1,024 of B whatever its length)
-  const int64_t want = (per * residues * tiles + 1215) / 1216;
+  // items short enough to give every SM eight blocks (64 samples at least: an
+  // item stages 1,024 of B whatever its length)
+  int dev = 0, sms = 0;
+  PE_TRY_CUDA(cudaGetDevice(&dev));
+  PE_TRY_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int64_t want = (per * residues * tiles + 8 * sms - 1) / (8 * sms);
   const int chunk = (int)std::min<int64_t>(kStChunk, (std::max<int64_t>(std::min(want, per), 64) + 15) / 16 * 16);
   const int64_t nchunk = (per + chunk - 1) / chunk, items = nchunk * residues;
   const dim3 grid((unsigned)tiles, (unsigned)std::max<int64_t>(1, std::min<int64_t>(items, 4096)));
