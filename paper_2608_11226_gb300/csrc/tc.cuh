@@ -335,9 +335,9 @@ __device__ __forceinline__ bool near_midpoint(uint32_t least) {
 // accumulators from taddr, columns from c0 on) in the K-major buffer `act` those
 // of tanhf; least[j]: tanh_bf16's of the thread's chunk j.  8% of a warp's chunks
 // need it, and all warps of a tile wait for the last one, so the latency of a
-// pass and the code it fetches count: two rows of a chunk at a time, a lane per
+// pass and the code it fetches count: one row of a chunk at a time, a lane per
 // column, in one loop for all chunks.  A 72B rollout of 65,536 envs x 64 steps
-// takes 3.79 ms, a Stress rollout of 262,144 x 8 4.23 ms; with tanhf for every
+// takes 3.75 ms, a Stress rollout of 262,144 x 8 4.18 ms; with tanhf for every
 // value, about 18 issue slots and both sides of its branch, 4.20 and 4.63; with
 // the rational alone, whose results are not tanhf's, 3.36 and 3.76.  (Settling
 // each chunk before the next, 4.05 and 4.51.)
@@ -352,11 +352,10 @@ __device__ __forceinline__ void tanh_exact(const uint32_t (&least)[NJ], uint32_t
   uint32_t near = 0;  // the thread's chunks to settle
 #pragma unroll
   for (int j = 0; j < NJ; ++j) near |= near_midpoint(least[j]) ? 1u << j : 0u;
-  while (const uint32_t any = __ballot_sync(0xffffffffu, near != 0)) {
-    const int j = __ffs(__shfl_sync(0xffffffffu, near, __ffs(any) - 1)) - 1;
-    const uint32_t rows = __ballot_sync(0xffffffffu, (near >> j) & 1u), rest = rows & (rows - 1);
-    const int ra = __ffs(rows) - 1, rb = rest ? __ffs(rest) - 1 : ra;
-    const int r = lane < 16 ? ra : rb, c = c0 + 16 * j + (lane & 15);
+  for (;;) {
+    const uint32_t key = __reduce_min_sync(0xffffffffu, near ? (uint32_t)(__ffs(near) << 5 | lane) : 0xFFFFFFFFu);
+    if (key == 0xFFFFFFFFu) break;
+    const int j = (int)(key >> 5) - 1, r = (int)(key & 31u), c = c0 + 16 * j + (lane & 15);
     float v[16], z = 0.0f;
     tmem_ld16(taddr + (uint32_t)(16 * j), v);
 #pragma unroll
@@ -367,7 +366,7 @@ __device__ __forceinline__ void tanh_exact(const uint32_t (&least)[NJ], uint32_t
     const __nv_bfloat16 h = __float2bfloat16_rn(tanhf(z + bias[c]));
     __syncwarp();  // after the rows' own stores
     *reinterpret_cast<__nv_bfloat16*>(act + swz_offset<128>(row0 + r, c, R)) = h;
-    if (lane == ra || lane == rb) near &= ~(1u << j);
+    if (lane == r) near &= near - 1;
   }
 }
 

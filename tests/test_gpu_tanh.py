@@ -1,15 +1,19 @@
-"""The hidden layers' bf16 tanh (csrc/tc.cuh, tanh_bf16) against CUDA's tanhf
-rounded to bf16: the same bits for every one of the 2^32 fp32 arguments, with
-and without a bias.  The kernel is compiled here with nvcc from the library's
-own header."""
+"""The hidden layers' bf16 tanh (csrc/tc.cuh) against CUDA's tanhf rounded to
+bf16.  tanh_bf16, compiled here with nvcc from the library's own header: for
+every one of the 2^32 fp32 arguments the same bits, or reported.  The networks,
+through pe_value: arguments around the rounding midpoints, in every row and
+column of both layers."""
 import ctypes as C
 import os
 import subprocess
 
+import numpy as np
 import pytest
 import torch
 
 from paper_2608_11226_gb300 import build as libbuild
+from paper_2608_11226_gb300 import pe
+from paper_2608_11226_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -65,3 +69,38 @@ def test_bf16_tanh_is_tanhf_for_every_argument(so, bias_step):
     assert so.sweep(bias_step, differ.data_ptr()) == 0
     torch.cuda.synchronize()
     assert int(differ[0]) == 0 and int(differ[1]) < 1 << 12, differ
+
+
+@pytest.mark.parametrize("D,H", [(32, 256), (64, 512)])
+@pytest.mark.parametrize("layer", [1, 2])
+def test_bf16_network_tanh_near_midpoints(D, H, layer):
+    """Zero observations, so that a layer's pre-activations are its biases: the
+    floats within four steps of where tanh crosses a midpoint between two bf16
+    values, both signs.  Every row of a tile then has values for tanhf in every
+    chunk.  The head picks one unit per call; behind layer 1 the second layer is
+    the identity."""
+    rng = np.random.default_rng(layer)
+    t = rng.uniform(0.02, 0.995, H).astype(np.float32)
+    mid = ((t.view(np.uint32) & 0xFFFF0000) | 0x8000).view(np.float32)
+    z = np.arctanh(mid.astype(np.float64)).astype(np.float32)
+    z = (z.view(np.int32) + rng.integers(-4, 5, H)).astype(np.int32).view(np.float32) * rng.choice([-1, 1], H)
+    z = torch.from_numpy(z.astype(np.float32)).cuda()
+    want = torch.tanh(z).bfloat16().float()
+    p = torch.zeros(W.param_count(D, H, 16), device="cuda")
+    v1 = H * D + H + H * H + H + 16 * H + 16  # the value network follows the policy
+    c1, v2 = v1 + H * D, v1 + H * D + H
+    c2, v3 = v2 + H * H, v2 + H * H + H
+    if layer == 1:
+        p[c1:c1 + H] = z
+        p[v2:v2 + H * H] = torch.eye(H, device="cuda").flatten()
+        want = torch.tanh(want).bfloat16().float()
+    else:
+        p[c2:c2 + H] = z
+    obs = torch.zeros(300, D, dtype=torch.bfloat16, device="cuda")
+    out = torch.empty(300, device="cuda")
+    for i in range(0, H, 5):
+        p[v3:v3 + H] = 0
+        p[v3 + i] = 1
+        pe.value(W.NetSpec(D, H, 16, pe.PE_BF16), p, obs, out)
+        assert torch.equal(out, want[i].expand(300)), (i, float(z[i]), float(want[i]), out)
+    pe.device_check()
