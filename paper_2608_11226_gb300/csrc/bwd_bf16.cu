@@ -32,8 +32,8 @@
 //   place, and each half of the next tile's h2 (and of its dh2 accumulators)
 //   follows as soon as that half of da1 has left (and of TMEM been read).  A
 //   dedicated warp issues the MMAs, another stores the da2 and da1 images:
-//   a half of the buffer is the image's bytes, so one bulk copy of 64 KB
-//   stores it.  (Stored by the epilogue threads, 16 bytes of a 128-byte row
+//   a half of the buffer is the image's bytes, so four bulk copies of 16 KB
+//   store it.  (Stored by the epilogue threads, 16 bytes of a 128-byte row
 //   each, every warp-wide store touched 32 lines.  With the forward's images
 //   stored the same way, a Stress update of 16 steps went from 7.85 to 7.38
 //   ms.)  One launch covers both networks: the policy's tiles,
@@ -438,8 +438,8 @@ constexpr int kWgThreads = 128;
 // second column chunk's stages hold da2 and h1 alone.  The kernel is bound by
 // the bytes it keeps in flight, so the stages are small and fill the shared
 // memory: 4 of 45 KB, or 8 of 24 KB.  With two slots of 90 KB for either, of
-// which column chunk 1 used 48, a Stress update took 6.55 ms and a 72B update
-// 5.73 ms; now 6.35 and 5.67.  (5 and 9 slots: 6.37 and 5.79 ms, the next
+// which column chunk 1 used 48, a Stress update took 3% longer (6.55 against
+// 6.35 ms) and a 72B update 1% (5.73, 5.67).  (5 and 9 slots: 6.37 and 5.79 ms, the next
 // kernel's blocks then find no shared memory beside this one's.)
 constexpr int kWgA = 2 * kWgSamples * 128;  // 8 KB
 constexpr int kWgDa2 = 0, kWgDa1 = kWgA, kWgH2 = 2 * kWgA, kWgH1 = 3 * kWgA;

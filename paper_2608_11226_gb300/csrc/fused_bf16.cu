@@ -23,7 +23,7 @@
 //   epilogue -> storer: h1in, h2in, d2in and d1in (da1, which takes da2's
 //   place in the slot's buffer once the dh1 MMAs have read it).
 // A slot's buffer holds h1, h2, da2 and da1 in turn, each byte for byte its
-// tile image, so that one bulk copy of 64 KB stores each; "stored" completes
+// tile image, so that bulk copies of 16 KB store each; "stored" completes
 // four times per pair, when a copy has read the buffer, and the epilogue that
 // overwrites it waits for that.  (Stored by the epilogue threads, 16 bytes of
 // a 128-byte row each, every warp-wide store touched 32 lines.

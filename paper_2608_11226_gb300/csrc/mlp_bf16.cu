@@ -76,7 +76,7 @@ __global__ void weight_image_kernel(const float* __restrict__ params, int A, int
 // stage s into slot s%2 once the MMAs that read the slot's previous stage
 // have completed (tcgen05.commit on the slot's "empty" barrier), warp 17
 // issues the MMAs, warp 18 stores the h1 and h2 tile images of a PPO forward
-// (the buffer's halves are the images' bytes, so one bulk copy of 64 KB stores
+// (the buffer's halves are the images' bytes, so plain bulk copies store
 // each; "sa" and "sb" complete when a copy has read its half, and the epilogue
 // that overwrites it waits for that).  A layer's 512 accumulator columns fill TMEM, so a tile
 // cannot overlap another tile; instead the epilogues hand over per 256-column
@@ -989,7 +989,7 @@ static pe_status launch_mlp(const uint8_t* img, const float* params, int A, int 
     ProfScope ps(prof_kind, st);
     // early in an update's chain of kernels; a rollout's policy launches gain
     // nothing (their blocks would sit waiting beside the env step: a Stress
-    // rollout of 262,144 envs x 8 steps took 4.00 ms so, and takes 3.90)
+    // rollout of 262,144 envs x 8 steps took 4.00 ms so, against 3.90)
     PE_TRY_CUDA(launch_pdl(kern, grid, kStreamThreads, bytes, st, second.img != nullptr, img, params, A, value_net, o, n,
                            out, out_stride, nout, err, save, second));
   } else {
@@ -1024,9 +1024,10 @@ static pe_status make_images(const float* params, int A, uint8_t* ws, cudaStream
 // the second half of the envs, split on a 128-env tile boundary), the first
 // on the caller's stream and the second on an auxiliary stream forked from
 // it and joined back before the value pass.  Each chain alternates its own
-// policy and env-step launches, so an env step (latency-bound, few
-// registers, no shared memory) can run beside the other chain's tensor-core
-// policy kernel, whose half-size grid leaves SMs free.  Every env's
+// policy and env-step launches, so an env step (latency-bound) can start while
+// the other chain's tensor-core policy kernel runs, on the SMs which that
+// kernel's half-size grid leaves (24 of 152; beside a policy CTA there are too
+// few registers for an env block).  Every env's
 // arithmetic is the single-chain arithmetic, so the results are the same
 // bits.  Measured on GB300 (65,536 envs x 64 steps): 4.89 ms against 5.16 ms
 // for one chain.  Forcing the two chains' policy kernels to alternate (an
