@@ -25,7 +25,6 @@
 // minibatches up front.
 #include <algorithm>
 #include <cmath>
-#include <vector>
 
 #include <cstddef>
 
@@ -1097,6 +1096,17 @@ static PpoPlan ppo_plan(const pe_net& net, const pe_ppo_config& cfg, int64_t N) 
   return p;
 }
 
+// The steps' bias corrections travel as a kernel argument: a copy from a host
+// array of this call would be read again, after the array is gone, by every
+// replay of a graph that captured the call.
+struct BcChunk {
+  static constexpr int kSteps = 1024;
+  float v[2 * kSteps];
+};
+__global__ void ppo_bc_kernel(const __grid_constant__ BcChunk bc, int n, float* __restrict__ out) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) out[i] = bc.v[i];
+}
+
 // advantage statistics of every (epoch, minibatch), in the order of a block of VT threads
 template <int VT>
 static pe_status advstats_run(const float* adv, int64_t N, int M, int nmb, int epochs, uint64_t seed,
@@ -1182,14 +1192,19 @@ static pe_status ppo_run(const pe_net& net, float* params, float* m, float* v, i
   // one CTA per SM for each network: as many CTAs as the GPU holds at once
   const int nc = std::min(pl.NC, per_sm * sms / 2);
   if (coop && nc >= 1) {
-    std::vector<float> bc(2 * (size_t)pl.steps);
-    for (int k = 0; k < pl.steps; ++k) {
-      const double tt = (double)(adam_t + k + 1);
-      bc[2 * k] = (float)(cfg.lr / (1.0 - std::pow((double)cfg.beta1, tt)));
-      bc[2 * k + 1] = (float)(1.0 / std::sqrt(1.0 - std::pow((double)cfg.beta2, tt)));
-    }
     float* bc_dev = reinterpret_cast<float*>(ws + pl.off_bc);
-    PE_TRY_CUDA(cudaMemcpyAsync(bc_dev, bc.data(), bc.size() * sizeof(float), cudaMemcpyHostToDevice, st));
+    for (int k0 = 0; k0 < pl.steps; k0 += BcChunk::kSteps) {
+      BcChunk bc;
+      const int n = std::min(pl.steps - k0, BcChunk::kSteps);
+      for (int k = 0; k < n; ++k) {
+        const double tt = (double)(adam_t + k0 + k + 1);
+        bc.v[2 * k] = (float)(cfg.lr / (1.0 - std::pow((double)cfg.beta1, tt)));
+        bc.v[2 * k + 1] = (float)(1.0 / std::sqrt(1.0 - std::pow((double)cfg.beta2, tt)));
+      }
+      ProfScope ps(PE_PROF_PPO_OTHER, st);
+      ppo_bc_kernel<<<1, 256, 0, st>>>(bc, 2 * n, bc_dev + 2 * (int64_t)k0);
+    }
+    PE_CHECK_LAUNCH("ppo_bc_kernel");
     PpoLoop L;
     L.g.obs = obs;
     L.g.act = act;

@@ -966,6 +966,42 @@ def test_ppo_advantage_statistics_clusters(n):
     assert_stats(gs, st, n)
 
 
+@pytest.mark.parametrize("preset", ["tiny", "7b", "72b", "stress"])
+def test_ppo_update_graph_replay(preset):
+    """An update captured into a CUDA graph and replayed twice, host memory
+    allocated and freed in between, gives the bits of the eager call each time:
+    nothing of the call's host state is read at replay."""
+    wl = {"tiny": W.make_tiny, "7b": W.make_7b, "72b": W.make_72b}[preset](n_envs=32) if preset != "stress" \
+        else W.make_stress(n_envs=32, horizon=64)
+    params, buf, adv, ret = _ppo_inputs(wl, 64, seed=2)
+    ppo = W.PPOSpec(epochs=2, minibatch=500)
+    N = 64 * 32
+    init = torch.from_numpy(params).cuda()
+    p, m, v, stats = init.clone(), torch.zeros_like(init), torch.zeros_like(init), torch.zeros(8, device="cuda")
+    ws = torch.empty(pe.ppo_workspace_bytes(wl.net, ppo, N), dtype=torch.uint8, device="cuda")
+
+    def reset():
+        p.copy_(init), m.zero_(), v.zero_(), stats.zero_(), ws.fill_(0xA5)
+
+    def call():
+        pe.ppo_update(wl.net, ppo, p, m, v, 3, buf["obs"], buf["act"], buf["logp"], adv, ret, stats, ws, seed=7,
+                      iteration=1)
+
+    reset()
+    call()
+    want = [t.clone() for t in (p, m, v, stats)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for _ in range(2):
+        reset()
+        junk = [np.full(n, 1e30, np.float32) for n in (2, 8, 20, 64, 2048)]
+        del junk
+        graph.replay()
+        for g, w in zip((p, m, v, stats), want):
+            assert torch.equal(g, w)
+
+
 # ------------------------------------------------------------------ bf16 PPO
 BF16_TOL = 2e-2
 
