@@ -1094,8 +1094,8 @@ BF16_UPDATE_SHA1 = {"72b": "9de9ceaad4b2d68e9a9084e73b71eb4e3ea1ef8b",
 
 @pytest.mark.parametrize("preset", ["72b", "stress"])
 def test_ppo_bf16_update_keeps_its_bits(preset):
-    """Two epochs of two ragged minibatches against the digest of the same update
-    by the kernels of the first release.  Adam's first steps are +-lr whatever
+    """Two epochs of two ragged minibatches against the digest recorded for them
+    (with tanhf throughout and one block's sums).  Adam's first steps are +-lr whatever
     the gradient's size, so any change of a rounding or of the order of a sum
     (a tanh, a chunk sum, the norm, the advantage statistics) moves parameters
     by up to 1e-3 and shows here, where tolerances cannot tell it from an error.
